@@ -120,6 +120,34 @@ __device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
         : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
+// Sum of products of FP32 values to more than FP64's precision on the FP32 pipe, two sums at a
+// time: each product split exactly by an FMA (p + e), each addition exactly by Knuth's two-sum,
+// the errors of the first level summed in a second level with its own exact additions and those
+// of the second in a third, so a sum's relative error is about 2^-70. GB300's FP64 pipe would
+// spend 64 cycles of a sub-partition on every converted operand and every multiply-add; a
+// product here takes about 20 packed instructions.
+struct Sum3 {
+    float2 h{0.f, 0.f}, m{0.f, 0.f}, l{0.f, 0.f};
+    __device__ __forceinline__ static void two_sum2(float2 &s, float2 b, float2 &err) {
+        const float2 t = f2_add(s, b);
+        const float2 bb = f2_sub(t, s);
+        err = f2_add(f2_sub(s, f2_sub(t, bb)), f2_sub(b, bb));
+        s = t;
+    }
+    // += a b elementwise
+    __device__ __forceinline__ void mac(float2 a, float2 b) {
+        const float2 p = f2_mul(a, b);
+        const float2 e = f2_fma(a, b, make_float2(-p.x, -p.y));
+        float2 t, u, w;
+        two_sum2(h, p, t);
+        two_sum2(m, t, u);
+        two_sum2(m, e, w);
+        l = f2_add(l, f2_add(u, w));
+    }
+    __device__ __forceinline__ double x() const { return ((double)h.x + (double)m.x) + (double)l.x; }
+    __device__ __forceinline__ double y() const { return ((double)h.y + (double)m.y) + (double)l.y; }
+};
+
 // (H, L) += (Ah + Al)(Bh + Bl) elementwise, dropping Al*Bl; nBh = -Bh is passed in (it is
 // formed once per operand and reused) so that no separate negation is issued: -p = Ah * nBh
 // exactly, the product error is fma(Ah, Bh, -p), and H + p = H - (-p) is Knuth's two-sum.

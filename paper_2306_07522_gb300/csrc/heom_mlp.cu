@@ -11,14 +11,18 @@
 //
 // The networks are small (widths of a few hundred, batches of a few thousand): one product
 // is a few hundred MFLOP at most, microseconds on this GPU next to the milliseconds of a
-// stationary solve, so the products use the synchronous warp-level MMA with plain shared-
-// memory staging rather than an asynchronous TMA / tcgen05 pipeline.
+// stationary solve, so the products use the synchronous warp-level MMA rather than a
+// TMA / tcgen05 pipeline. What bounds them is the number of blocks and the latency of the staging
+// loads, so long reductions are split over blocks (the weight gradients) and the next tile is
+// loaded while the current one is multiplied.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
+#include "heom_ff.cuh"
 #include "heom_internal.h"
 
 struct heom_mlp {
@@ -36,32 +40,95 @@ struct heom_mlp {
 namespace heom {
 namespace {
 
-constexpr int kBM = 64, kBN = 64, kBK = 16, kPad = 8;
+constexpr int kBM = 64, kBN = 64, kBK = 32, kPad = 8;
+constexpr int kGemmThreads = 128;
 
 enum Epi { EPI_STORE = 0, EPI_BIAS = 1, EPI_TANH = 2, EPI_DTANH = 3 };
 
-__device__ __forceinline__ uint32_t ld_pair(const __nv_bfloat16 *p) {
-    return *reinterpret_cast<const uint32_t *>(p);
+// four 8 x 8 BF16 matrices from shared memory, one row address per lane
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+    if constexpr (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
 }
 
+// One operand tile of 64 (m or n) x kBK, staged from FP32 global memory through registers into
+// BF16 shared memory in its own storage order: CONTIG_K (element (i, k) at P[i ld + k]) as
+// [64][kBK + pad], else (P[k ld + i]) as [kBK][64 + pad]; ldmatrix transposes where needed. A
+// thread moves four groups of four neighbouring elements; VEC: whole groups by one 16-byte
+// load (ld a multiple of four, P 16-byte aligned). Elements outside are zero.
+template <bool CONTIG_K, bool VEC>
+struct TileLoader {
+    static constexpr int kRow = CONTIG_K ? kBK + kPad : 64 + kPad;
+    static constexpr int kPerRow = CONTIG_K ? kBK / 4 : 16;  // groups per stored row
+    float4 v[4];
+    __device__ __forceinline__ void load(const float *__restrict__ P, int ld, int i0, int n_i, int k0, int k1) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = threadIdx.x + u * kGemmThreads, row = g / kPerRow, c = (g % kPerRow) * 4;
+            const int i = i0 + (CONTIG_K ? row : c), k = k0 + (CONTIG_K ? c : row);
+            const int left = CONTIG_K ? k1 - k : n_i - i;  // elements of the group inside
+            const bool in = CONTIG_K ? i < n_i : k < k1;
+            const float *p = CONTIG_K ? P + (int64_t)i * ld + k : P + (int64_t)k * ld + i;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (in && left > 0) {
+                if (VEC && left >= 4) {
+                    x = __ldg(reinterpret_cast<const float4 *>(p));
+                } else {
+                    x.x = __ldg(p);
+                    if (left > 1) x.y = __ldg(p + 1);
+                    if (left > 2) x.z = __ldg(p + 2);
+                    if (left > 3) x.w = __ldg(p + 3);
+                }
+            }
+            v[u] = x;
+        }
+    }
+    __device__ __forceinline__ void store(__nv_bfloat16 *s) const {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int g = threadIdx.x + u * kGemmThreads;
+            const __nv_bfloat162 a = __floats2bfloat162_rn(v[u].x, v[u].y), b = __floats2bfloat162_rn(v[u].z, v[u].w);
+            uint2 w;
+            w.x = *reinterpret_cast<const uint32_t *>(&a);
+            w.y = *reinterpret_cast<const uint32_t *>(&b);
+            *reinterpret_cast<uint2 *>(s + (g / kPerRow) * kRow + (g % kPerRow) * 4) = w;
+        }
+    }
+};
+
 // C[M][N] (row-major, ldc) = op(A) op(B) with an epilogue. op(A) is M x K: element (m, k) at
-// A[m lda + k], or at A[k lda + m] when transA; op(B) is K x N: element (k, n) at B[k ldb + n],
-// or at B[n ldb + k] when transB. Operands are rounded to BF16 when staged into shared memory.
+// A[m lda + k], or at A[k lda + m] with TA; op(B) is K x N: element (k, n) at B[k ldb + n],
+// or at B[n ldb + k] with TB. Operands are rounded to BF16 when staged into shared memory.
 // Epilogues: STORE C = acc; BIAS C = acc + bias[n]; TANH C = tanh(acc + bias[n]);
 // DTANH C = acc (1 - aux[m ldc + n]^2) (back-propagation through a tanh layer whose output
-// is aux). Block: 128 threads = 2 x 2 warps, 64 x 64 tile, each warp 32 x 32 as 2 x 4 MMA
-// tiles of 16 x 8.
-template <int EPI>
-__global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const float *__restrict__ A, int lda,
-                                              int transA, const float *__restrict__ B, int ldb, int transB,
-                                              float *__restrict__ C, int ldc, const float *__restrict__ bias,
-                                              const float *__restrict__ aux) {
-    __shared__ __align__(16) __nv_bfloat16 As[kBM][kBK + kPad];
-    __shared__ __align__(16) __nv_bfloat16 Bs[kBN][kBK + kPad];  // n-major: Bs[n][k]
+// is aux). Block: 4 warps, 64 x 64 tile, each warp 32 x 32 as 2 x 4 MMA tiles of 16 x 8.
+// Block z sums k in [z kchunk, (z + 1) kchunk) into C + z M N (STORE, the weight gradients: their
+// K is the batch, thousands, and their M x N tiles are few, so without the split 52 blocks of
+// 152 SMs would walk 4,096 rows one after another). colsum (with TA): also the column sums of B
+// over the block's k range, unrounded, into colsum + z N (the bias gradients).
+// Staging: the next tile's global loads are in registers while the current tile is multiplied, two
+// shared-memory buffers, one block barrier per 32 k.
+template <int EPI, bool TA, bool TB, bool VEC>
+__global__ void __launch_bounds__(kGemmThreads) k_gemm(int M, int N, int K, const float *__restrict__ A, int lda,
+                                                       const float *__restrict__ B, int ldb, float *__restrict__ C,
+                                                       int ldc, const float *__restrict__ bias,
+                                                       const float *__restrict__ aux, int kchunk,
+                                                       float *__restrict__ colsum) {
+    using LA = TileLoader<!TA, VEC>;
+    using LB = TileLoader<TB, VEC>;
+    __shared__ __align__(16) __nv_bfloat16 As[2][TA ? kBK * LA::kRow : 64 * LA::kRow];
+    __shared__ __align__(16) __nv_bfloat16 Bs[2][TB ? 64 * LB::kRow : kBK * LB::kRow];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp >> 1, wn = warp & 1;
-    const int gq = lane >> 2, tq = lane & 3;
+    const int gq = lane >> 2, tq = lane & 3, mi = lane >> 3, mr = lane & 7;
     const int m0 = blockIdx.y * kBM, n0 = blockIdx.x * kBN;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
     float acc[2][4][4];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
@@ -69,55 +136,60 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const float *
         for (int b = 0; b < 4; ++b)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-    for (int k0 = 0; k0 < K; k0 += kBK) {
-        for (int idx = tid; idx < kBM * kBK; idx += 128) {
-            int r, c;
-            if (transA) { c = idx / kBM; r = idx - c * kBM; }  // consecutive threads: consecutive m
-            else { r = idx / kBK; c = idx - r * kBK; }         // consecutive threads: consecutive k
-            const int m = m0 + r, k = k0 + c;
-            float val = 0.f;
-            if (m < M && k < K) val = transA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k];
-            As[r][c] = __float2bfloat16_rn(val);
-        }
-        for (int idx = tid; idx < kBN * kBK; idx += 128) {
-            int n, c;
-            if (transB) { n = idx / kBK; c = idx - n * kBK; }  // consecutive k
-            else { c = idx / kBN; n = idx - c * kBN; }         // consecutive n
-            const int nn = n0 + n, k = k0 + c;
-            float val = 0.f;
-            if (nn < N && k < K) val = transB ? B[(int64_t)nn * ldb + k] : B[(int64_t)k * ldb + nn];
-            Bs[n][c] = __float2bfloat16_rn(val);
-        }
-        __syncthreads();
-        uint32_t af[2][4], bf[4][2];
+    float4 cs = make_float4(0.f, 0.f, 0.f, 0.f);  // column sums of this thread's four columns
+    const bool sums = EPI == EPI_STORE && TA && colsum && blockIdx.y == 0;
+    LA la;
+    LB lb;
+    la.load(A, lda, m0, M, kb, ke);
+    lb.load(B, ldb, n0, N, kb, ke);
+    int buf = 0;
+    for (int k0 = kb; k0 < ke; k0 += kBK, buf ^= 1) {
+        la.store(As[buf]);
+        lb.store(Bs[buf]);
+        if (sums) {
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            const int rb = wm * 32 + mt * 16;
-            af[mt][0] = ld_pair(&As[rb + gq][2 * tq]);
-            af[mt][1] = ld_pair(&As[rb + gq + 8][2 * tq]);
-            af[mt][2] = ld_pair(&As[rb + gq][2 * tq + 8]);
-            af[mt][3] = ld_pair(&As[rb + gq + 8][2 * tq + 8]);
-        }
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            const int cb = wn * 32 + nt * 8;
-            bf[nt][0] = ld_pair(&Bs[cb + gq][2 * tq]);
-            bf[nt][1] = ld_pair(&Bs[cb + gq][2 * tq + 8]);
-        }
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                float *d = acc[mt][nt];
-                asm volatile(
-                    "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, "
-                    "{%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-                    : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                    : "r"(af[mt][0]), "r"(af[mt][1]), "r"(af[mt][2]), "r"(af[mt][3]),
-                      "r"(bf[nt][0]), "r"(bf[nt][1]));
+            for (int u = 0; u < 4; ++u) {
+                cs.x += lb.v[u].x;
+                cs.y += lb.v[u].y;
+                cs.z += lb.v[u].z;
+                cs.w += lb.v[u].w;
             }
+        }
         __syncthreads();
+        if (k0 + kBK < ke) {
+            la.load(A, lda, m0, M, k0 + kBK, ke);
+            lb.load(B, ldb, n0, N, k0 + kBK, ke);
+        }
+#pragma unroll
+        for (int ks = 0; ks < kBK; ks += 16) {
+            uint32_t af[2][4], bf[2][4];
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt) {
+                const int rb = wm * 32 + mt * 16;
+                if constexpr (TA) ldmatrix4<true>(af[mt], &As[buf][(ks + (mi >> 1) * 8 + mr) * LA::kRow + rb + (mi & 1) * 8]);
+                else ldmatrix4<false>(af[mt], &As[buf][(rb + (mi & 1) * 8 + mr) * LA::kRow + ks + (mi >> 1) * 8]);
+            }
+#pragma unroll
+            for (int nt = 0; nt < 2; ++nt) {
+                const int cb = wn * 32 + nt * 16;
+                if constexpr (TB) ldmatrix4<false>(bf[nt], &Bs[buf][(cb + (mi >> 1) * 8 + mr) * LB::kRow + ks + (mi & 1) * 8]);
+                else ldmatrix4<true>(bf[nt], &Bs[buf][(ks + (mi & 1) * 8 + mr) * LB::kRow + cb + (mi >> 1) * 8]);
+            }
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 4; ++nt) {
+                    float *d = acc[mt][nt];
+                    asm volatile(
+                        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, "
+                        "{%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+                        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                        : "r"(af[mt][0]), "r"(af[mt][1]), "r"(af[mt][2]), "r"(af[mt][3]),
+                          "r"(bf[nt >> 1][(nt & 1) * 2]), "r"(bf[nt >> 1][(nt & 1) * 2 + 1]));
+                }
+        }
     }
+    float *Cz = C + (int64_t)blockIdx.z * M * N;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -134,8 +206,36 @@ __global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, const float *
                     const float a = aux[(int64_t)m * ldc + n];
                     v *= 1.f - a * a;
                 }
-                C[(int64_t)m * ldc + n] = v;
+                Cz[(int64_t)m * ldc + n] = v;
             }
+    if constexpr (EPI == EPI_STORE && TA) {
+        if (sums) {  // threads tid, tid + 16, ... hold the same four columns: a fixed-order sum
+            __syncthreads();
+            float4 *sh = reinterpret_cast<float4 *>(As[0]);
+            sh[tid] = cs;
+            __syncthreads();
+            if (tid < 64 && n0 + tid < N) {
+                float x = 0.f;
+                for (int w = 0; w < kGemmThreads / 16; ++w) x += reinterpret_cast<const float *>(sh + w * 16 + tid / 4)[tid % 4];
+                colsum[(int64_t)blockIdx.z * N + n0 + tid] = x;
+            }
+        }
+    }
+}
+
+// out[i] = sum_z part[z][i] for i < n, then the same for the nb values after each (fixed order)
+__global__ void k_sum_parts(int Z, int64_t n, const float *__restrict__ part, float *__restrict__ out, int nb,
+                            const float *__restrict__ bpart, float *__restrict__ bout) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n + nb;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const bool w = i < n;
+        const float *p = w ? part + i : bpart + (i - n);
+        const int64_t st = w ? n : nb;
+        float x = 0.f;
+        for (int z = 0; z < Z; ++z) x += p[z * st];
+        if (w) out[i] = x;
+        else bout[i - n] = x;
+    }
 }
 
 // out[m][i] = (x[m][i] - mean[i]) / sd[i]
@@ -158,20 +258,24 @@ __global__ void k_destandardise(int64_t M, int n, const float *__restrict__ y, c
     }
 }
 
-// g = 2 (y - t) / (M n); per-block partial sums of (y - t)^2 into part[block]
-__global__ void __launch_bounds__(256) k_mse_grad(int64_t total, const float *__restrict__ y,
-                                                  const float *__restrict__ t, float *__restrict__ g,
+// g = 2 (y - ts) / (M n) with ts the standardised targets (t - mean) / sd; per-block partial sums
+// of (y - ts)^2 into part[block] (exact FP32 sums, see Sum3: an FP64 multiply-add per element
+// would take longer than the rest)
+__global__ void __launch_bounds__(256) k_mse_grad(int64_t total, int n, const float *__restrict__ y,
+                                                  const float *__restrict__ t, const float *__restrict__ mean,
+                                                  const float *__restrict__ sd, float *__restrict__ g,
                                                   double *__restrict__ part) {
     __shared__ double sh[256];
-    double acc = 0.0;
+    Sum3 acc;
     const float scale = 2.f / (float)total;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float dlt = y[i] - t[i];
+        const int c = (int)(i % n);
+        const float dlt = y[i] - (t[i] - mean[c]) / sd[c];
         g[i] = scale * dlt;
-        acc += (double)dlt * dlt;
+        acc.mac(make_float2(dlt, 0.f), make_float2(dlt, 0.f));
     }
-    sh[threadIdx.x] = acc;
+    sh[threadIdx.x] = acc.x();
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
@@ -192,15 +296,6 @@ __global__ void k_loss_finish(int n, const double *__restrict__ part, double tot
         __syncthreads();
     }
     if (threadIdx.x == 0) out[0] = sh[0] / total;
-}
-
-// db[n] = sum_m g[m][n] (one thread per output column, fixed order)
-__global__ void k_colsum(int M, int N, const float *__restrict__ g, float *__restrict__ db) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float acc = 0.f;
-    for (int m = 0; m < M; ++m) acc += g[(int64_t)m * N + n];
-    db[n] = acc;
 }
 
 // Adam (Kingma & Ba), bias-corrected: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
@@ -265,11 +360,21 @@ __global__ void k_features(int64_t B, int d, int n1, const int *__restrict__ ado
 
 int nblk(int64_t n) { return (int)std::min<int64_t>(std::max<int64_t>((n + 255) / 256, 1), 152 * 8); }
 
-template <int EPI>
-cudaError_t gemm(int M, int N, int K, const float *A, int lda, int tA, const float *B, int ldb, int tB,
-                 float *C, int ldc, const float *bias, const float *aux, cudaStream_t s) {
-    dim3 grid((unsigned)((N + kBN - 1) / kBN), (unsigned)((M + kBM - 1) / kBM));
-    k_gemm<EPI><<<grid, 128, 0, s>>>(M, N, K, A, lda, tA, B, ldb, tB, C, ldc, bias, aux);
+// parts of a weight-gradient product's K (the batch): enough blocks for two per SM, at least 256
+// rows each
+int gemm_splits(int M, int N, int K) {
+    const int tiles = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
+    return std::max(1, std::min((304 + tiles - 1) / tiles, K / 256));
+}
+
+template <int EPI, bool TA, bool TB>
+cudaError_t gemm(int M, int N, int K, const float *A, int lda, const float *B, int ldb, float *C, int ldc,
+                 const float *bias, const float *aux, cudaStream_t s, int splits = 1, float *colsum = nullptr) {
+    const int kchunk = ((K + splits - 1) / splits + kBK - 1) / kBK * kBK;
+    const dim3 grid((unsigned)((N + kBN - 1) / kBN), (unsigned)((M + kBM - 1) / kBM), (unsigned)splits);
+    const bool vec = lda % 4 == 0 && ldb % 4 == 0 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0;
+    if (vec) k_gemm<EPI, TA, TB, true><<<grid, kGemmThreads, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, aux, kchunk, colsum);
+    else k_gemm<EPI, TA, TB, false><<<grid, kGemmThreads, 0, s>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, aux, kchunk, colsum);
     return cudaGetLastError();
 }
 
@@ -283,7 +388,8 @@ uint64_t splitmix64(uint64_t &x) {
 
 struct Work {
     std::vector<float *> act;  // act[0] standardised input, act[l] layer outputs, act[L] = y
-    float *tn, *g0, *g1;       // standardised targets, two gradient buffers
+    float *g0, *g1;            // two gradient buffers
+    float *gpart, *bpart;      // weight- and bias-gradient parts of the split products
     double *part, *loss;
     int nblocks;
 };
@@ -296,16 +402,24 @@ heom_status work_for(heom_mlp *net, int64_t M, Work &w) {
     size_t off = 0;
     std::vector<size_t> aoff(L + 1);
     for (int l = 0; l <= L; ++l) { aoff[l] = off; off += (size_t)M * net->width[l] * 4; off = (off + 255) & ~size_t(255); }
-    const size_t otn = off; off += (size_t)M * net->width[L] * 4; off = (off + 255) & ~size_t(255);
     const size_t og0 = off; off += (size_t)M * maxw * 4; off = (off + 255) & ~size_t(255);
     const size_t og1 = off; off += (size_t)M * maxw * 4; off = (off + 255) & ~size_t(255);
+    size_t ngp = 0, nbp = 0;
+    for (int l = 0; l < L; ++l) {
+        const size_t z = gemm_splits(net->width[l], net->width[l + 1], (int)M);
+        ngp = std::max(ngp, z * net->width[l] * net->width[l + 1]);
+        nbp = std::max(nbp, z * net->width[l + 1]);
+    }
+    const size_t ogp = off; off += ngp * 4; off = (off + 255) & ~size_t(255);
+    const size_t obp = off; off += nbp * 4; off = (off + 255) & ~size_t(255);
     const size_t opart = off; off += (size_t)nb * 8 + 8; off = (off + 255) & ~size_t(255);
     heom_status st = ensure_ws(net->ws, off);
     if (st != HEOM_OK) return st;
     char *base = (char *)net->ws.p;
     w.act.resize(L + 1);
     for (int l = 0; l <= L; ++l) w.act[l] = (float *)(base + aoff[l]);
-    w.tn = (float *)(base + otn);
+    w.gpart = (float *)(base + ogp);
+    w.bpart = (float *)(base + obp);
     w.g0 = (float *)(base + og0);
     w.g1 = (float *)(base + og1);
     w.part = (double *)(base + opart);
@@ -334,8 +448,8 @@ heom_status forward(heom_mlp *net, const float *x, int64_t M, Work &w, cudaStrea
     for (int l = 0; l < L; ++l) {
         const int K = net->width[l], N = net->width[l + 1];
         const float *W = P + net->w_off[l], *b = P + net->b_off[l];
-        if (l + 1 < L) HEOM_CUDA(gemm<EPI_TANH>((int)M, N, K, w.act[l], K, 0, W, N, 0, w.act[l + 1], N, b, nullptr, s));
-        else HEOM_CUDA(gemm<EPI_BIAS>((int)M, N, K, w.act[l], K, 0, W, N, 0, w.act[l + 1], N, b, nullptr, s));
+        if (l + 1 < L) HEOM_CUDA((gemm<EPI_TANH, false, false>((int)M, N, K, w.act[l], K, W, N, w.act[l + 1], N, b, nullptr, s)));
+        else HEOM_CUDA((gemm<EPI_BIAS, false, false>((int)M, N, K, w.act[l], K, W, N, w.act[l + 1], N, b, nullptr, s)));
     }
     return HEOM_OK;
 }
@@ -345,8 +459,7 @@ heom_status backward(heom_mlp *net, const float *x, const float *t, int64_t M, W
     const int L = net->n_layers, out = net->width[L];
     heom_status st = forward(net, x, M, w, s);
     if (st != HEOM_OK) return st;
-    k_standardise<<<nblk(M * out), 256, 0, s>>>(M, out, t, norm_ptr(net, 2), norm_ptr(net, 3), w.tn);
-    k_mse_grad<<<w.nblocks, 256, 0, s>>>(M * out, w.act[L], w.tn, w.g0, w.part);
+    k_mse_grad<<<w.nblocks, 256, 0, s>>>(M * out, out, w.act[L], t, norm_ptr(net, 2), norm_ptr(net, 3), w.g0, w.part);
     k_loss_finish<<<1, 256, 0, s>>>(w.nblocks, w.part, (double)M * out, w.loss);
     HEOM_CUDA(cudaGetLastError());
     const float *P = (const float *)net->params.p;
@@ -355,11 +468,13 @@ heom_status backward(heom_mlp *net, const float *x, const float *t, int64_t M, W
     for (int l = L - 1; l >= 0; --l) {
         const int K = net->width[l], N = net->width[l + 1];
         // dW_l = act_l^T g (K x N), db_l = column sums of g
-        HEOM_CUDA(gemm<EPI_STORE>(K, N, (int)M, w.act[l], K, 1, g, N, 0, G + net->w_off[l], N, nullptr, nullptr, s));
-        k_colsum<<<(N + 127) / 128, 128, 0, s>>>((int)M, N, g, G + net->b_off[l]);
+        const int z = gemm_splits(K, N, (int)M);
+        HEOM_CUDA((gemm<EPI_STORE, true, false>(K, N, (int)M, w.act[l], K, g, N, w.gpart, N, nullptr, nullptr, s, z, w.bpart)));
+        k_sum_parts<<<nblk((int64_t)K * N + N), 256, 0, s>>>(z, (int64_t)K * N, w.gpart, G + net->w_off[l], N, w.bpart,
+                                                             G + net->b_off[l]);
         HEOM_CUDA(cudaGetLastError());
         if (l > 0) {  // g_{l-1} = (g W_l^T) * (1 - act_l^2)
-            HEOM_CUDA(gemm<EPI_DTANH>((int)M, K, N, g, N, 0, P + net->w_off[l], N, 1, gp, K, nullptr, w.act[l], s));
+            HEOM_CUDA((gemm<EPI_DTANH, false, true>((int)M, K, N, g, N, P + net->w_off[l], N, gp, K, nullptr, w.act[l], s)));
             std::swap(g, gp);
         }
     }
@@ -517,7 +632,7 @@ extern "C" heom_status heom_mlp_gradients(heom_mlp *net, const float *x, const f
     if (r != HEOM_OK) return r;
     {
         heom::Prof pr(HEOM_KC_OTHER, st, (double)batch);
-        pr.kernels = 4 + 4 * net->n_layers;
+        pr.kernels = 2 + 4 * net->n_layers;
         if ((r = heom::backward(net, x, t, batch, w, st)) != HEOM_OK) return r;
     }
     if (grad_out) HEOM_CUDA(cudaMemcpyAsync(grad_out, net->grads.p, net->n_params * 4, cudaMemcpyDeviceToDevice, st));
