@@ -1,16 +1,11 @@
 // The hot path: y = M x over all ADOs and batch columns (Eq. HEOM), matrix-free.
 //
-// Mapping: one thread per output element (ADO n, element e = r*d + c, column b). A block is
-// (bx, by) threads with bx consecutive batch columns and by consecutive (n, e) rows, so a
-// warp reads 32 consecutive columns of one row (batched solves, coalesced 256/512-byte
-// segments) or 32 consecutive elements of neighbouring ADOs (batch 1). Every operand of an
-// output element -- its own block, the blocks of its raised and lowered neighbours -- is
-// read straight from global memory; re-reads of a block by its neighbours are served by L1
-// and L2. Operators are applied through their sparse row/column lists, so the d_sigma of
-// the fermionic baths cost one multiply-add per neighbour and side.
+// Two kernels: the tiled one (heom_tile.cuh) for many columns of one parameter set, and the
+// row kernel below (heom_rows.cuh) for everything else.
 #include <algorithm>
 #include <cstdint>
 
+#include "heom_block.cuh"
 #include "heom_tile.cuh"
 
 namespace heom {
@@ -31,28 +26,89 @@ Geom make_geom(int64_t rows, int64_t B, int max_blocks_x) {
     return g;
 }
 
-template <class R>
-__global__ void __launch_bounds__(256) k_apply(DevView<R> v, const cx<R> *__restrict__ x,
-                                               cx<R> *__restrict__ y, int64_t B,
-                                               int64_t cols_per_set, ApplyMods<R> mods) {
-    const int64_t b = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    const int64_t rows = v.N * v.d2;
-    if (b >= B) return;
-    const int set = (int)(b / cols_per_set);
-    for (int64_t row = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; row < rows;
-         row += (int64_t)gridDim.x * blockDim.y) {
-        const int64_t n = row / v.d2;
-        const int e = (int)(row - n * v.d2);
-        const cx<R> damp = damping_of(v, n, set);
-        cx<R> acc = apply_point(v, x, n, e, b, B, set, damp);
-        if (mods.shift) fma_to(acc, mods.shift[b], x[row * B + b]);
-        if (mods.aug != R(0) && row == 0) {
-            cx<R> tr{R(0), R(0)};
-            for (int i = 0; i < v.d; ++i) tr = tr + x[(int64_t)(i * v.d + i) * B + b];
-            acc = acc + mods.aug * tr;
-        }
-        y[row * B + b] = acc;
+// y = M x (+ shift, trace augmentation), one thread per run of elements and column
+template <class R, class Ly>
+__global__ void __launch_bounds__(256, Ly::VEC ? 3 : 1) k_apply(DevView<R> v, const cx<R> *__restrict__ x,
+                                               cx<R> *__restrict__ y, int64_t B, ColSets cps,
+                                               ApplyMods<R> mods) {
+    constexpr int NE = Ly::NE;
+    const auto s_ops = Ly::stage(v);
+    const int64_t total = v.N * Ly::per_ado(v) * B;
+    const bool small = total < (int64_t(1) << 31);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        int64_t q, b, n;
+        int e0;
+        run_col(i, B, small, q, b);
+        Ly::pos(v, q, small, n, e0);
+        const int set = cps.set(b);
+        const int64_t i0 = (n * v.d2 + e0) * B + b;
+        cx<R> x0[NE], o[NE];
+        if (beyond_cap(v, n, set)) zero_rows<R, NE>(mods.shift ? x + i0 : nullptr, B, x0, o);
+        else Ly::apply(v, s_ops, x, n, e0, b, B, set, x0, o);
+        apply_mods<R, NE>(mods, v, x, n, e0, b, B, x0, o);
+        st_row<R, NE, Ly::VEC>(y + i0, B, o);
     }
+}
+
+// One column of a large hierarchy of small blocks: 32 ADOs per warp (heom_block.cuh). The warp
+// hands its blocks through shared memory and writes whole lines.
+template <class R, int D, int W>
+__global__ void __launch_bounds__(kWarpWarps * 32) k_apply_warp(DevView<R> v, const cx<R> *__restrict__ x,
+                                                                cx<R> *__restrict__ y, ApplyMods<R> mods) {
+    constexpr int D2 = D * D, SL = warp_slot<R, D>();
+    extern __shared__ __align__(16) unsigned char warp_sm[];
+    OpRec<R> *s_ops = reinterpret_cast<OpRec<R> *>(warp_sm);
+    stage_ops<R, W>(v, s_ops);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    cx<R> *ring = reinterpret_cast<cx<R> *>(s_ops + v.n_ops * 2 * D * W) +
+                  (size_t)warp * (warp_smem<R, D>() / sizeof(cx<R>));
+    for (int64_t n0 = ((int64_t)blockIdx.x * kWarpWarps + warp) * 32; n0 < v.N;
+         n0 += (int64_t)gridDim.x * kWarpWarps * 32) {
+        const int n = n0 + lane < v.N ? __ldg(v.perm + n0 + lane) : -1;
+        cx<R> s[D2];
+        apply_warp<R, D, W>(v, s_ops, ring, x, n, s);
+        if (n >= 0) {
+            if (mods.shift) {
+                const cx<R> sh = mods.shift[0];
+#pragma unroll
+                for (int e = 0; e < D2; ++e) fma_to(s[e], sh, x[(int64_t)n * D2 + e]);
+            }
+            if (mods.aug != R(0) && n == 0) {
+                cx<R> tr{R(0), R(0)};
+                for (int k = 0; k < D; ++k) tr = tr + x[k * D + k];
+                s[0] = s[0] + mods.aug * tr;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < D2; ++e) ring[lane * SL + e] = s[e];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < D2; ++k) {
+            const int i = k * 32 + lane, blk = i / D2, e = i % D2;
+            const int to = __shfl_sync(0xffffffffu, n, blk);
+            if (to >= 0) y[(int64_t)to * D2 + e] = ring[blk * SL + e];
+        }
+    }
+}
+
+// The same for a few columns, neighbour blocks staged through shared memory (heom_staged.cuh)
+template <class R, int CW, bool BLOCK, int W>
+__global__ void __launch_bounds__(512) k_apply_staged(DevView<R> v, const cx<R> *__restrict__ x, cx<R> *__restrict__ y, int64_t B,
+                               ColSets cps, ApplyMods<R> mods, bool vec) {
+    staged_items<R, CW, BLOCK, W>(v, B, cps, [&](bool in, int64_t n, int64_t b, int set, int g, cx<R> *ring,
+                                                 const OpRec<R> *s_ops) {
+        const bool cut = beyond_cap(v, n, set);
+        const int64_t i0 = (n * v.d2 + g * CW) * B + b;
+        cx<R> x0[CW], o[CW];
+        apply_staged<R, CW, BLOCK, W>(v, s_ops, ring, x, in && !cut, n, g, b, B, set, vec, x0, o);
+        if (!in || (BLOCK && g >= v.d2 / CW)) return;
+        if (cut) zero_rows<R, CW>(mods.shift ? x + i0 : nullptr, B, x0, o);
+        apply_mods<R, CW>(mods, v, x, n, g * CW, b, B, x0, o);
+        if (vec) st_row<R, CW, true>(y + i0, B, o);
+        else st_row<R, CW, false>(y + i0, B, o);
+    });
 }
 
 template <class R>
@@ -69,9 +125,69 @@ cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t 
         a.B = B;
         return launch_tile<R, TM_STORE>(a, s);
     }
-    Geom g = make_geom(v.N * v.d2, B, 1 << 30);
-    k_apply<R><<<g.grid, g.block, 0, s>>>(v, x, y, B, B / v.n_sets, mods);
+    const ColSets cps(B / v.n_sets);
+    const bool quad = quad_ok(v, B, x, y);
+    if (warp_ok(v, B, x, y)) {
+        const unsigned grid = (unsigned)((v.N + 32 * kWarpWarps - 1) / (32 * kWarpWarps));
+#define CALL(D, W)                                                                                       \
+    do {                                                                                                 \
+        const size_t sm = warp_launch_smem<R, D>(v);                                                     \
+        const cudaError_t e =                                                                            \
+            cudaFuncSetAttribute(k_apply_warp<R, D, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm); \
+        if (e != cudaSuccess) return e;                                                                  \
+        k_apply_warp<R, D, W><<<grid, kWarpWarps * 32, sm, s>>>(v, x, y, mods);                          \
+    } while (0)
+        if (v.d == 4 && v.op_width == 1) CALL(4, 1);
+        else if (v.d == 4) CALL(4, 2);
+        else if (v.op_width == 1) CALL(2, 1);
+        else CALL(2, 2);
+#undef CALL
+        return cudaGetLastError();
+    }
+    const StageGeom sg = stage_geom(v, B);
+    if (sg.cw && !quad) {
+        const bool vec = row_vec<R>(B, x, y);
+#define CALL(CW, BLOCK, W) \
+    return launch_staged(k_apply_staged<R, CW, BLOCK, W>, sg, s, v, x, y, B, cps, mods, vec)
+        HEOM_STAGE_DISPATCH(sg, CALL);
+#undef CALL
+    }
+    const LayoutPick p = pick_layout(v, B, quad);
+    const Geom g = flat_geom(v.N * v.d2 / p.ne * B);
+#define CALL(Ly) k_apply<R, Ly><<<g.grid, g.block, p.smem, s>>>(v, x, y, B, cps, mods)
+    HEOM_FLAT_DISPATCH(R, p, CALL);
+#undef CALL
     return cudaGetLastError();
+}
+
+// damp[n][set] = sum_k count_k rate_k over the occupied exponents of ADO n, in FP64 and rounded
+// to FP32 (one table entry per ADO and set, read by every element of the ADO's block)
+__global__ void k_damping(int64_t N, int n_sets, const int32_t *__restrict__ occ_ptr, const OccEntry *__restrict__ occ,
+                          const cx<double> *__restrict__ rate, cx<double> *__restrict__ d64, cx<float> *__restrict__ d32) {
+    const int64_t total = N * n_sets;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t n = i / n_sets;
+        const int set = (int)(i - n * n_sets);
+        cx<double> a{0.0, 0.0};
+        for (int o = occ_ptr[n]; o < occ_ptr[n + 1]; ++o)
+            a = a + (double)occ[o].count * rate[(int64_t)occ[o].k * n_sets + set];
+        d64[i] = a;
+        d32[i] = cast<float>(a);
+    }
+}
+
+heom_status fill_damping(heom_hier *h, int n_sets, cudaStream_t s) {
+    const int64_t total = h->N * n_sets;
+    heom_status st = dalloc(h->d_damp64, total * sizeof(cx<double>));
+    if (st == HEOM_OK) st = dalloc(h->d_damp32, total * sizeof(cx<float>));
+    if (st != HEOM_OK) return st;
+    const Geom g = flat_geom(std::min<int64_t>(total, 152 * 16 * 256));
+    k_damping<<<g.grid, g.block, 0, s>>>(h->N, n_sets, (const int32_t *)h->d_occ_ptr.p, (const OccEntry *)h->d_occ.p,
+                                         (const cx<double> *)h->d_rate64.p, (cx<double> *)h->d_damp64.p,
+                                         (cx<float> *)h->d_damp32.p);
+    HEOM_CUDA(cudaGetLastError());
+    return HEOM_OK;
 }
 
 template cudaError_t launch_apply<double>(const DevView<double> &, const cx<double> *,
@@ -176,7 +292,7 @@ heom_status autotune(heom_hier *h, int64_t B, double *cand, int *tiled, int *per
     k_tune_fill<R><<<(unsigned)std::min<int64_t>((total + 255) / 256, 152 * 16), 256, 0, s>>>(total, x);
     const int per_sm0 = h->tile_per_sm, var0 = h->tile_var;
     const int64_t min_b0 = h->tile_min_b;
-    // candidate 0: the per-element kernel (tiled kernel switched off)
+    // candidate 0: the row kernel (tiled kernel switched off)
     h->tile_min_b = INT64_MAX;
     double t0 = 0.0;
     st = tune_time<R>(h, x, y, B, s, &t0);

@@ -18,6 +18,8 @@
 #include <mutex>
 #include <new>
 
+#include <array>
+
 #include "heom_internal.h"
 
 using heom::cx;
@@ -383,6 +385,17 @@ std::vector<cx<R>> to_cx(const std::vector<heom_c64> &v) {
     return o;
 }
 
+// operator nonzeros as records: value, column (or row) index, kind
+template <class R>
+std::vector<heom::OpRec<R>> to_rec(const std::vector<heom_c64> &v, const std::vector<int32_t> &idx) {
+    std::vector<heom::OpRec<R>> o(v.size());
+    for (size_t i = 0; i < v.size(); ++i) {
+        const int kind = v[i].im != 0.0 ? heom::OK_COMPLEX : std::fabs(v[i].re) == 1.0 ? heom::OK_UNIT : heom::OK_REAL;
+        o[i] = heom::OpRec<R>{R(v[i].re), R(v[i].im), idx[i], kind};
+    }
+    return o;
+}
+
 // float-float {hi.re, hi.im, lo.re, lo.im} of each value (hi = nearest float, lo = the
 // nearest float to the rest)
 std::vector<float4> to_ff(const std::vector<heom_c64> &v) {
@@ -406,16 +419,18 @@ void boson_ab(int kind, heom_c64 c, heom_c64 &a, heom_c64 &b) {
 heom::DevView<double> heom_hier::view64() const {
     heom::DevView<double> v{};
     v.N = N; v.d = d; v.d2 = d2; v.K = K; v.n_sets = n_sets; v.nS = nS;
+    v.n_ops = n_ops; v.op_width = op_width; v.op_real = op_real; v.perm = (const int32_t *)d_perm.p;
     v.row_ptr = (const int32_t *)d_row_ptr.p; v.ent = (const NbEntry *)d_ent.p;
     v.occ_ptr = (const int32_t *)d_occ_ptr.p; v.occ = (const OccEntry *)d_occ.p;
     v.op_rptr = (const int32_t *)d_op_rptr.p; v.op_rcol = (const int32_t *)d_op_rcol.p;
-    v.op_rval = (const cx<double> *)d_op_rval64.p;
+    v.op_rrec = (const heom::OpRec<double> *)d_op_rrec64.p;
     v.op_cptr = (const int32_t *)d_op_cptr.p; v.op_crow = (const int32_t *)d_op_crow.p;
-    v.op_cval = (const cx<double> *)d_op_cval64.p;
+    v.op_crec = (const heom::OpRec<double> *)d_op_crec64.p;
+    v.op_ell = (const heom::OpRec<double> *)d_op_ell64.p;
     v.s_ptr = (const int32_t *)d_s_ptr.p; v.s_src = (const int32_t *)d_s_src.p;
     v.s_val = (const cx<double> *)d_sval64.p; v.sdiag = (const cx<double> *)d_sdiag64.p;
     v.coefL = (const cx<double> *)d_coefL64.p; v.coefR = (const cx<double> *)d_coefR64.p;
-    v.rate = (const cx<double> *)d_rate64.p;
+    v.rate = (const cx<double> *)d_rate64.p; v.damp = (const cx<double> *)d_damp64.p;
     v.floor = (const double *)d_floor64.p;
     v.t_ptr = (const int32_t *)d_t_ptr.p; v.t_src = (const int32_t *)d_t_src.p;
     v.t_val = (const cx<double> *)d_t_val64.p;
@@ -425,6 +440,7 @@ heom::DevView<double> heom_hier::view64() const {
     v.tile_var = tile_var;
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
+    v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;
     v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_ranges = pers_ranges;
     v.pers_terms = pers_terms; v.pers_slots = pers_slots; v.pers_ados = pers_ados;
     v.op_rvalf = (const float4 *)d_op_rvalff.p; v.op_cvalf = (const float4 *)d_op_cvalff.p;
@@ -436,16 +452,18 @@ heom::DevView<double> heom_hier::view64() const {
 heom::DevView<float> heom_hier::view32() const {
     heom::DevView<float> v{};
     v.N = N; v.d = d; v.d2 = d2; v.K = K; v.n_sets = n_sets; v.nS = nS;
+    v.n_ops = n_ops; v.op_width = op_width; v.op_real = op_real; v.perm = (const int32_t *)d_perm.p;
     v.row_ptr = (const int32_t *)d_row_ptr.p; v.ent = (const NbEntry *)d_ent.p;
     v.occ_ptr = (const int32_t *)d_occ_ptr.p; v.occ = (const OccEntry *)d_occ.p;
     v.op_rptr = (const int32_t *)d_op_rptr.p; v.op_rcol = (const int32_t *)d_op_rcol.p;
-    v.op_rval = (const cx<float> *)d_op_rval32.p;
+    v.op_rrec = (const heom::OpRec<float> *)d_op_rrec32.p;
     v.op_cptr = (const int32_t *)d_op_cptr.p; v.op_crow = (const int32_t *)d_op_crow.p;
-    v.op_cval = (const cx<float> *)d_op_cval32.p;
+    v.op_crec = (const heom::OpRec<float> *)d_op_crec32.p;
+    v.op_ell = (const heom::OpRec<float> *)d_op_ell32.p;
     v.s_ptr = (const int32_t *)d_s_ptr.p; v.s_src = (const int32_t *)d_s_src.p;
     v.s_val = (const cx<float> *)d_sval32.p; v.sdiag = (const cx<float> *)d_sdiag32.p;
     v.coefL = (const cx<float> *)d_coefL32.p; v.coefR = (const cx<float> *)d_coefR32.p;
-    v.rate = (const cx<float> *)d_rate32.p;
+    v.rate = (const cx<float> *)d_rate32.p; v.damp = (const cx<float> *)d_damp32.p;
     v.floor = (const float *)d_floor32.p;
     v.t_ptr = (const int32_t *)d_t_ptr.p; v.t_src = (const int32_t *)d_t_src.p;
     v.t_val = (const cx<float> *)d_t_val32.p;
@@ -455,6 +473,7 @@ heom::DevView<float> heom_hier::view32() const {
     v.tile_var = tile_var;
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
+    v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;
     v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_ranges = pers_ranges;
     v.pers_terms = pers_terms; v.pers_slots = pers_slots; v.pers_ados = pers_ados;
     return v;
@@ -464,14 +483,14 @@ namespace {
 
 void free_all(heom_hier *h) {
     DBuf *bufs[] = {&h->d_row_ptr, &h->d_ent, &h->d_occ_ptr, &h->d_occ, &h->d_op_rptr,
-                    &h->d_op_rcol, &h->d_op_cptr, &h->d_op_crow, &h->d_op_rval64,
-                    &h->d_op_cval64, &h->d_op_rval32, &h->d_op_cval32, &h->d_s_ptr,
+                    &h->d_op_rcol, &h->d_op_cptr, &h->d_op_crow, &h->d_op_rrec64,
+                    &h->d_op_crec64, &h->d_op_rrec32, &h->d_op_crec32, &h->d_op_ell64, &h->d_op_ell32, &h->d_perm, &h->d_damp64, &h->d_damp32, &h->d_s_ptr,
                     &h->d_s_src, &h->d_sval64, &h->d_sval32, &h->d_coefL64, &h->d_coefL32,
                     &h->d_coefR64, &h->d_coefR32, &h->d_rate64, &h->d_rate32, &h->d_sdiag64,
                     &h->d_sdiag32, &h->d_tdval64, &h->d_floor64, &h->d_floor32, &h->ws,
                     &h->ws_small,
                     &h->d_t_ptr, &h->d_t_src, &h->d_t_val64, &h->d_t_val32, &h->d_cta_ado,
-                    &h->d_pers_ado, &h->d_ar_ado, &h->ws_pers, &h->d_ado_tier, &h->d_set_cap,
+                    &h->d_pers_ado, &h->d_ar_ado, &h->ws_pers, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
                     &h->d_op_rvalff, &h->d_op_cvalff, &h->d_svalff, &h->d_coefLff, &h->d_coefRff,
                     &h->d_rateff};
     for (DBuf *b : bufs) heom::dfree(*b);
@@ -633,14 +652,14 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     }
     std::vector<int32_t> sptr(d2 + 1, 0), ssrc;
     std::vector<std::vector<heom_c64>> scols;  // per kept term: values per set
-    std::vector<heom_c64> sd((size_t)n_sets * d2, heom_c64{0.0, 0.0});
+    std::vector<heom_c64> sd((size_t)n_sets * d2, heom_c64{0.0, 0.0});  // [d2][n_sets]
     for (int e = 0; e < d2; ++e) {
         for (auto &kv : terms[e]) {
             bool nz = false;
             for (const heom_c64 &v : kv.second) nz = nz || v.re != 0.0 || v.im != 0.0;
             if (!nz) continue;
             if (kv.first == e)
-                for (int s = 0; s < n_sets; ++s) sd[(size_t)s * d2 + e] = kv.second[s];
+                for (int s = 0; s < n_sets; ++s) sd[(size_t)e * n_sets + s] = kv.second[s];
             ssrc.push_back(kv.first);
             scols.push_back(kv.second);
         }
@@ -655,7 +674,7 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     std::vector<heom_c64> sval((size_t)n_sets * std::max(nS, 1), heom_c64{0.0, 0.0});
     std::vector<heom_c64> tdval((size_t)std::max(n_drive, 1) * std::max(nS, 1), heom_c64{0.0, 0.0});
     for (int j = 0; j < nS; ++j) {
-        for (int s = 0; s < n_sets; ++s) sval[(size_t)s * nS + j] = scols[j][s];
+        for (int s = 0; s < n_sets; ++s) sval[(size_t)j * n_sets + s] = scols[j][s];
         for (int k = 0; k < n_drive; ++k) tdval[(size_t)k * nS + j] = scols[j][n_sets + k];
     }
     std::vector<heom_c64> cl((size_t)n_sets * K), cr((size_t)n_sets * K), rt((size_t)n_sets * K);
@@ -673,9 +692,9 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
                 a = c;
                 b = {p.re, -p.im};
             }
-            cl[(size_t)s * K + k] = a;
-            cr[(size_t)s * K + k] = b;
-            rt[(size_t)s * K + k] = rate[(size_t)s * K + k];
+            cl[(size_t)k * n_sets + s] = a;  // device tables: [K][n_sets]
+            cr[(size_t)k * n_sets + s] = b;
+            rt[(size_t)k * n_sets + s] = rate[(size_t)s * K + k];
             double re = rate[(size_t)s * K + k].re;
             if (re > 0 && (first || re < floor)) { floor = re; first = false; }
         }
@@ -753,6 +772,7 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     UP(d_rate64, to_cx<double>(rt)); UP(d_rate32, to_cx<float>(rt));
     UP(d_floor64, fl); UP(d_floor32, fl32);
 #undef UP
+    if ((st = heom::fill_damping(h, n_sets, 0)) != HEOM_OK) return st;
     HEOM_CUDA(cudaStreamSynchronize(0));  // every upload of this call (and of the build) landed
     h->n_sets = n_sets;
     h->H0.assign(H, H + (size_t)n_sets * d * d);
@@ -846,6 +866,36 @@ void for_each_occupation(int Kb, int tb, F &&fn) {
 
 heom_status build_impl(int d, const heom_c64 *H, int n_baths, const heom_bath *baths, int tier_b,
                        int tier_f, int parity, double th, heom_hier **out);
+
+// The ADOs, ordered so that ADOs with the same sequence of exponent classes follow each other
+// (stable within: bosonic index, then fermionic tier, then the sequence of classes of the
+// occupied exponents). A class is a bath and sign nu -- one operator -- and whether the
+// coefficient is real, imaginary or complex, so the terms of such ADOs agree in everything
+// but the values. Only speed depends on it: a change of parameters leaves it valid.
+std::vector<int32_t> operator_order(const heom_hier *h, const std::vector<heom_c64> &coef) {
+    std::vector<int> cls(h->K_f);
+    std::map<std::array<int, 3>, int> seen;
+    for (int q = 0; q < h->K_f; ++q) {
+        const heom_c64 &c = coef[(size_t)h->K_b + q];
+        const int type = c.im == 0.0 ? 0 : c.re == 0.0 ? 1 : 2;
+        cls[q] = (int)seen.emplace(std::array<int, 3>{h->exp_bath[h->K_b + q], h->exp_nu[h->K_b + q], type},
+                                   (int)seen.size()).first->second;
+    }
+    std::vector<uint64_t> key((size_t)h->N_f);
+    for (int64_t f = 0; f < h->N_f; ++f) {
+        uint64_t k = 0;
+        for (uint64_t T = h->fer[(size_t)f]; T; T &= T - 1) k = k * 67 + (uint64_t)cls[__builtin_ctzll(T)] + 1;
+        key[(size_t)f] = (k & ((uint64_t(1) << 58) - 1)) | ((uint64_t)__builtin_popcountll(h->fer[(size_t)f]) << 58);
+    }
+    std::vector<int32_t> perm((size_t)h->N);
+    for (int64_t n = 0; n < h->N; ++n) perm[(size_t)n] = (int32_t)n;
+    std::stable_sort(perm.begin(), perm.end(), [&](int32_t a, int32_t b) {
+        const int64_t fa = h->full_of(a), fb = h->full_of(b);
+        const int64_t ba = fa / h->N_f, bb = fb / h->N_f;
+        return ba != bb ? ba < bb : key[(size_t)(fa % h->N_f)] < key[(size_t)(fb % h->N_f)];
+    });
+    return perm;
+}
 
 }  // namespace
 
@@ -1055,13 +1105,34 @@ heom_status build_impl(int d, const heom_c64 *H, int n_baths, const heom_bath *b
                 ocp.push_back((int32_t)ocr.size());
             }
         }
+        for (int i = 0; i < n_ops * (d + 1); ++i)
+            if (i % (d + 1) != d)
+                h->op_width = std::max(h->op_width, std::max(orp[i + 1] - orp[i], ocp[i + 1] - ocp[i]));
         heom_status st;
 #define UP(buf, vec) if ((st = upload(h->buf, vec)) != HEOM_OK) { free_all(h); delete h; return st; }
         UP(d_row_ptr, h->row_ptr); UP(d_ent, h->ent); UP(d_occ_ptr, occ_ptr); UP(d_occ, occ);
         UP(d_op_rptr, orp); UP(d_op_rcol, orc); UP(d_op_cptr, ocp); UP(d_op_crow, ocr);
-        UP(d_op_rval64, to_cx<double>(orv)); UP(d_op_cval64, to_cx<double>(ocv));
-        UP(d_op_rval32, to_cx<float>(orv)); UP(d_op_cval32, to_cx<float>(ocv));
+        UP(d_op_rrec64, to_rec<double>(orv, orc)); UP(d_op_crec64, to_rec<double>(ocv, ocr));
+        UP(d_op_rrec32, to_rec<float>(orv, orc)); UP(d_op_crec32, to_rec<float>(ocv, ocr));
         UP(d_op_rvalff, to_ff(orv)); UP(d_op_cvalff, to_ff(ocv));
+        for (const heom_c64 &z : orv) if (z.im != 0.0) h->op_real = 0;
+        if (h->op_width >= 1 && h->op_width <= 2) {  // fixed-width records
+            const int W = h->op_width;
+            std::vector<heom_c64> ev((size_t)n_ops * 2 * d * W, heom_c64{0.0, 0.0});
+            std::vector<int32_t> ei(ev.size(), -1);
+            for (int o = 0; o < n_ops; ++o)
+                for (int side = 0; side < 2; ++side)
+                    for (int e = 0; e < d; ++e) {
+                        const std::vector<int32_t> &ptr = side ? ocp : orp;
+                        const size_t at = (size_t)o * (d + 1) + e, to = (((size_t)o * 2 + side) * d + e) * W;
+                        for (int32_t j = ptr[at]; j < ptr[at + 1]; ++j) {
+                            ev[to + j - ptr[at]] = side ? ocv[j] : orv[j];
+                            ei[to + j - ptr[at]] = side ? ocr[j] : orc[j];
+                        }
+                    }
+            UP(d_op_ell64, to_rec<double>(ev, ei)); UP(d_op_ell32, to_rec<float>(ev, ei));
+        }
+        if ((d == 2 || d == 4) && h->N >= heom::kWarpMinAdos && h->N < INT32_MAX) UP(d_perm, operator_order(h, coef));
         // per-element term lists of every operator slot (tiled kernels)
         std::vector<int32_t> tp(1, 0), tsrc;
         std::vector<heom_c64> tval;
@@ -1212,6 +1283,17 @@ extern "C" heom_status heom_set_truncation(heom_hier *h, const int *tier_b, cons
                 h->kept_rowsets += h->d2;
                 ++h->set_kept[(size_t)s];
             }
+    // sets that keep exactly their leading ADOs: the kernels then test an index
+    std::vector<int32_t> end((size_t)h->n_sets);
+    bool prefix = h->N < INT32_MAX;
+    for (int s = 0; s < h->n_sets && prefix; ++s) {
+        end[(size_t)s] = (int32_t)h->set_kept[(size_t)s];
+        for (int64_t n = 0; n < h->set_kept[(size_t)s] && prefix; ++n)
+            prefix = (at[n] & 0xffff) <= tier_f[s] && (at[n] >> 16) <= tier_b[s];
+    }
+    if (prefix && (st = upload(h->d_set_end, end)) != HEOM_OK) return st;
+    h->cap_prefix = prefix;
+    h->set_end = end;
     bool mono = true;
     for (int s = 1; s < h->n_sets; ++s)
         mono = mono && tier_b[s] <= tier_b[s - 1] && tier_f[s] <= tier_f[s - 1];

@@ -63,34 +63,55 @@ struct OccEntry {  // damping term: count * rate_k
     int16_t count;
 };
 
+// One nonzero of an operator: its value, its column (row lists) or row (column lists), and its
+// kind -- fermionic annihilators hold +-1 (Jordan-Wigner signs) and most other operators are
+// real, which saves multiplications (see apply_rows).
+enum OpKind { OK_COMPLEX = 0, OK_UNIT = 1 /* +-1 */, OK_REAL = 2 };
+template <class R>
+struct alignas(16) OpRec {
+    R re, im;
+    int32_t idx, kind;
+};
+
 // Device view of a hierarchy in one precision (R = double or float).
 template <class R>
 struct DevView {
     int64_t N;          // number of ADOs
-    int d, d2, K, n_sets, nS;
+    int d, d2, K, n_sets, nS, n_ops;
+    int op_width;             // most nonzeros in a row or column of any operator
+    // fixed-width operator records [op][side][i][w], w < op_width, side 0 the nonzeros of row i
+    // and 1 those of column i, idx = -1 where there is none (null for op_width > 2)
+    const OpRec<R> *op_ell;
+    int op_real;              // 1 when every operator is real
+    // ADO order of the one-column layout (heom_block.cuh): ADOs whose neighbour entries use the
+    // same operators one after another are neighbours (null: none)
+    const int32_t *perm;
     const int32_t *row_ptr;   // [N+1]
     const NbEntry *ent;       // [E]
     const int32_t *occ_ptr;   // [N+1]
     const OccEntry *occ;      // [Eo]
-    const int32_t *op_rptr;   // [n_ops*(d+1)] absolute offsets into op_rcol/op_rval
+    const int32_t *op_rptr;   // [n_ops*(d+1)] absolute offsets into op_rcol / op_rrec
     const int32_t *op_rcol;
-    const cx<R> *op_rval;
-    const int32_t *op_cptr;   // [n_ops*(d+1)] absolute offsets into op_crow/op_cval
+    const OpRec<R> *op_rrec;  // the same nonzeros row by row as records (idx = column)
+    const int32_t *op_cptr;   // [n_ops*(d+1)] absolute offsets into op_crow / op_crec
     const int32_t *op_crow;
-    const cx<R> *op_cval;
-    const cx<R> *coefL;       // [n_sets][K]
-    const cx<R> *coefR;       // [n_sets][K]
-    const cx<R> *rate;        // [n_sets][K]
+    const OpRec<R> *op_crec;  // column by column (idx = row)
+    // Parameter-dependent tables keep the set index fastest, so that the lanes of a warp, which
+    // hold neighbouring columns (and so neighbouring sets), read one contiguous run.
+    const cx<R> *coefL;       // [K][n_sets]
+    const cx<R> *coefR;       // [K][n_sets]
+    const cx<R> *rate;        // [K][n_sets]
+    const cx<R> *damp;        // [N][n_sets]  sum_k count_k rate_k of every ADO
     const R *floor;           // [n_sets]      damping floor for undamped ADOs (preconditioner)
     // ADO-local system superoperator L_s X = -i (H X - X H) + sum_k gamma_k J(F_k)[X] (the
     // commutator of Eq. HEOM plus the Lindblad terms of Eq. Lindbladian), one term list per
     // output element: element e reads local element s_src[j] of the same ADO with coefficient
-    // s_val[set * nS + j], j = s_ptr[e] .. s_ptr[e+1]-1. Terms with the same source element
+    // s_val[j * n_sets + set], j = s_ptr[e] .. s_ptr[e+1]-1. Terms with the same source element
     // are merged; terms that vanish in every parameter set are dropped.
     const int32_t *s_ptr;     // [d2 + 1]
     const int32_t *s_src;     // [nS]
-    const cx<R> *s_val;       // [n_sets][nS]
-    const cx<R> *sdiag;       // [n_sets][d2]  coefficient of element e on itself (preconditioner)
+    const cx<R> *s_val;       // [nS][n_sets]
+    const cx<R> *sdiag;       // [d2][n_sets]  coefficient of element e on itself (preconditioner)
     // Per-element term lists of every operator, for the tiled kernels: for operator slot o
     // and output element e = r*d + c, terms t_ptr[o*d2+e] .. t_ptr[o*d2+e+1]-1 read local
     // element (t_src & 0xffff) of the source block, as a left product (bit 16 clear:
@@ -119,6 +140,8 @@ struct DevView {
     // and holds every other ADO at zero (the apply writes zero there).
     const int32_t *ado_tier;  // [N]
     const int32_t *set_cap;   // [n_sets]
+    // ADOs each set keeps, when it keeps a leading run of them for every set (else null)
+    const int32_t *set_end;   // [n_sets]
     // Float-float copies {hi.re, hi.im, lo.re, lo.im} of the FP64 tables for the float-float
     // apply (FP64 view only; null in the FP32 view)
     const float4 *op_rvalf, *op_cvalf, *s_valf, *coefLf, *coefRf, *ratef;
@@ -128,6 +151,7 @@ struct DevView {
 template <class R>
 HD bool beyond_cap(const DevView<R> &v, int64_t n, int s) {
     if (!v.set_cap) return false;
+    if (v.set_end) return n >= v.set_end[s];
     const int t = v.ado_tier[n], c = v.set_cap[s];
     return (t & 0xffff) > (c & 0xffff) || (t >> 16) > (c >> 16);
 }
@@ -180,16 +204,19 @@ struct heom_hier {
     int n_drive = 0;
     // device tables
     heom::DBuf d_row_ptr, d_ent, d_occ_ptr, d_occ;
-    heom::DBuf d_op_rptr, d_op_rcol, d_op_cptr, d_op_crow, d_op_rval64, d_op_cval64,
-        d_op_rval32, d_op_cval32, d_op_rvalff, d_op_cvalff;
+    heom::DBuf d_op_rptr, d_op_rcol, d_op_cptr, d_op_crow, d_op_rrec64, d_op_crec64,
+        d_op_rrec32, d_op_crec32, d_op_ell64, d_op_ell32, d_perm, d_op_rvalff, d_op_cvalff;
     heom::DBuf d_s_ptr, d_s_src;
     heom::DBuf d_tdval64;                   // [n_drive][nS] system-term values of -i[H_k, .]
     int nS = 0;                             // system terms (all elements)
     // tiled-kernel term lists (see DevView)
     heom::DBuf d_t_ptr, d_t_src, d_t_val64, d_t_val32;
     std::vector<int> op_terms;              // total terms of operator slot o over all elements
-    int max_terms = 0, max_entries = 0;
+    int max_terms = 0, max_entries = 0, op_width = 0, op_real = 1;
     heom::DBuf d_cta_ado, d_pers_ado;
+    heom::DBuf d_set_end;
+    std::vector<int32_t> set_end;        // its host copy
+    bool cap_prefix = false;             // every set keeps a leading run of ADOs
     heom::DBuf d_ado_tier, d_set_cap;    // per-set truncation (heom_set_truncation)
     // When the sets' truncation tiers do not increase from one set to the next, the sets that
     // keep ADO n are sets 0 .. act_ado[n]-1 (has_act), so the columns of a vector that can be
@@ -212,7 +239,7 @@ struct heom_hier {
     int ar_ranges = 0, ar_terms = 0, ar_slots = 0, ar_ados = 0;
     // device parameters (per set), both precisions and float-float
     heom::DBuf d_sval64, d_sval32, d_coefL64, d_coefL32, d_coefR64, d_coefR32, d_rate64,
-        d_rate32, d_sdiag64, d_sdiag32, d_floor64, d_floor32, d_svalff, d_coefLff, d_coefRff,
+        d_rate32, d_damp64, d_damp32, d_sdiag64, d_sdiag32, d_floor64, d_floor32, d_svalff, d_coefLff, d_coefRff,
         d_rateff;
     // solver workspace (grown on demand)
     heom::DBuf ws;
@@ -278,6 +305,8 @@ constexpr int kRangeTerms = 4096;
 constexpr int kRangeSlots = 8192;
 constexpr int kRangeAdos = 64;
 constexpr int kPersistTerms = 6144;  // terms of one persistent range (FP64: 20 B each)
+// one-column layout of small blocks: enough ADOs that every SM sub-partition has a warp of 32
+constexpr int64_t kWarpMinAdos = 32 * 608;
 constexpr int64_t kArElemWeight = 128;  // persistent Arnoldi: balance weight of one element
 
 // launch geometry shared by every row x column kernel: block (bx, by), grid (gx, gy)
@@ -313,7 +342,10 @@ struct Prof {
 cudaError_t memcpy_counted(void *dst, const void *src, size_t bytes, cudaMemcpyKind kind,
                            cudaStream_t s);
 
-// kernels (heom_kernels.cu)
+// damping sums of every (ADO, set) into h->d_damp64 / d_damp32 from the uploaded rates
+heom_status fill_damping(heom_hier *h, int n_sets, cudaStream_t s);
+
+// kernels (heom_apply.cu)
 template <class R>
 cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t B,
                          const ApplyMods<R> &mods, cudaStream_t s);

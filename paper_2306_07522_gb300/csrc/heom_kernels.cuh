@@ -1,5 +1,5 @@
-// Device building blocks shared by the kernels: the matrix-free HEOM apply at one point,
-// the block-local preconditioner and block reductions into per-column FP64 accumulators.
+// Device building blocks shared by the kernels: the damping table, the block-local
+// preconditioner and block reductions into per-column FP64 accumulators.
 #pragma once
 
 #include "heom_internal.h"
@@ -26,6 +26,18 @@ struct ColState {
     int pad_;
 };
 
+// The parameter set of batch column b: (map ? map[b] : b) / cps, where map gives the original
+// column of each column of a compacted working layout (null: the layout is the original).
+struct ColSets {
+    int64_t cps;
+    const int *map;
+    __host__ __device__ ColSets(int64_t c, const int *m = nullptr) : cps(c), map(m) {}
+    __device__ __forceinline__ int set(int64_t b) const {
+        const uint32_t c = map ? (uint32_t)__ldg(map + b) : (uint32_t)b;  // batches stay below 2^21
+        return cps == 1 ? (int)c : (int)(c / (uint32_t)cps);
+    }
+};
+
 template <class R>
 __device__ __forceinline__ cx<R> ldc(const cx<R> *p) {
     if constexpr (sizeof(R) == 8) {
@@ -37,71 +49,34 @@ __device__ __forceinline__ cx<R> ldc(const cx<R> *p) {
     }
 }
 
+// Whether parameter set `set` keeps ADO n (heom_set_truncation). Where every set keeps a leading run
+// of ADOs -- always with a single kind of bath -- that is a comparison (v.set_end), else a
+// look at the ADO's tiers.
+struct Kept {
+    const int32_t *tier = nullptr;
+    int cap = 0;
+    int64_t end = INT64_MAX;
+    template <class R>
+    __device__ __forceinline__ Kept(const DevView<R> &v, int set) {
+        if (v.set_end) {
+            end = __ldg(v.set_end + set);
+        } else if (v.set_cap) {
+            tier = v.ado_tier;
+            cap = __ldg(v.set_cap + set);
+        }
+    }
+    __device__ __forceinline__ bool operator()(int64_t n) const {
+        if (n >= end) return false;
+        if (!tier) return true;
+        const int t = __ldg(tier + n);
+        return (t & 0xffff) <= (cap & 0xffff) && (t >> 16) <= (cap >> 16);
+    }
+};
+
+// damping sum_k count_k rate_k of ADO n in parameter set `set`
 template <class R>
 __device__ __forceinline__ cx<R> damping_of(const DevView<R> &v, int64_t n, int set) {
-    cx<R> dmp{R(0), R(0)};
-    const int o1 = __ldg(v.occ_ptr + n + 1);
-    for (int o = __ldg(v.occ_ptr + n); o < o1; ++o) {
-        const int packed = __ldg(reinterpret_cast<const int *>(v.occ) + o);
-        const int k = (int)(int16_t)(packed & 0xffff);
-        const int cnt = (int)(int16_t)(packed >> 16);
-        dmp = dmp + R(cnt) * ldc(v.rate + (int64_t)set * v.K + k);
-    }
-    return dmp;
-}
-
-// (M X)[n][e][b]: Eq. HEOM evaluated at ADO n, element e = r*d + c, batch column b.
-// X points at the start of the ADO vector ([N][d2][B]). Zero for an ADO beyond the
-// truncation of the column's parameter set (heom_set_truncation): with the input zero there
-// too, this is the apply of that set's own, shallower hierarchy, whose ADOs are those of this
-// one within the set's tiers, in the same relative order (neighbours beyond the tiers are
-// not read: their couplings are the ones the truncation drops).
-template <class R>
-__device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *__restrict__ X,
-                                             int64_t n, int e, int64_t b, int64_t B, int set,
-                                             const cx<R> &damp) {
-    if (beyond_cap(v, n, set)) return cx<R>{R(0), R(0)};  // held at zero by its set's truncation
-    const int d = v.d;
-    const int r = e / d, c = e - r * d;
-    const cx<R> *Xn = X + n * v.d2 * B + b;
-    const cx<R> x0 = Xn[(int64_t)e * B];
-    cx<R> acc{-(damp.re * x0.re - damp.im * x0.im), -(damp.re * x0.im + damp.im * x0.re)};
-    // system superoperator: -i (H X - X H) plus the Lindblad terms, one merged term list
-    const cx<R> *sv = v.s_val + (int64_t)set * v.nS;
-    for (int j = __ldg(v.s_ptr + e), j1 = __ldg(v.s_ptr + e + 1); j < j1; ++j)
-        fma_to(acc, ldc(sv + j), Xn[(int64_t)__ldg(v.s_src + j) * B]);
-    // couplings to the neighbouring ADOs
-    const int cap = v.set_cap ? __ldg(v.set_cap + set) : 0;
-    const int t1 = __ldg(v.row_ptr + n + 1);
-    for (int t = __ldg(v.row_ptr + n); t < t1; ++t) {
-        const int4 raw = __ldg(reinterpret_cast<const int4 *>(v.ent) + t);
-        const int nb = raw.x;
-        if (v.set_cap) {  // a neighbour beyond the set's tiers is not in its hierarchy
-            const int tn = __ldg(v.ado_tier + nb);
-            if ((tn & 0xffff) > (cap & 0xffff) || (tn >> 16) > (cap >> 16)) continue;
-        }
-        const int op = (int)(int16_t)(raw.y & 0xffff);
-        const int k = (int)(int16_t)(raw.y >> 16);
-        const int dir = (int)(int16_t)(raw.z & 0xffff);
-        const R ml = R((int16_t)(raw.z >> 16));
-        const R mr = R((int16_t)(raw.w & 0xffff));
-        cx<R> cl, cr;  // -i * mult * (a | b)
-        if (dir > 0) {
-            cl = cx<R>{R(0), -ml};
-            cr = cx<R>{R(0), -mr};
-        } else {
-            const int64_t pk = (int64_t)set * v.K + k;
-            cl = mul_mi(ml * ldc(v.coefL + pk));
-            cr = mul_mi(mr * ldc(v.coefR + pk));
-        }
-        const cx<R> *Xb = X + (int64_t)nb * v.d2 * B + b;
-        const int base = op * (d + 1);
-        for (int j = __ldg(v.op_rptr + base + r), j1 = __ldg(v.op_rptr + base + r + 1); j < j1; ++j)
-            fma_to(acc, cl * ldc(v.op_rval + j), Xb[(int64_t)(__ldg(v.op_rcol + j) * d + c) * B]);
-        for (int j = __ldg(v.op_cptr + base + c), j1 = __ldg(v.op_cptr + base + c + 1); j < j1; ++j)
-            fma_to(acc, cr * ldc(v.op_cval + j), Xb[(int64_t)(r * d + __ldg(v.op_crow + j)) * B]);
-    }
-    return acc;
+    return ldc(v.damp + n * v.n_sets + set);
 }
 
 // Inverse of the ADO-local diagonal: 1 / (L_s[e][e] - damp + shift), with L_s[e][e] the
@@ -111,9 +86,10 @@ __device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *_
 template <class R>
 __device__ __forceinline__ cx<R> precond_inv(const DevView<R> &v, int64_t n, int e, int set,
                                              const cx<R> &damp, cx<R> shift) {
-    cx<R> loc = ldc(v.sdiag + (int64_t)set * v.d2 + e) - damp + shift;
-    if (__ldg(v.occ_ptr + n) == __ldg(v.occ_ptr + n + 1)) loc.re -= __ldg(v.floor + set);
-    return cdiv(cx<R>{R(1), R(0)}, loc);
+    cx<R> loc = ldc(v.sdiag + (int64_t)e * v.n_sets + set) - damp + shift;
+    if (n == 0) loc.re -= __ldg(v.floor + set);  // the only ADO without an occupied exponent
+    const R inv = R(1) / norm2(loc);
+    return cx<R>{inv * loc.re, -inv * loc.im};
 }
 
 // Complex Givens rotation zeroing b in (a, b): G = [c s; -conj(s) c] with c real, so that
@@ -135,29 +111,6 @@ __device__ __forceinline__ void givens_rot(cx<double> a, cx<double> b, double &c
     c = a2 * ia * inr;
     s = (ia * inr) * (a * conj(b));
     r = ((a2 + b2) * inr * ia) * a;
-}
-
-// Sum a per-thread FP64 complex value over threadIdx.y and atomically add it to acc[col].
-// Block is (bx, by) with by a power of two; every thread of the block must call this.
-__device__ __forceinline__ void block_add(double re, double im, double *acc_re, double *acc_im,
-                                          bool valid) {
-    __shared__ double sre[256], sim[256];
-    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    sre[tid] = re;
-    sim[tid] = im;
-    __syncthreads();
-    for (int s = blockDim.y >> 1; s > 0; s >>= 1) {
-        if (threadIdx.y < s) {
-            sre[tid] += sre[tid + s * blockDim.x];
-            sim[tid] += sim[tid + s * blockDim.x];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.y == 0 && valid) {
-        atomicAdd(acc_re, sre[threadIdx.x]);
-        if (acc_im) atomicAdd(acc_im, sim[threadIdx.x]);
-    }
-    __syncthreads();
 }
 
 }  // namespace heom

@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(256, 3) k_apply_ff(DevView<double> v, const fl
                 const int packed = __ldg(reinterpret_cast<const int *>(v.occ) + o);
                 const int k = (int)(int16_t)(packed & 0xffff);
                 const float cnt = (float)(int16_t)(packed >> 16);
-                const float4 rt = v.ratef[(int64_t)set * v.K + k];
+                const float4 rt = v.ratef[(int64_t)k * v.n_sets + set];
                 ff2_mac(DH, DL, make_float2(cnt, cnt), make_float2(0.f, 0.f), make_float2(rt.x, rt.y),
                         make_float2(rt.z, rt.w), make_float2(-rt.x, -rt.y));
             }
@@ -348,9 +348,9 @@ __global__ void __launch_bounds__(256, 3) k_apply_ff(DevView<double> v, const fl
 #pragma unroll
             for (int u = 0; u < CPT; ++u) cmac_ff(H[u], L[u], ndm, Xn[(int64_t)e * B + u]);
         }
-        const float4 *sv = v.s_valf + (int64_t)set * v.nS;
+        const float4 *sv = v.s_valf + set;
         for (int j = __ldg(v.s_ptr + e), j1 = __ldg(v.s_ptr + e + 1); j < j1; ++j) {
-            const float4 cv = sv[j];
+            const float4 cv = sv[(int64_t)j * v.n_sets];
             const float4 *xs = Xn + (int64_t)__ldg(v.s_src + j) * B;
 #pragma unroll
             for (int u = 0; u < CPT; ++u) cmac_ff(H[u], L[u], cv, xs[u]);
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256, 3) k_apply_ff(DevView<double> v, const fl
                 cl = make_float4(0.f, -ml, 0.f, 0.f);
                 cr = make_float4(0.f, -mr, 0.f, 0.f);
             } else {
-                const int64_t pk = (int64_t)set * v.K + k;
+                const int64_t pk = (int64_t)k * v.n_sets + set;
                 cl = mul_mi_ff(ml, v.coefLf[pk]);
                 cr = mul_mi_ff(mr, v.coefRf[pk]);
             }

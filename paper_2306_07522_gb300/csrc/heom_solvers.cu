@@ -11,6 +11,7 @@
 #include <cmath>
 #include <vector>
 
+#include "heom_block.cuh"
 #include "heom_tile.cuh"
 
 namespace heom {
@@ -38,73 +39,118 @@ __device__ __forceinline__ void reduce_add(double (&val)[NV], double *const (&ds
     }
 }
 
-// The parameter set of batch column b: (map ? map[b] : b) / cps, where map gives the original
-// column of each column of a compacted working layout (null: the layout is the original).
-struct ColSets {
-    int64_t cps;
-    const int *map;
-    __host__ __device__ ColSets(int64_t c, const int *m = nullptr) : cps(c), map(m) {}
-};
-
 #define COLUMN_PROLOGUE                                                    \
     const int64_t b = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;      \
     const bool inb = b < B;                                                \
     const int64_t rows = v.N * v.d2;                                       \
-    const int set = inb ? (int)((cps.map ? (int64_t)cps.map[b] : b) / cps.cps) : 0; \
-    (void)set;
+    const int set = inb ? cps.set(b) : 0;                                  \
+    (void)set; (void)rows;
+
+// Per-column dot products of a thread over its entries: c = sum conj(a) b and n = sum |b|^2. FP64
+// vectors in FP64; FP32 vectors in exact FP32 sums (Sum3).
+template <class R>
+struct ColDots;
+template <>
+struct ColDots<double> {
+    double re = 0, im = 0, nn = 0;
+    __device__ __forceinline__ void cross(cx<double> a, cx<double> b) {
+        re += a.re * b.re + a.im * b.im;
+        im += a.re * b.im - a.im * b.re;
+    }
+    __device__ __forceinline__ void norm(cx<double> b) { nn += norm2(b); }
+    __device__ __forceinline__ double c_re() const { return re; }
+    __device__ __forceinline__ double c_im() const { return im; }
+    __device__ __forceinline__ double n() const { return nn; }
+};
+template <>
+struct ColDots<float> {
+    Sum3 c, q;
+    __device__ __forceinline__ void cross(cx<float> a, cx<float> b) {
+        c.mac(make_float2(a.re, a.re), make_float2(b.re, b.im));
+        c.mac(make_float2(a.im, a.im), make_float2(b.im, -b.re));
+    }
+    __device__ __forceinline__ void norm(cx<float> b) {
+        const float2 x = make_float2(b.re, b.im);
+        q.mac(x, x);
+    }
+    __device__ __forceinline__ double c_re() const { return c.x(); }
+    __device__ __forceinline__ double c_im() const { return c.y(); }
+    __device__ __forceinline__ double n() const { return q.x() + q.y(); }
+};
+
+// ADO of a row, by a 32-bit division where the vector allows it
+__device__ __forceinline__ int64_t ado_of(int64_t row, int d2, int64_t rows) {
+    return rows < (int64_t(1) << 31) ? (int64_t)((uint32_t)row / (uint32_t)d2) : row / d2;
+}
+
+// The columns of a solver's working layout that can be nonzero, region by region: ADOs ado0 ..
+// ado1 - 1 of columns col0 .. col0 + acols - 1. Sets truncated at their own tiers keep a leading run
+// of ADOs, so the rows of the deepest tier, most of a hierarchy, are zero in most columns: the
+// solver's kernels start threads for the columns of a region only (before, 32 lanes a row of
+// which a third were in use). Block (x, y): region y, chunk x of its rows; the first
+// (256 / acols) acols threads each own one column, neighbouring threads neighbouring columns.
+struct ColRegion {
+    int32_t ado0, ado1, col0, acols;
+};
+constexpr int kRegThreads = 256;
+
+#define REGION_PROLOGUE                                                                           \
+    const ColRegion rg = regions[blockIdx.y];                                                     \
+    const int rstep = kRegThreads / rg.acols, lcol = threadIdx.x % rg.acols, lrun = threadIdx.x / rg.acols; \
+    const int64_t b = rg.col0 + lcol;                                                             \
+    const bool inb = lrun < rstep;                                                                \
+    const int set = inb ? cps.set(b) : 0;                                                         \
+    const bool lead = blockIdx.x == 0 && lrun == 0 && rg.ado0 == 0; /* once per column */         \
+    (void)set; (void)lead;
+
+// rows (elements) of the region this thread visits
+#define REGION_ROWS                                                                               \
+    _Pragma("unroll 4")                                                                           \
+    for (int64_t row = (int64_t)rg.ado0 * v.d2 + (int64_t)blockIdx.x * rstep + lrun,               \
+                 row_end = (int64_t)rg.ado1 * v.d2;                                               \
+         row < row_end; row += (int64_t)gridDim.x * rstep)
+// element runs of the region
+#define REGION_RUNS(Ly)                                                                           \
+    const bool small = v.N * Ly::per_ado(v) < (int64_t(1) << 31);                                 \
+    for (int64_t q = (int64_t)rg.ado0 * Ly::per_ado(v) + (int64_t)blockIdx.x * rstep + lrun,       \
+                 q_end = (int64_t)rg.ado1 * Ly::per_ado(v);                                       \
+         q < q_end; q += (int64_t)gridDim.x * rstep)
+
+// Adds the block's sums of NV per-column values to dst (fixed-order tree over the threads of a
+// column); every thread of the block calls it.
+template <int NV>
+__device__ __forceinline__ void region_add(const ColRegion &rg, double (&val)[NV], double *const (&dst)[NV], bool on) {
+    __shared__ double sh[NV][kRegThreads];
+    const int A = rg.acols, n = kRegThreads / A, k = threadIdx.x / A;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) sh[i][threadIdx.x] = val[i];
+    __syncthreads();
+    int h = 1;
+    while (h < n) h <<= 1;
+    for (h >>= 1; h > 0; h >>= 1) {
+        if (k < h && k + h < n) {
+#pragma unroll
+            for (int i = 0; i < NV; ++i) sh[i][threadIdx.x] += sh[i][threadIdx.x + h * A];
+        }
+        __syncthreads();
+    }
+    if (k == 0 && on) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i)
+            if (dst[i]) atomicAdd(dst[i], sh[i][threadIdx.x]);
+    }
+}
 
 #define ROW_LOOP _Pragma("unroll 4") \
                  for (int64_t row = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; row < rows; \
                       row += (int64_t)gridDim.x * blockDim.y)
 
-__device__ __forceinline__ bool designated() { return blockIdx.x == 0 && threadIdx.y == 0; }
-
-// ------------------------------------------------------------------ RK4
-// One fused stage of classical RK4: k = M z_in, then
-//   stage 1: acc = k,       z_out = y + dt/2 k
-//   stage 2: acc += 2k,     z_out = y + dt/2 k
-//   stage 3: acc += 2k,     z_out = y + dt k
-//   stage 4: y += dt/6 (acc + k)
-template <class R>
-__global__ void __launch_bounds__(256) k_rk4_stage(DevView<R> v, const cx<R> *__restrict__ z_in,
-                                                   cx<R> *__restrict__ z_out, cx<R> *y,
-                                                   cx<R> *__restrict__ acc, int64_t B,
-                                                   ColSets cps, R dt, int stage) {
-    COLUMN_PROLOGUE
-    if (!inb) return;
-    ROW_LOOP {
-        const int64_t n = row / v.d2;
-        const int e = (int)(row - n * v.d2);
-        const cx<R> k = apply_point(v, z_in, n, e, b, B, set, damping_of(v, n, set));
-        const int64_t i = row * B + b;
-        if (stage == 1) {
-            acc[i] = k;
-            z_out[i] = y[i] + (R(0.5) * dt) * k;
-        } else if (stage == 2) {
-            acc[i] = acc[i] + R(2) * k;
-            z_out[i] = y[i] + (R(0.5) * dt) * k;
-        } else if (stage == 3) {
-            acc[i] = acc[i] + R(2) * k;
-            z_out[i] = y[i] + dt * k;
-        } else {
-            y[i] = y[i] + (dt / R(6)) * (acc[i] + k);
-        }
-    }
-}
-
-template <class R>
-cudaError_t launch_rk4_stage(const DevView<R> &v, const cx<R> *z_in, cx<R> *z_out, cx<R> *y,
-                             cx<R> *acc, int64_t B, R dt, int stage, cudaStream_t s) {
-    const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
-    k_rk4_stage<R><<<g.grid, g.block, 0, s>>>(v, z_in, z_out, y, acc, B, B / v.n_sets, dt, stage);
-    return cudaGetLastError();
-}
-template cudaError_t launch_rk4_stage<double>(const DevView<double> &, const cx<double> *,
-                                              cx<double> *, cx<double> *, cx<double> *, int64_t,
-                                              double, int, cudaStream_t);
-template cudaError_t launch_rk4_stage<float>(const DevView<float> &, const cx<float> *,
-                                             cx<float> *, cx<float> *, cx<float> *, int64_t,
-                                             float, int, cudaStream_t);
+// the element runs of an apply kernel with per-column sums
+#define RUN_LOOP(Ly)                                                                              \
+    const int64_t runs = v.N * Ly::per_ado(v);                                                    \
+    const bool small = runs < (int64_t(1) << 31);                                                 \
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; q < runs;                    \
+         q += (int64_t)gridDim.x * blockDim.y)
 
 // ------------------------------------------------------------------ BiCGStab
 __global__ void k_state_init(ColState *st, int64_t B, const int *active) {
@@ -118,42 +164,26 @@ __global__ void k_state_init(ColState *st, int64_t B, const int *active) {
     st[b] = c;
 }
 
-// r = b - A x (or r = b when x is zero), rh = r, p = v = 0; acc_rr = (rh, r), acc_nr = |r|^2,
-// bnorm2 = |b|^2.
+// x = 0: r = b, rh = r, p = v = 0; acc_rr = (rh, r), acc_nr = |r|^2, bnorm2 = |b|^2.
 template <class R>
-__global__ void __launch_bounds__(256) k_bicg_init(DevView<R> v, const cx<R> *__restrict__ bb,
-                                                   const cx<R> *__restrict__ x, cx<R> *r,
+__global__ void __launch_bounds__(256) k_bicg_init(DevView<R> v, const cx<R> *__restrict__ bb, cx<R> *r,
                                                    cx<R> *rh, cx<R> *p, cx<R> *vv, int64_t B,
-                                                   ColSets cps, ApplyMods<R> mods, int x_zero,
-                                                   ColState *st) {
+                                                   ColSets cps, ColState *st) {
     COLUMN_PROLOGUE
     const bool act = inb && st[b].active;
-    double nr = 0, nb = 0;
+    double nr = 0;
     if (act) {
         ROW_LOOP {
             const int64_t i = row * B + b;
-            cx<R> ri = bb[i];
-            if (!x_zero) {
-                const int64_t n = row / v.d2;
-                const int e = (int)(row - n * v.d2);
-                cx<R> ax = apply_point(v, x, n, e, b, B, set, damping_of(v, n, set));
-                if (mods.shift) fma_to(ax, mods.shift[b], x[i]);
-                if (mods.aug != R(0) && row == 0) {
-                    cx<R> tr{R(0), R(0)};
-                    for (int q = 0; q < v.d; ++q) tr = tr + x[(int64_t)(q * v.d + q) * B + b];
-                    ax = ax + mods.aug * tr;
-                }
-                ri = ri - ax;
-            }
+            const cx<R> ri = bb[i];
             r[i] = ri;
             rh[i] = ri;
             p[i] = cx<R>{R(0), R(0)};
             vv[i] = cx<R>{R(0), R(0)};
             nr += (double)norm2(ri);
-            nb += (double)norm2(bb[i]);
         }
     }
-    double val[3] = {nr, nr, nb};
+    double val[3] = {nr, nr, nr};
     double *const dst[3] = {act ? &st[b].acc_rr.re : nullptr, act ? &st[b].acc_nr : nullptr,
                             act ? &st[b].bnorm2 : nullptr};
     reduce_add<3>(val, dst, act);
@@ -178,10 +208,10 @@ __global__ void __launch_bounds__(256) k_bicg_p(DevView<R> v, const cx<R> *__res
                                                 cx<R> *p, const cx<R> *__restrict__ vv,
                                                 cx<R> *__restrict__ ph, cx<R> *rh, int64_t B,
                                                 ColSets cps, const cx<R> *shift, int precond,
-                                                ColState *st) {
-    COLUMN_PROLOGUE
-    __shared__ ColScalars<R> sc[32];
-    if (threadIdx.y == 0) {
+                                                const ColRegion *__restrict__ regions, ColState *st) {
+    REGION_PROLOGUE
+    __shared__ ColScalars<R> sc[kRegThreads];
+    if (lrun == 0) {
         ColScalars<R> c{};
         c.on = inb && st[b].active;
         if (c.on) {
@@ -190,29 +220,30 @@ __global__ void __launch_bounds__(256) k_bicg_p(DevView<R> v, const cx<R> *__res
             c.a = cast<R>(cdiv(cs.acc_rr, cs.rho_old) * cdiv(cs.alpha, cs.omega));  // beta
             c.b = cast<R>(cs.omega);
         }
-        sc[threadIdx.x] = c;
+        sc[lcol] = c;
     }
     __syncthreads();
-    const ColScalars<R> c = sc[threadIdx.x];
-    if (!c.on) return;
+    const ColScalars<R> c = sc[lcol];
+    if (!c.on || !inb) return;
     const cx<R> bt = c.a, om = c.b;
     const bool rs = c.rs != 0;
     const cx<R> shv = shift ? shift[b] : cx<R>{R(0), R(0)};
-    ROW_LOOP {
-        const int64_t i = row * B + b;
+    const Kept kept(v, set);
+    REGION_ROWS {
+        const int64_t i = row * B + b, n = ado_of(row, v.d2, v.N * v.d2);
+        if (!kept(n)) continue;
         const cx<R> ri = r[i];
         const cx<R> pi = rs ? ri : ri + bt * (p[i] - om * vv[i]);
         if (rs) rh[i] = ri;
         p[i] = pi;
         if (precond) {
-            const int64_t n = row / v.d2;
             const int e = (int)(row - n * v.d2);
             ph[i] = pi * precond_inv(v, n, e, set, damping_of(v, n, set), shv);
         } else {
             ph[i] = pi;
         }
     }
-    if (designated()) {
+    if (lead) {
         st[b].acc_rv = {0.0, 0.0};
         st[b].restart = rs;
     }
@@ -221,49 +252,50 @@ __global__ void __launch_bounds__(256) k_bicg_p(DevView<R> v, const cx<R> *__res
 // out = A in (apply with shift / trace augmentation), plus FP64 dots against two vectors:
 //   mode 0 (v = A ph):  acc_rv += (rh, v)
 //   mode 1 (t = A sh):  acc_ts += (t, s), acc_tt += (t, t)
-template <class R>
+template <class R, class Ly>
 __global__ void __launch_bounds__(256) k_bicg_apply(DevView<R> v, const cx<R> *__restrict__ in,
                                                     cx<R> *__restrict__ out,
                                                     const cx<R> *__restrict__ w, int64_t B,
                                                     ColSets cps, ApplyMods<R> mods, int mode,
-                                                    ColState *st) {
-    COLUMN_PROLOGUE
+                                                    const ColRegion *__restrict__ regions, ColState *st) {
+    constexpr int NE = Ly::NE;
+    const OpRec<R> *s_ops = Ly::stage(v);
+    REGION_PROLOGUE
     const bool act = inb && st[b].active;
-    double a_re = 0, a_im = 0, tt = 0;
+    ColDots<R> dots;
     if (act) {
-        ROW_LOOP {
-            const int64_t n = row / v.d2;
-            const int e = (int)(row - n * v.d2);
-            const int64_t i = row * B + b;
-            cx<R> y = apply_point(v, in, n, e, b, B, set, damping_of(v, n, set));
-            if (mods.shift) fma_to(y, mods.shift[b], in[i]);
-            if (mods.aug != R(0) && row == 0) {
-                cx<R> tr{R(0), R(0)};
-                for (int q = 0; q < v.d; ++q) tr = tr + in[(int64_t)(q * v.d + q) * B + b];
-                y = y + mods.aug * tr;
-            }
-            out[i] = y;
-            const cx<double> yd = cast<double>(y), wd = cast<double>(w[i]);
-            if (mode == 0) {  // (rh, v) = sum conj(rh) v
-                a_re += wd.re * yd.re + wd.im * yd.im;
-                a_im += wd.re * yd.im - wd.im * yd.re;
-            } else {          // (t, s) = sum conj(t) s ; (t, t)
-                a_re += yd.re * wd.re + yd.im * wd.im;
-                a_im += yd.re * wd.im - yd.im * wd.re;
-                tt += yd.re * yd.re + yd.im * yd.im;
+        REGION_RUNS(Ly) {
+            int64_t n;
+            int e0;
+            Ly::pos(v, q, small, n, e0);
+            if (beyond_cap(v, n, set)) continue;  // zero there, and nothing reads it
+            const int64_t i0 = (n * v.d2 + e0) * B + b;
+            cx<R> x0[NE], y[NE];
+            Ly::apply(v, s_ops, in, n, e0, b, B, set, x0, y);
+            apply_mods<R, NE>(mods, v, in, n, e0, b, B, x0, y);
+            st_row<R, NE, false>(out + i0, B, y);
+#pragma unroll
+            for (int u = 0; u < NE; ++u) {
+                const cx<R> wv = ldc(w + i0 + u * B);
+                if (mode == 0) {  // (rh, v) = sum conj(rh) v
+                    dots.cross(wv, y[u]);
+                } else {          // (t, s) = sum conj(t) s ; (t, t)
+                    dots.cross(y[u], wv);
+                    dots.norm(y[u]);
+                }
             }
         }
     }
     if (mode == 0) {
-        double val[2] = {a_re, a_im};
+        double val[2] = {dots.c_re(), dots.c_im()};
         double *const dst[2] = {act ? &st[b].acc_rv.re : nullptr, act ? &st[b].acc_rv.im : nullptr};
-        reduce_add<2>(val, dst, act);
+        region_add<2>(rg, val, dst, act);
     } else {
-        double val[3] = {a_re, a_im, tt};
+        double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
         double *const dst[3] = {act ? &st[b].acc_ts.re : nullptr, act ? &st[b].acc_ts.im : nullptr,
                                 act ? &st[b].acc_tt.re : nullptr};
-        reduce_add<3>(val, dst, act);
-        if (act && designated()) {
+        region_add<3>(rg, val, dst, act);
+        if (act && lead) {
             st[b].acc_rr = {0.0, 0.0};
             st[b].acc_nr = 0.0;
         }
@@ -274,10 +306,10 @@ __global__ void __launch_bounds__(256) k_bicg_apply(DevView<R> v, const cx<R> *_
 template <class R>
 __global__ void __launch_bounds__(256) k_bicg_s(DevView<R> v, cx<R> *r, const cx<R> *__restrict__ vv,
                                                 cx<R> *__restrict__ sh, int64_t B, ColSets cps,
-                                                const cx<R> *shift, int precond, ColState *st) {
-    COLUMN_PROLOGUE
-    __shared__ ColScalars<R> sc[32];
-    if (threadIdx.y == 0) {
+                                                const cx<R> *shift, int precond, const ColRegion *__restrict__ regions, ColState *st) {
+    REGION_PROLOGUE
+    __shared__ ColScalars<R> sc[kRegThreads];
+    if (lrun == 0) {
         ColScalars<R> c{};
         c.on = inb && st[b].active;
         if (c.on) {
@@ -289,26 +321,27 @@ __global__ void __launch_bounds__(256) k_bicg_s(DevView<R> v, cx<R> *r, const cx
             c.a = cast<R>(c.keep);
             c.b = cx<R>{bad ? R(1) : R(0), R(0)};
         }
-        sc[threadIdx.x] = c;
+        sc[lcol] = c;
     }
     __syncthreads();
-    const ColScalars<R> c = sc[threadIdx.x];
-    if (!c.on) return;
+    const ColScalars<R> c = sc[lcol];
+    if (!c.on || !inb) return;
     const cx<R> al = c.a;
     const cx<R> shf = shift ? shift[b] : cx<R>{R(0), R(0)};
-    ROW_LOOP {
-        const int64_t i = row * B + b;
+    const Kept kept(v, set);
+    REGION_ROWS {
+        const int64_t i = row * B + b, n = ado_of(row, v.d2, v.N * v.d2);
+        if (!kept(n)) continue;
         const cx<R> s = r[i] - al * vv[i];
         r[i] = s;
         if (precond) {
-            const int64_t n = row / v.d2;
             const int e = (int)(row - n * v.d2);
             sh[i] = s * precond_inv(v, n, e, set, damping_of(v, n, set), shf);
         } else {
             sh[i] = s;
         }
     }
-    if (designated()) {
+    if (lead) {
         const cx<double> rr = c.rs ? cx<double>{st[b].acc_nr, 0.0} : st[b].acc_rr;
         if (c.rs) st[b].rhn = st[b].acc_nr;
         st[b].alpha = c.keep;
@@ -322,16 +355,16 @@ __global__ void __launch_bounds__(256) k_bicg_s(DevView<R> v, cx<R> *r, const cx
 // omega = (t, s) / (t, t); x += alpha ph + omega sh; r = s - omega t;
 // acc_rr += (rh, r), acc_nr += |r|^2
 template <class R>
-__global__ void __launch_bounds__(256) k_bicg_x(int64_t rows, cx<R> *x, const cx<R> *__restrict__ ph,
+__global__ void __launch_bounds__(256) k_bicg_x(DevView<R> v, cx<R> *x, const cx<R> *__restrict__ ph,
                                                 const cx<R> *__restrict__ sh, cx<R> *r,
                                                 const cx<R> *__restrict__ t,
                                                 const cx<R> *__restrict__ rh, int64_t B,
-                                                ColState *st) {
-    const int64_t b = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    __shared__ ColScalars<R> sc[32];
-    if (threadIdx.y == 0) {
+                                                ColSets cps, const ColRegion *__restrict__ regions, ColState *st) {
+    REGION_PROLOGUE
+    __shared__ ColScalars<R> sc[kRegThreads];
+    if (lrun == 0) {
         ColScalars<R> c{};
-        c.on = b < B && st[b].active;
+        c.on = inb && st[b].active;
         if (c.on) {
             const ColState cs = st[b];
             const cx<double> omega =
@@ -343,30 +376,30 @@ __global__ void __launch_bounds__(256) k_bicg_x(int64_t rows, cx<R> *x, const cx
             c.b = cast<R>(omega);
             c.on = bad ? 2 : 1;
         }
-        sc[threadIdx.x] = c;
+        sc[lcol] = c;
     }
     __syncthreads();
-    const ColScalars<R> c = sc[threadIdx.x];
-    const bool act = c.on == 1;
-    double rr_re = 0, rr_im = 0, nr = 0;
+    const ColScalars<R> c = sc[lcol];
+    const bool act = inb && c.on == 1;
+    ColDots<R> dots;
     if (act) {
         const cx<R> al = c.a, om = c.b;
-        ROW_LOOP {
+        const Kept kept(v, set);
+    REGION_ROWS {
+            if (!kept(ado_of(row, v.d2, v.N * v.d2))) continue;
             const int64_t i = row * B + b;
             x[i] = x[i] + al * ph[i] + om * sh[i];
             const cx<R> ri = r[i] - om * t[i];
             r[i] = ri;
-            const cx<double> rd = cast<double>(ri), hd = cast<double>(rh[i]);
-            rr_re += hd.re * rd.re + hd.im * rd.im;
-            rr_im += hd.re * rd.im - hd.im * rd.re;
-            nr += rd.re * rd.re + rd.im * rd.im;
+            dots.cross(rh[i], ri);
+            dots.norm(ri);
         }
     }
-    double val[3] = {rr_re, rr_im, nr};
+    double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
     double *const dst[3] = {act ? &st[b].acc_rr.re : nullptr, act ? &st[b].acc_rr.im : nullptr,
                             act ? &st[b].acc_nr : nullptr};
-    reduce_add<3>(val, dst, act);
-    if (c.on && designated()) {
+    region_add<3>(rg, val, dst, act);
+    if (c.on && lead) {
         st[b].omega = c.keep;
         if (c.on == 2) st[b].flag = 1;
     }
@@ -374,30 +407,34 @@ __global__ void __launch_bounds__(256) k_bicg_x(int64_t rows, cx<R> *x, const cx
 
 // ------------------------------------------------------------------ refinement helpers
 // r64 = b - A x64 in FP64 with |r|^2 -> acc_nr and |b|^2 -> bnorm2 of the outer state
+template <class Ly>
 __global__ void __launch_bounds__(256) k_residual64(DevView<double> v, const cx<double> *__restrict__ bb,
                                                     const cx<double> *__restrict__ x,
                                                     cx<double> *__restrict__ r, int64_t B,
                                                     ColSets cps, ApplyMods<double> mods,
                                                     ColState *st) {
+    constexpr int NE = Ly::NE;
+    const OpRec<double> *s_ops = Ly::stage(v);
     COLUMN_PROLOGUE
     const bool act = inb && st[b].active;
     double nr = 0, nb = 0;
     if (act) {
-        ROW_LOOP {
-            const int64_t n = row / v.d2;
-            const int e = (int)(row - n * v.d2);
-            const int64_t i = row * B + b;
-            cx<double> ax = apply_point(v, x, n, e, b, B, set, damping_of(v, n, set));
-            if (mods.shift) fma_to(ax, mods.shift[b], x[i]);
-            if (mods.aug != 0.0 && row == 0) {
-                cx<double> tr{0.0, 0.0};
-                for (int q = 0; q < v.d; ++q) tr = tr + x[(int64_t)(q * v.d + q) * B + b];
-                ax = ax + mods.aug * tr;
+        RUN_LOOP(Ly) {
+            int64_t n;
+            int e0;
+            Ly::pos(v, q, small, n, e0);
+            const int64_t i0 = (n * v.d2 + e0) * B + b;
+            cx<double> x0[NE], ax[NE];
+            if (beyond_cap(v, n, set)) zero_rows<double, NE>(mods.shift ? x + i0 : nullptr, B, x0, ax);
+            else Ly::apply(v, s_ops, x, n, e0, b, B, set, x0, ax);
+            apply_mods<double, NE>(mods, v, x, n, e0, b, B, x0, ax);
+#pragma unroll
+            for (int u = 0; u < NE; ++u) {
+                const cx<double> bi = bb[i0 + u * B], ri = bi - ax[u];
+                r[i0 + u * B] = ri;
+                nr += norm2(ri);
+                nb += norm2(bi);
             }
-            const cx<double> ri = bb[i] - ax;
-            r[i] = ri;
-            nr += norm2(ri);
-            nb += norm2(bb[i]);
         }
     }
     double val[2] = {nr, nb};
@@ -433,17 +470,26 @@ __global__ void k_accum(int64_t rows, cx<double> *__restrict__ x, const cx<RI> *
 }
 
 // per column: |M x|^2 and |x|^2 (FP64, no shift, no augmentation) into out[2*b], out[2*b+1]
+template <class Ly>
 __global__ void __launch_bounds__(256) k_apply_norms(DevView<double> v, const cx<double> *__restrict__ x,
                                                      int64_t B, ColSets cps, double *out) {
+    constexpr int NE = Ly::NE;
+    const OpRec<double> *s_ops = Ly::stage(v);
     COLUMN_PROLOGUE
     double mx = 0, xx = 0;
     if (inb) {
-        ROW_LOOP {
-            const int64_t n = row / v.d2;
-            const int e = (int)(row - n * v.d2);
-            const cx<double> y = apply_point(v, x, n, e, b, B, set, damping_of(v, n, set));
-            mx += norm2(y);
-            xx += norm2(x[row * B + b]);
+        RUN_LOOP(Ly) {
+            int64_t n;
+            int e0;
+            Ly::pos(v, q, small, n, e0);
+            cx<double> x0[NE], y[NE];
+            if (beyond_cap(v, n, set)) zero_rows<double, NE>(x + (n * v.d2 + e0) * B + b, B, x0, y);
+            else Ly::apply(v, s_ops, x, n, e0, b, B, set, x0, y);
+#pragma unroll
+            for (int u = 0; u < NE; ++u) {
+                mx += norm2(y[u]);
+                xx += norm2(x0[u]);
+            }
         }
     }
     double val[2] = {mx, xx};
@@ -553,12 +599,10 @@ struct SolveOut {
     std::vector<double> res;  // final relative residual sqrt(acc_nr / bnorm2)
 };
 
-// Batched right-preconditioned BiCGStab on A x = b, A = M + diag(shift) (+ trace aug).
-// Columns with active[b] = 0 are left untouched. x holds the initial guess (x_zero: zero).
 constexpr int kStallIters = 96;
 
-// Batched right-preconditioned BiCGStab on A x = b, A = M + diag(shift) (+ trace aug).
-// Columns with active[b] = 0 are left untouched. x holds the initial guess (x_zero: zero).
+// Batched right-preconditioned BiCGStab on A x = b, A = M + diag(shift) (+ trace aug), from
+// x = 0. Columns with active[b] = 0 are left untouched.
 //
 // The solver works on a compact copy of the active columns ([rows][Bc] with Bc <= B) and
 // re-compacts whenever the still-active columns fall to 60 % of the working width, so that
@@ -568,9 +612,9 @@ constexpr int kStallIters = 96;
 // rows x B (two sets of x, r, rh, p, v and the scratch ph, sh, t).
 template <class R>
 heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const cx<R> *shift,
-                     R aug, bool x_zero, double tol, int max_iter, const std::vector<int> &active,
+                     R aug, double tol, int max_iter, const std::vector<int> &active,
                      cx<R> *work, ColState *st, int *d_map, int *d_lmap, cx<R> *shift_c,
-                     SolveOut &out, cudaStream_t s) {
+                     ColRegion *d_reg, int64_t reg_cap, SolveOut &out, cudaStream_t s) {
     const DevView<R> v = view_of<R>(h);
     const int64_t rows = h->N * h->d2, L = rows * B;
     cx<R> *set_a[5], *set_b[5];
@@ -595,11 +639,10 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
     cx<R> **cur = set_a, **nxt = set_b;
     const cx<R> *shc = nullptr;
     {
-        Prof pr(HEOM_KC_OTHER, s, (double)rows * Bc, (3.0 + (x_zero ? 0 : 2)) * rows * Bc * sizeof(cx<R>));
-        pr.kernels = 1 + (x_zero ? 0 : 1) + (shift ? 1 : 0);
+        Prof pr(HEOM_KC_OTHER, s, (double)rows * Bc, 3.0 * rows * Bc * sizeof(cx<R>));
+        pr.kernels = 1 + (shift ? 1 : 0);
         k_gather_cols<R><<<flat_blocks(rows * Bc), 256, 0, s>>>(rows, bvec, B, t, Bc, d_map);
-        if (x_zero) HEOM_CUDA(cudaMemsetAsync(cur[0], 0, rows * Bc * sizeof(cx<R>), s));
-        else k_gather_cols<R><<<flat_blocks(rows * Bc), 256, 0, s>>>(rows, x, B, cur[0], Bc, d_map);
+        HEOM_CUDA(cudaMemsetAsync(cur[0], 0, rows * Bc * sizeof(cx<R>), s));
         if (shift) {
             k_gather_cols<R><<<flat_blocks(Bc), 256, 0, s>>>(1, shift, B, shift_c, Bc, d_map);
             shc = shift_c;
@@ -609,19 +652,61 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
         Prof pr(HEOM_KC_KRYLOV_VECTOR, s, (double)Bc);
         k_state_init<<<(unsigned)((Bc + 255) / 256), 256, 0, s>>>(st, Bc, d_lmap);
     }
-    auto geoms = [&](int64_t w, Geom &gd, Geom &gv) {
-        // kernels with per-column dot products: a capped grid (few atomics per column);
-        // pure vector updates: a larger grid
-        gd = make_geom(rows, w, std::max<int64_t>(1, 4096 / ((w + 31) / 32)));
-        gv = make_geom(rows, w, std::max<int64_t>(1, 16384 / ((w + 31) / 32)));
+    // geometry of the current layout: the regions of its columns (groups of at most 64), the apply's
+    // layout, and the blocks per region -- few for kernels with per-column sums (each block adds
+    // its sums with one atomic per column), more for pure vector updates
+    LayoutPick lp;
+    std::vector<ColRegion> regs;
+    dim3 ga, gd, gv;
+    Geom gi;  // start-up: every row of every column
+    auto geoms = [&]() -> heom_status {
+        lp = pick_layout(v, Bc, false, 4);  // a warp holds the rows of few ADOs from 4 columns on
+        regs.clear();
+        for (int64_t c0 = 0; c0 < Bc;) {
+            const int64_t w = Bc - c0 <= 64 ? Bc - c0 : 32;
+            std::vector<int32_t> end((size_t)w);  // ADOs each column keeps
+            for (int64_t j = 0; j < w; ++j)
+                end[(size_t)j] = !alive[(size_t)(c0 + j)] ? 0
+                                 : h->has_caps && h->cap_prefix ? h->set_end[(size_t)(cols[(size_t)(c0 + j)] / cps_g)]
+                                                                : (int32_t)h->N;
+            for (int32_t n = 0; n < h->N;) {
+                int64_t a = 0;       // columns up to the last one that keeps ADO n
+                int32_t n1 = (int32_t)h->N;
+                for (int64_t j = 0; j < w; ++j)
+                    if (end[(size_t)j] > n) { a = j + 1; n1 = std::min(n1, end[(size_t)j]); }
+                if (a == 0) break;
+                regs.push_back(ColRegion{n, n1, (int32_t)c0, (int32_t)a});
+                n = n1;
+            }
+            c0 += w;
+        }
+        if (regs.empty()) regs.push_back(ColRegion{0, 0, 0, 1});
+        if ((int64_t)regs.size() > reg_cap) {
+            set_error("BiCGStab: region table overflow");
+            return HEOM_EINVAL;
+        }
+        HEOM_CUDA(memcpy_counted(d_reg, regs.data(), regs.size() * sizeof(ColRegion), cudaMemcpyHostToDevice, s));
+        const int64_t nr = (int64_t)regs.size();
+        auto grid = [&](int ne, int64_t most) {
+            int64_t need = 1;
+            for (const ColRegion &r : regs) {
+                const int64_t step = kRegThreads / r.acols;
+                need = std::max(need, ((int64_t)(r.ado1 - r.ado0) * h->d2 / ne + step - 1) / step);
+            }
+            return dim3((unsigned)std::min(need, std::max<int64_t>(1, most / nr)), (unsigned)nr, 1);
+        };
+        ga = grid(lp.ne, 152 * 12);
+        gd = grid(1, 152 * 12);
+        gv = grid(1, 152 * 64);
+        gi = make_geom(rows, Bc, std::max<int64_t>(1, 4096 / ((Bc + 31) / 32)));
+        return HEOM_OK;
     };
-    Geom gd, gv;
-    geoms(Bc, gd, gv);
+    heom_status gst = geoms();
+    if (gst != HEOM_OK) return gst;
     {
-        ApplyMods<R> mods{shc, aug};
-        Prof pr(HEOM_KC_KRYLOV_VECTOR, s, (double)rows * Bc, (x_zero ? 5.0 : 6.0) * rows * Bc * sizeof(cx<R>));
-        k_bicg_init<R><<<gd.grid, gd.block, 0, s>>>(v, t, cur[0], cur[1], cur[2], cur[3], cur[4],
-                                                    Bc, ColSets(cps_g, d_map), mods, x_zero, st);
+        Prof pr(HEOM_KC_KRYLOV_VECTOR, s, (double)rows * Bc, 5.0 * rows * Bc * sizeof(cx<R>));
+        k_bicg_init<R><<<gi.grid, gi.block, 0, s>>>(v, t, cur[1], cur[2], cur[3], cur[4], Bc,
+                                                    ColSets(cps_g, d_map), st);
     }
     HEOM_CUDA(cudaGetLastError());
     std::vector<ColState> hs(Bc);
@@ -701,7 +786,7 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
                 Prof pr(HEOM_KC_OTHER, s, (double)Bc);
                 k_gather_cols<R><<<flat_blocks(Bc), 256, 0, s>>>(1, shift, B, shift_c, Bc, d_map);
             }
-            geoms(Bc, gd, gv);
+            if ((gst = geoms()) != HEOM_OK) return gst;
         }
         HEOM_CUDA(memcpy_counted(st, hs.data(), Bc * sizeof(ColState), cudaMemcpyHostToDevice, s));
         const int steps = std::min(check, max_iter - it);
@@ -726,19 +811,27 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
         auto launch_iter = [&](cudaStream_t q, bool prof, bool set_attr) -> cudaError_t {
             cudaError_t e = cudaSuccess;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 5.0 * e_vec); pr.on = pr.on && prof;
-              k_bicg_p<R><<<gv.grid, gv.block, 0, q>>>(v, r, p, vv, ph, rh, Bc, cps, shc, 1, st); }
+              k_bicg_p<R><<<gv, kRegThreads, 0, q>>>(v, r, p, vv, ph, rh, Bc, cps, shc, 1, d_reg, st); }
             { Prof pr(kc_apply, q, u_app, 3.0 * e_vec); pr.on = pr.on && prof;
               if (tiled) { ta.x = ph; ta.out = vv; ta.w = rh; e = launch_tile<R, TM_BICG_V>(ta, q, set_attr); }
-              else k_bicg_apply<R><<<gd.grid, gd.block, 0, q>>>(v, ph, vv, rh, Bc, cps, mods, 0, st); }
+              else {
+#define CALL(Ly) k_bicg_apply<R, Ly><<<ga, kRegThreads, lp.smem, q>>>(v, ph, vv, rh, Bc, cps, mods, 0, d_reg, st)
+                  HEOM_LAYOUT_DISPATCH(R, lp, CALL);
+#undef CALL
+              } }
             if (e != cudaSuccess) return e;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 4.0 * e_vec); pr.on = pr.on && prof;
-              k_bicg_s<R><<<gv.grid, gv.block, 0, q>>>(v, r, vv, sh, Bc, cps, shc, 1, st); }
+              k_bicg_s<R><<<gv, kRegThreads, 0, q>>>(v, r, vv, sh, Bc, cps, shc, 1, d_reg, st); }
             { Prof pr(kc_apply, q, u_app, 3.0 * e_vec); pr.on = pr.on && prof;
               if (tiled) { ta.x = sh; ta.out = t; ta.w = r; e = launch_tile<R, TM_BICG_T>(ta, q, set_attr); }
-              else k_bicg_apply<R><<<gd.grid, gd.block, 0, q>>>(v, sh, t, r, Bc, cps, mods, 1, st); }
+              else {
+#define CALL(Ly) k_bicg_apply<R, Ly><<<ga, kRegThreads, lp.smem, q>>>(v, sh, t, r, Bc, cps, mods, 1, d_reg, st)
+                  HEOM_LAYOUT_DISPATCH(R, lp, CALL);
+#undef CALL
+              } }
             if (e != cudaSuccess) return e;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 8.0 * e_vec); pr.on = pr.on && prof;
-              k_bicg_x<R><<<gd.grid, gd.block, 0, q>>>(rows, xw, ph, sh, r, t, rh, Bc, st); }
+              k_bicg_x<R><<<gd, kRegThreads, 0, q>>>(v, xw, ph, sh, r, t, rh, Bc, cps, d_reg, st); }
             return cudaGetLastError();
         };
         // Without launch accounting the iteration runs as a CUDA graph, captured once per
@@ -853,13 +946,18 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
                          2 * align_up(B * sizeof(cx<RI>));
     heom_status stt = ensure_ws(h->ws, bytes);
     if (stt != HEOM_OK) return stt;
-    stt = ensure_ws(h->ws_small, align_up(2 * B * sizeof(ColState)) + 3 * align_up(B * sizeof(int)));
+    // regions of the working layout: per group of columns at most one more than the different
+    // depths of its sets
+    const int64_t reg_cap = (B + 31) / 32 + std::min<int64_t>(B, h->n_sets) + 1;
+    stt = ensure_ws(h->ws_small, align_up(2 * B * sizeof(ColState)) + 3 * align_up(B * sizeof(int)) +
+                                     align_up(reg_cap * sizeof(ColRegion)));
     if (stt != HEOM_OK) return stt;
     ColState *st = (ColState *)h->ws_small.p;
     ColState *st_out = st + B;
     int *d_flags = (int *)((char *)h->ws_small.p + align_up(2 * B * sizeof(ColState)));
     int *d_map = (int *)((char *)d_flags + align_up(B * sizeof(int)));
     int *d_lmap = (int *)((char *)d_map + align_up(B * sizeof(int)));
+    ColRegion *d_reg = (ColRegion *)((char *)d_lmap + align_up(B * sizeof(int)));
     res.iters.assign(B, 0);
     res.refine.assign(B, 0);
     res.status.assign(B, HEOM_OK);
@@ -879,6 +977,8 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
     const DevView<double> v64 = h->view64();
     const int64_t cps = B / h->n_sets;
     const Geom gd = make_geom(rows, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
+    const LayoutPick lp = pick_layout(v64, B);
+    const Geom ga = make_geom(rows / lp.ne, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
     ApplyMods<double> m64{shift64, aug};
     std::vector<ColState> hs(B);
     std::vector<int> breakdowns(B, 0);
@@ -903,7 +1003,9 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
               ta.st = st_out; ta.B = B;
               HEOM_CUDA((launch_tile<double, TM_RESID>(ta, s)));
           } else {
-              k_residual64<<<gd.grid, gd.block, 0, s>>>(v64, b64, x64, r64, B, cps, m64, st_out);
+#define CALL(Ly) k_residual64<Ly><<<ga.grid, ga.block, lp.smem, s>>>(v64, b64, x64, r64, B, cps, m64, st_out)
+              HEOM_LAYOUT_DISPATCH(double, lp, CALL);
+#undef CALL
           } }
         HEOM_CUDA(cudaGetLastError());
         HEOM_CUDA(memcpy_counted(hs.data(), st_out, B * sizeof(ColState), cudaMemcpyDeviceToHost, s));
@@ -962,8 +1064,8 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
                                           inner_tol, inner_max, kStallIters, &o.iters[0],
                                           &o.status[0], &o.res[0], s);
         } else {
-            stt = bicgstab<RI>(h, rhs, dv, B, shift64 ? shift_in : nullptr, (RI)aug, true, inner_tol,
-                               inner_max, active, w, st, d_map, d_lmap, shift_c, o, s);
+            stt = bicgstab<RI>(h, rhs, dv, B, shift64 ? shift_in : nullptr, (RI)aug, inner_tol,
+                               inner_max, active, w, st, d_map, d_lmap, shift_c, d_reg, reg_cap, o, s);
         }
         if (stt != HEOM_OK) return stt;
         bool skip_any = false;
@@ -1035,7 +1137,7 @@ heom_status solve_system(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
 }
 
 // System-term values of H(t) = H + sum_k f_k(t) H_k at cnt consecutive samples j0 .. j0+cnt-1
-// of the drive table f [n_drive][T] (row-major): sv[j][set][t] = s_val[set][t] +
+// of the drive table f [n_drive][T] (row-major): sv[j][t][set] = s_val[t][set] +
 // sum_k f[k][j0 + j] td[k][t], formed in FP64 and stored in the apply's precision.
 template <class R>
 __global__ void k_td_sval(cx<R> *__restrict__ sv, const cx<double> *__restrict__ s_val,
@@ -1045,7 +1147,7 @@ __global__ void k_td_sval(cx<R> *__restrict__ sv, const cx<double> *__restrict__
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = i / per, r = i - j * per;
-        const int t = (int)(r % nS);
+        const int t = (int)(r / n_sets);
         cx<double> v = s_val[r];
         for (int k = 0; k < n_drive; ++k) {
             const double fk = f[(int64_t)k * T + j0 + j];
@@ -1070,8 +1172,6 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
     heom_status st = ensure_ws(h->ws, 3 * L * sizeof(cx<R>));
     if (st != HEOM_OK) return st;
     cx<R> *za = (cx<R> *)h->ws.p, *zb = za + L, *acc = za + 2 * L;
-    const Geom g = make_geom(rows, B, 1 << 30);
-    const int64_t cps = B / h->n_sets;
     const size_t blk = (size_t)h->d2 * B * sizeof(cx<R>);
     int64_t saved = 0;
     if (traj) HEOM_CUDA(memcpy_counted(traj, y, blk, cudaMemcpyDeviceToDevice, s));
@@ -1119,8 +1219,7 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
             ta.stage = st_no;
             return launch_tile<R, TM_RK4>(ta, s);
         }
-        k_rk4_stage<R><<<g.grid, g.block, 0, s>>>(vt, zi, zo, y, acc, B, cps, (R)dt, st_no);
-        return cudaGetLastError();
+        return launch_rk4_stage<R>(vt, zi, zo, y, acc, B, (R)dt, st_no, s);
     };
     auto at = [&](int64_t j) -> heom_status {
         if (!td) return HEOM_OK;
@@ -1250,14 +1349,18 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
     { Prof pr(HEOM_KC_OTHER, st, (double)L);
       k_scale_cols<double><<<flat_blocks(L), 256, 0, st>>>(L, x, batch, dfac); }
     HEOM_CUDA(cudaMemsetAsync(norms, 0, 2 * batch * sizeof(double), st));
-    const Geom gd = make_geom(rows, batch, std::max<int64_t>(1, 2048 / ((batch + 31) / 32)));
+    const LayoutPick lp = pick_layout(h->view64(), batch);
+    const Geom gd = make_geom(rows / lp.ne, batch, std::max<int64_t>(1, 2048 / ((batch + 31) / 32)));
     { Prof pr(HEOM_KC_RESIDUAL64, st, (double)h->N * batch, (double)L * sizeof(cx<double>));
       if (tile_ok(h->view64(), batch)) {
           TileArgs<double> ta{};
           ta.v = h->view64(); ta.x = x; ta.norms = norms; ta.B = batch;
           HEOM_CUDA((launch_tile<double, TM_NORMS>(ta, st)));
       } else {
-          k_apply_norms<<<gd.grid, gd.block, 0, st>>>(h->view64(), x, batch, batch / h->n_sets, norms);
+          const DevView<double> v64 = h->view64();
+#define CALL(Ly) k_apply_norms<Ly><<<gd.grid, gd.block, lp.smem, st>>>(v64, x, batch, batch / h->n_sets, norms)
+          HEOM_LAYOUT_DISPATCH(double, lp, CALL);
+#undef CALL
       } }
     std::vector<double> hn(2 * batch);
     HEOM_CUDA(memcpy_counted(hn.data(), norms, hn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -14,8 +14,8 @@
 // once per ADO per CTA instead of once per lane and term.
 //
 // Program order per element: damping, system superoperator, then every neighbour entry (left
-// products before right products), then the trace row -- the order in which the
-// per-element kernel (apply_point) adds the same terms. The FP32 sweep accumulates the real
+// products before right products), then the trace row -- the order in which the row kernel
+// (apply_rows) adds the same terms. The FP32 sweep accumulates the real
 // and imaginary parts of the coefficients in separate sums, so its rounding differs from the
 // per-element kernel's (both within FP32 accuracy of the exact apply).
 #pragma once
@@ -156,7 +156,7 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
                 cl = cx<R>{R(0), -ml};
                 cr = cx<R>{R(0), -mr};
             } else {
-                const int64_t pk = (int64_t)set * v.K + k;
+                const int64_t pk = (int64_t)k * v.n_sets + set;
                 cl = mul_mi(ml * ldc(v.coefL + pk));
                 cr = mul_mi(mr * ldc(v.coefR + pk));
             }
@@ -225,7 +225,6 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
         s_item[i] = s_off[d2 * s_pb[p] + e * (s_pb[p + 1] - s_pb[p])];
     }
     // ---------------- fill the programs
-    const cx<R> *sv = v.s_val + (int64_t)set * v.nS;
     for (int z = tid; z < n_triples; z += blockDim.x) {
         const int p = ado_of_pair(z / d2);
         const int E1 = s_pb[p + 1] - s_pb[p];
@@ -244,7 +243,7 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
         } else if (op == -1) {
             for (int j = __ldg(v.s_ptr + e), j1 = __ldg(v.s_ptr + e + 1); j < j1; ++j, ++pos) {
                 s_src[pos] = nbase + __ldg(v.s_src + j);
-                s_coef[pos] = ldc(sv + j);
+                s_coef[pos] = ldc(v.s_val + (int64_t)j * v.n_sets + set);
             }
         } else if (op == -3) {
             const cx<R> dmp = damping_of(v, (int64_t)(n0 + p), set);
