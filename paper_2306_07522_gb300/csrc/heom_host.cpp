@@ -490,7 +490,7 @@ void free_all(heom_hier *h) {
                     &h->d_sdiag32, &h->d_tdval64, &h->d_floor64, &h->d_floor32, &h->ws,
                     &h->ws_small,
                     &h->d_t_ptr, &h->d_t_src, &h->d_t_val64, &h->d_t_val32, &h->d_cta_ado,
-                    &h->d_pers_ado, &h->d_ar_ado, &h->ws_pers, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
+                    &h->d_pers_ado, &h->d_ar_ado, &h->ws_pers, &h->ws_res, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
                     &h->d_op_rvalff, &h->d_op_cvalff, &h->d_svalff, &h->d_coefLff, &h->d_coefRff,
                     &h->d_rateff};
     for (DBuf *b : bufs) heom::dfree(*b);
@@ -702,6 +702,9 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     }
     std::vector<float> fl32(fl.begin(), fl.end());
     h->nS = nS;
+    h->s_ptr = sptr;
+    h->s_src = ssrc;
+    h->res = heom::ResPlan{};  // its program follows the system terms
     // largest term program of one ADO: damping (1 per element) + system terms + neighbour
     // terms + trace row
     {
@@ -1426,6 +1429,7 @@ extern "C" void heom_destroy(heom_hier *h) {
     heom::ws_release(h->ws, h->device);
     heom::ws_release(h->ws_small, h->device);
     heom::ws_release(h->ws_pers, h->device);
+    heom::ws_release(h->ws_res, h->device);
     free_all(h);
     delete h;
 }

@@ -169,6 +169,21 @@ struct DBuf {
     size_t bytes = 0;
 };
 
+// Term program of the shared-memory RK4 (heom_resident.cu): structure only, shared by all parameter
+// sets and both precisions.
+struct ResCoef {  // l (-i a) + r (-i b): a, b of exponent k, or 1 (raised, k = -1)
+    double lre, lim, rre, rim;
+    int32_t k, pad;
+};
+struct ResPlan {
+    enum State { kNone, kBuilt, kTooLarge } state = kNone;
+    bool uploaded = false;
+    int chunks = 0, nc = 0, nS = 0;
+    std::vector<uint32_t> prog;
+    std::vector<int32_t> elem, sown, row;
+    std::vector<ResCoef> coef;
+};
+
 }  // namespace heom
 
 // The opaque handle of the public ABI.
@@ -244,6 +259,9 @@ struct heom_hier {
     // solver workspace (grown on demand)
     heom::DBuf ws;
     heom::DBuf ws_small;
+    std::vector<int32_t> s_ptr, s_src;   // system terms (host copies of d_s_ptr, d_s_src)
+    heom::ResPlan res;                   // shared-memory RK4: program, and its device copy
+    heom::DBuf ws_res;
     heom::DBuf ws_pers;  // cooperative persistent solver (vectors, block partials)
     heom::DevView<double> view64() const;
     heom::DevView<float> view32() const;
@@ -373,6 +391,15 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
                                double *rot_c, cx<double> *rot_s, cx<double> *rdiag, cx<double> *g,
                                float2 *rot_cf, float4 *rot_sf, const double *beta, double *res,
                                double tol, int *steps, bool *converged, cudaStream_t s);
+
+// RK4 of small hierarchies from shared memory (heom_resident.cu). resident_steps runs `steps` steps
+// from step0 on and writes the snapshots due in them; s_stride: elements of s_val from one sample of a
+// drive to the next (0: none, s_val unused). *done = false: the hierarchy does not fit.
+bool resident_ok(const heom_hier *h, int64_t B, int prec_bytes);
+template <class R>
+heom_status resident_steps(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t step0, int64_t steps,
+                           int64_t save, cx<R> *traj, const cx<R> *s_val, int64_t s_stride, bool *done,
+                           cudaStream_t s);
 
 // one fused RK4 stage over all ADOs and columns (the launch heom_evolve uses)
 template <class R>

@@ -1169,9 +1169,7 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
                         int64_t save_every, cx<R> *traj, const double *f_host, cudaStream_t s) {
     const DevView<R> v = view_of<R>(h);
     const int64_t rows = h->N * h->d2, L = rows * B;
-    heom_status st = ensure_ws(h->ws, 3 * L * sizeof(cx<R>));
-    if (st != HEOM_OK) return st;
-    cx<R> *za = (cx<R> *)h->ws.p, *zb = za + L, *acc = za + 2 * L;
+    heom_status st = HEOM_OK;
     const size_t blk = (size_t)h->d2 * B * sizeof(cx<R>);
     int64_t saved = 0;
     if (traj) HEOM_CUDA(memcpy_counted(traj, y, blk, cudaMemcpyDeviceToDevice, s));
@@ -1192,8 +1190,8 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
         sv = (cx<R> *)((char *)tdbuf.p + ((fb + 15) / 16) * 16);
         HEOM_CUDA(memcpy_counted(fdev, f_host, fb, cudaMemcpyHostToDevice, s));
     }
-    auto view_at = [&](int64_t j) -> heom_status {  // values of sample j (refills the chunk)
-        if (j < j0 || j >= j0 + jcnt) {
+    auto view_at = [&](int64_t j, bool first = false) -> heom_status {  // values of sample j (refills the chunk)
+        if (first || j < j0 || j >= j0 + jcnt) {
             j0 = j;
             jcnt = std::min(kTdChunk, T - j);
             Prof pr(HEOM_KC_OTHER, s, (double)(jcnt * per));
@@ -1204,6 +1202,27 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
         }
         return HEOM_OK;
     };
+    // small hierarchies: whole columns in shared memory
+    if (n_steps > 0 && resident_ok(h, B, (int)sizeof(cx<R>))) {
+        bool done = true;
+        const int64_t chunk = td ? (kTdChunk - 1) / 2 : n_steps;
+        for (int64_t n = 0; n < n_steps && done && st == HEOM_OK; n += chunk) {
+            if (td) st = view_at(2 * n, true);
+            if (st == HEOM_OK)
+                st = resident_steps<R>(h, y, B, dt, n, std::min(chunk, n_steps - n), std::max<int64_t>(save_every, 1),
+                                       traj, sv, td ? per : 0, &done, s);
+        }
+        if (st == HEOM_OK && done) HEOM_CUDA(cudaStreamSynchronize(s));
+        if (st != HEOM_OK || done) {
+            dfree(tdbuf);
+            return st;
+        }
+    }
+    if ((st = ensure_ws(h->ws, 3 * L * sizeof(cx<R>))) != HEOM_OK) {
+        dfree(tdbuf);
+        return st;
+    }
+    cx<R> *za = (cx<R> *)h->ws.p, *zb = za + L, *acc = za + 2 * L;
     TileArgs<R> ta{};
     ta.v = v;
     ta.y = y;
