@@ -114,6 +114,8 @@ __global__ void __launch_bounds__(512) k_apply_staged(DevView<R> v, const cx<R> 
 template <class R>
 cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t B,
                          const ApplyMods<R> &mods, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4)
+        if (!mods.shift && mods.aug == 0.f && dense_ok(v, B)) return launch_apply_dense(v, x, y, B, s);
     // the tiled kernel reads and writes 16-byte vectors: both buffers must be 16-byte aligned
     if (tile_ok(v, B) && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) {
         TileArgs<R> a{};

@@ -451,6 +451,7 @@ heom::DevView<double> heom_hier::view64() const {
 
 heom::DevView<float> heom_hier::view32() const {
     heom::DevView<float> v{};
+    v.dense = has_dense ? (const heom::cx<float> *)d_dense32.p : nullptr;
     v.N = N; v.d = d; v.d2 = d2; v.K = K; v.n_sets = n_sets; v.nS = nS;
     v.n_ops = n_ops; v.op_width = op_width; v.op_real = op_real; v.perm = (const int32_t *)d_perm.p;
     v.row_ptr = (const int32_t *)d_row_ptr.p; v.ent = (const NbEntry *)d_ent.p;
@@ -490,7 +491,7 @@ void free_all(heom_hier *h) {
                     &h->d_sdiag32, &h->d_tdval64, &h->d_floor64, &h->d_floor32, &h->ws,
                     &h->ws_small,
                     &h->d_t_ptr, &h->d_t_src, &h->d_t_val64, &h->d_t_val32, &h->d_cta_ado,
-                    &h->d_pers_ado, &h->d_ar_ado, &h->ws_pers, &h->ws_res, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
+                    &h->d_pers_ado, &h->d_ar_ado, &h->d_dense32, &h->ws_pers, &h->ws_res, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
                     &h->d_op_rvalff, &h->d_op_cvalff, &h->d_svalff, &h->d_coefLff, &h->d_coefRff,
                     &h->d_rateff};
     for (DBuf *b : bufs) heom::dfree(*b);
@@ -774,6 +775,16 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     UP(d_coefR64, to_cx<double>(cr)); UP(d_coefR32, to_cx<float>(cr));
     UP(d_rate64, to_cx<double>(rt)); UP(d_rate32, to_cx<float>(rt));
     UP(d_floor64, fl); UP(d_floor32, fl32);
+    // dense apply: blocks of 8 to 32 with at least a quarter of the operators' entries non-zero (term
+    // by term an entry costs about four times what it costs in a block product, zero or not)
+    size_t nnz = 0;
+    for (const heom_c64 &o : h->ops) nnz += o.re != 0.0 || o.im != 0.0;
+    h->has_dense = n_sets == 1 && n_lind == 0 && d % 8 == 0 && d <= 32 && 4 * nnz >= h->ops.size() && h->n_ops > 0;
+    if (h->has_dense) {
+        std::vector<heom_c64> dn(h->ops);
+        dn.insert(dn.end(), H, H + d2);
+        UP(d_dense32, to_cx<float>(dn));
+    }
 #undef UP
     if ((st = heom::fill_damping(h, n_sets, 0)) != HEOM_OK) return st;
     HEOM_CUDA(cudaStreamSynchronize(0));  // every upload of this call (and of the build) landed

@@ -82,6 +82,9 @@ struct DevView {
     // fixed-width operator records [op][side][i][w], w < op_width, side 0 the nonzeros of row i
     // and 1 those of column i, idx = -1 where there is none (null for op_width > 2)
     const OpRec<R> *op_ell;
+    // operators and H without zeros as [n_ops + 1][d2], H last (FP32 view; null unless one parameter
+    // set, no Lindblad terms and a block size the dense kernel takes: heom_dense.cu)
+    const cx<R> *dense;
     int op_real;              // 1 when every operator is real
     // ADO order of the one-column layout (heom_block.cuh): ADOs whose neighbour entries use the
     // same operators one after another are neighbours (null: none)
@@ -259,6 +262,8 @@ struct heom_hier {
     // solver workspace (grown on demand)
     heom::DBuf ws;
     heom::DBuf ws_small;
+    heom::DBuf d_dense32;       // operators and H for the dense apply
+    bool has_dense = false;
     std::vector<int32_t> s_ptr, s_src;   // system terms (host copies of d_s_ptr, d_s_src)
     heom::ResPlan res;                   // shared-memory RK4: program, and its device copy
     heom::DBuf ws_res;
@@ -359,6 +364,10 @@ struct Prof {
 // cudaMemcpyAsync that adds host<->device bytes to the accounting when it is on
 cudaError_t memcpy_counted(void *dst, const void *src, size_t bytes, cudaMemcpyKind kind,
                            cudaStream_t s);
+
+// FP32 apply of operators without zeros (heom_dense.cu)
+bool dense_ok(const DevView<float> &v, int64_t B);
+cudaError_t launch_apply_dense(const DevView<float> &v, const cx<float> *x, cx<float> *y, int64_t B, cudaStream_t s);
 
 // damping sums of every (ADO, set) into h->d_damp64 / d_damp32 from the uploaded rates
 heom_status fill_damping(heom_hier *h, int n_sets, cudaStream_t s);
