@@ -421,20 +421,38 @@ __global__ void __launch_bounds__(256, 3) k_apply_ff(DevView<double> v, const fl
 // step is the subdiagonal entry); column j of Hb becomes final one step later. q_0 = p_0 =
 // b / beta exactly (step 0 takes sigma = 1).
 
+// 16-byte asynchronous global -> shared copies (each thread copies and later reads only its
+// own slots, so completion of its own groups is all the ordering it needs)
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
 // part[c][i][r][b] = sum over chunk c of conj(V_i) x_r for x_0 = p (= slot nv - 1 of the
 // basis) and x_1 = z: the two dot-product sets of one step in one read of the basis, tiled
 // kD2Tile basis vectors per block as in k_multidot_ff_tiled (deterministic, per-column fixed
 // order, zero for the chunk's inactive columns).
-constexpr int kD2Tile = 6;
+// Each thread streams its rows through a ring of kD2Depth stages in shared memory filled by asynchronous
+// copies, so the loads of the next rows are in flight while it computes: bytes and
+// float-float arithmetic take about the same time here and have to overlap. The sums over a column's
+// threads are formed in float-float by all threads of the block (by one thread per column in FP64 they
+// took a third of a block's time at 32 columns). 16 sets of uneven depth, 12,951 ADOs, 140 steps: 143.6 -> 76.8 ms
+// of the solve's 336, now at the rate of the update (k_update2_ff, 85.9 ms).
+constexpr int kD2Tile = 6, kD2Depth = 3;
+constexpr size_t kD2Smem = (size_t)kD2Depth * (kD2Tile + 2) * kDotThreads * sizeof(float4);
+static_assert(kD2Depth * (kD2Tile + 2) >= 2 * kD2Tile, "the ring holds the block's sums at the end");
 __global__ void __launch_bounds__(kDotThreads, 2) k_dots2_ff_tiled(int64_t B, int nv, const float4 *__restrict__ Vf,
                                                                 int64_t vstride, const float4 *__restrict__ zf,
                                                                 cx<double> *__restrict__ part,
                                                                 const GsChunk *__restrict__ chunks) {
+    extern __shared__ float4 dring[];  // [kD2Depth][kD2Tile + 2][kDotThreads]
     const int i0 = blockIdx.x * kD2Tile, c = blockIdx.y;
     const int nt = min(kD2Tile, nv - i0);
     const GsChunk ch = chunks[c];
     const float4 *pf = Vf + (int64_t)(nv - 1) * vstride;
-    __shared__ double sre[kD2Tile][kDotThreads], sim[kD2Tile][kDotThreads];
     // accumulators of <V_k, x_r> as packed (re, im) pairs: high and low words
     float2 H[kD2Tile][2], L[kD2Tile][2];
 #pragma unroll
@@ -445,13 +463,29 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_dots2_ff_tiled(int64_t B, in
     int col, rstep;
     int64_t row;
     if (chunk_lane(ch, col, rstep, row)) {
+        auto slot = [&](int st, int k) { return dring + (size_t)(st * (kD2Tile + 2) + k) * kDotThreads + threadIdx.x; };
+        auto issue = [&](int st, int64_t rw) {
+            if (rw < ch.row1) {
+                const int64_t t = rw * B + col;
+                cp_async16(slot(st, kD2Tile), pf + t);
+                cp_async16(slot(st, kD2Tile + 1), zf + t);
+#pragma unroll
+                for (int k = 0; k < kD2Tile; ++k)
+                    if (k < nt) cp_async16(slot(st, k), V0 + (int64_t)k * vstride + t);
+            }
+            cp_async_commit();
+        };
+#pragma unroll
+        for (int q = 0; q < kD2Depth - 1; ++q) issue(q, row + (int64_t)q * rstep);
+        int st = 0;
         for (; row < ch.row1; row += rstep) {
-            const int64_t t = row * B + col;
+            issue(st == 0 ? kD2Depth - 1 : st - 1, row + (int64_t)(kD2Depth - 1) * rstep);
+            cp_async_wait<kD2Depth - 1>();
             // conj(a) x = a.re (x.re, x.im) + a.im (x.im, -x.re): the two packed products
             float2 XH[2], XL[2], nXH[2], YH[2], YL[2], nYH[2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                const float4 x = r ? zf[t] : pf[t];
+                const float4 x = *slot(st, kD2Tile + r);
                 XH[r] = make_float2(x.x, x.y);
                 XL[r] = make_float2(x.z, x.w);
                 nXH[r] = make_float2(-x.x, -x.y);
@@ -459,15 +493,12 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_dots2_ff_tiled(int64_t B, in
                 YL[r] = make_float2(x.w, -x.z);
                 nYH[r] = make_float2(-x.y, x.x);
             }
-            float4 a[kD2Tile];
-#pragma unroll
-            for (int k = 0; k < kD2Tile; ++k)
-                if (k < nt) a[k] = V0[(int64_t)k * vstride + t];
 #pragma unroll
             for (int k = 0; k < kD2Tile; ++k) {
                 if (k < nt) {
-                    const float2 ARh = make_float2(a[k].x, a[k].x), ARl = make_float2(a[k].z, a[k].z);
-                    const float2 AIh = make_float2(a[k].y, a[k].y), AIl = make_float2(a[k].w, a[k].w);
+                    const float4 a = *slot(st, k);
+                    const float2 ARh = make_float2(a.x, a.x), ARl = make_float2(a.z, a.z);
+                    const float2 AIh = make_float2(a.y, a.y), AIl = make_float2(a.w, a.w);
 #pragma unroll
                     for (int r = 0; r < 2; ++r) {
                         ff2_mac(H[k][r], L[k][r], ARh, ARl, XH[r], XL[r], nXH[r]);
@@ -475,39 +506,47 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_dots2_ff_tiled(int64_t B, in
                     }
                 }
             }
+            st = st == kD2Depth - 1 ? 0 : st + 1;
         }
+        cp_async_wait<0>();
     }
+    __syncthreads();  // every thread has used its ring
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        if (r) __syncthreads();
+    for (int k = 0; k < kD2Tile; ++k)
 #pragma unroll
-        for (int k = 0; k < kD2Tile; ++k) {
-            sre[k][threadIdx.x] = (double)H[k][r].x + (double)L[k][r].x;
-            sim[k][threadIdx.x] = (double)H[k][r].y + (double)L[k][r].y;
-        }
-        __syncthreads();
-        if (threadIdx.x < B) {
-            const int per = kDotThreads / ch.acols;
-            for (int k = 0; k < nt; ++k) {
-                double re = 0.0, im = 0.0;
-                if ((int)threadIdx.x < ch.acols)
-                    for (int q = 0; q < per; ++q) {
-                        re += sre[k][threadIdx.x + q * ch.acols];
-                        im += sim[k][threadIdx.x + q * ch.acols];
-                    }
-                part[(((int64_t)c * nv + i0 + k) * 2 + r) * B + threadIdx.x] = cx<double>{re, im};
+        for (int r = 0; r < 2; ++r) dring[(k * 2 + r) * kDotThreads + threadIdx.x] = ff_pack(H[k][r], L[k][r]);
+    __syncthreads();
+    const int per = kDotThreads / max(ch.acols, 1);
+    for (int t = threadIdx.x; t < nt * 2 * (int)B; t += kDotThreads) {
+        const int kr = t / (int)B, cl = t - kr * (int)B;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (cl < ch.acols)
+            for (int q = 0; q < per; ++q) {
+                const float4 x = dring[kr * kDotThreads + cl + q * ch.acols];
+                ff_add(acc.x, acc.z, x.x, x.z);
+                ff_add(acc.y, acc.w, x.y, x.w);
             }
-        }
+        part[((int64_t)c * nv + i0) * 2 * B + t] = ff_join(acc);
     }
 }
 
-// D[i][r][b] = sum_c part[c][i][r][b]
-__global__ void k_reduce_dots2(int nc, int nv, int64_t B, const cx<double> *__restrict__ part,
-                               cx<double> *__restrict__ D) {
-    const int64_t n = (int64_t)nv * 2 * B;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        cx<double> acc{0.0, 0.0};
-        for (int c = 0; c < nc; ++c) acc = acc + part[(int64_t)c * n + t];
+// D[i][r][b] = sum_c part[c][i][r][b]: a block takes 32 sums, its eight warps every eighth chunk each (one thread
+// per sum walked all chunks: 16.2 -> 2.1 ms in the same solve)
+__global__ void __launch_bounds__(256) k_reduce_dots2(int nc, int nv, int64_t B, const cx<double> *__restrict__ part,
+                                                      cx<double> *__restrict__ D) {
+    __shared__ cx<double> s_part[8][32];
+    const int64_t n = (int64_t)nv * 2 * B, t = (int64_t)blockIdx.x * 32 + (threadIdx.x & 31);
+    const int w = threadIdx.x >> 5;
+    cx<double> acc{0.0, 0.0};
+    if (t < n) {
+#pragma unroll 4
+        for (int c = w; c < nc; c += 8) acc = acc + ldc(part + (int64_t)c * n + t);
+    }
+    s_part[w][threadIdx.x & 31] = acc;
+    __syncthreads();
+    if (w == 0 && t < n) {
+#pragma unroll
+        for (int q = 1; q < 8; ++q) acc = acc + s_part[q][threadIdx.x];
         D[t] = acc;
     }
 }
@@ -592,16 +631,6 @@ __global__ void __launch_bounds__(256) k_dcgs_coef(int j, int mmax, int64_t B, c
         }
     }
 }
-
-// 16-byte asynchronous global -> shared copies (each thread copies and later reads only its
-// own slots, so completion of its own groups is all the ordering it needs)
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // The update of step j on the active entries (blocks stride over the chunks): slot j of the
 // basis turns from p_j into q_j = (p_j - Q_j a) / sigma (float-float; FP64 in its first
@@ -850,7 +879,8 @@ __global__ void __launch_bounds__(64) k_shift_steps(int j0, int j1, int mmax, in
                                                     cx<double> *__restrict__ rdiag, cx<double> *__restrict__ g,
                                                     const double *__restrict__ beta, double *__restrict__ res,
                                                     const float4 *__restrict__ Hbf, float2 *__restrict__ rot_cf,
-                                                    float4 *__restrict__ rot_sf, const int *__restrict__ klist) {
+                                                    float4 *__restrict__ rot_sf, const int *__restrict__ klist,
+                                                    int64_t sf) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= S) return;
     const int64_t k = klist ? klist[t] : t;
@@ -859,8 +889,8 @@ __global__ void __launch_bounds__(64) k_shift_steps(int j0, int j1, int mmax, in
     double *rc = rot_c + k * mmax;
     cx<double> *rs = rot_s + k * mmax;
     cx<double> *gk = g + k * (mmax + 1);
-    float2 *rcf = Hbf ? rot_cf + k * mmax : nullptr;
-    float4 *rsf = Hbf ? rot_sf + k * mmax : nullptr;
+    float2 *rcf = Hbf ? rot_cf + k : nullptr;  // [i][shift], sf apart: a warp's shifts read whole lines
+    float4 *rsf = Hbf ? rot_sf + k : nullptr;
     const float4 shf = ff_split(shk);
     for (int j = j0; j < j1; ++j) {
         // (the chain is walked from the stored rotations; see the comment above)
@@ -877,7 +907,7 @@ __global__ void __launch_bounds__(64) k_shift_steps(int j0, int j1, int mmax, in
                     ff_add(hi1.x, hi1.z, shf.x, shf.z);
                     ff_add(hi1.y, hi1.w, shf.y, shf.w);
                 }
-                h = ff_rot_step(rcf[i], rsf[i], hi1, h);
+                h = ff_rot_step(rcf[i * sf], rsf[i * sf], hi1, h);
             }
             hj = ff_join(h);
         } else {
@@ -896,8 +926,8 @@ __global__ void __launch_bounds__(64) k_shift_steps(int j0, int j1, int mmax, in
         rs[j] = sn;
         if (Hbf) {
             const float ch = __double2float_rn(c);
-            rcf[j] = make_float2(ch, __double2float_rn(c - (double)ch));
-            rsf[j] = ff_split(sn);
+            rcf[j * sf] = make_float2(ch, __double2float_rn(c - (double)ch));
+            rsf[j * sf] = ff_split(sn);
         }
         rdiag[k * mmax + j] = r;
         const cx<double> gj = gk[j];
@@ -1093,8 +1123,9 @@ __global__ void k_shift_solve_long(int m, int mmax, int64_t B, int64_t S, int d2
 // The same solve in float-float (any m): R(i, l) regenerated by the float-float chains from
 // Hbf and the split rotations, y_l = g_l / R(l, l) in FP64 (one division per column), the
 // back substitution's updates of g and x0 = V_0 y from the float-float tier-0 rows of the
-// basis (Vf), for the S shifts klist[0 .. S-1]. Work arrays gw [S][mmax+1] and y [S][mmax]
-// (indexed by shift) hold float-float values.
+// basis (Vf), for the S shifts klist[0 .. S-1]. Work arrays gw [mmax+1][sf] and y [mmax][sf]
+// (shift fastest, like the split rotations, so that a warp's shifts read whole lines: 33.1 -> 26.3 ms of the
+// solve above; sf = all shifts) hold float-float values.
 __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t B, int64_t S, int d2,
                                                        const float4 *__restrict__ Hbf,
                                                        const cx<double> *__restrict__ shift,
@@ -1105,21 +1136,21 @@ __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t 
                                                        const cx<double> *__restrict__ g, float4 *__restrict__ gw,
                                                        float4 *__restrict__ y, const float4 *__restrict__ Vf,
                                                        int64_t vstride, cx<double> *__restrict__ x0,
-                                                       const int *__restrict__ klist) {
+                                                       const int *__restrict__ klist, int64_t sf) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= S) return;
     const int64_t k = klist[t];
     const int64_t b = col_of[k];
     const float4 shf = ff_split(shift[k]);
-    const float2 *rcf = rot_cf + k * mmax;
-    const float4 *rsf = rot_sf + k * mmax;
-    float4 *gk = gw + k * (mmax + 1);
-    float4 *yk = y + k * mmax;
-    for (int i = 0; i < m; ++i) gk[i] = ff_split(g[k * (mmax + 1) + i]);
+    const float2 *rcf = rot_cf + k;
+    const float4 *rsf = rot_sf + k;
+    float4 *gk = gw + k;
+    float4 *yk = y + k;
+    for (int i = 0; i < m; ++i) gk[i * sf] = ff_split(g[k * (mmax + 1) + i]);
     for (int l = m - 1; l >= 0; --l) {
-        const cx<double> yl = cdiv(ff_join(gk[l]), rdiag[k * mmax + l]);
+        const cx<double> yl = cdiv(ff_join(gk[l * sf]), rdiag[k * mmax + l]);
         const float4 yf = ff_split(yl);
-        yk[l] = yf;
+        yk[l * sf] = yf;
         const float4 nyf = make_float4(-yf.x, -yf.y, -yf.z, -yf.w);
         float4 carry = Hbf[hb_at(0, l, mmax, B, b)];
         if (l == 0) {
@@ -1132,8 +1163,8 @@ __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t 
                 ff_add(a1.x, a1.z, shf.x, shf.z);
                 ff_add(a1.y, a1.w, shf.y, shf.w);
             }
-            const float2 c = rcf[i];
-            const float4 sn = rsf[i];
+            const float2 c = rcf[i * sf];
+            const float4 sn = rsf[i * sf];
             // R(i, l) = c carry + s a1; carry <- c a1 - conj(s) carry
             float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
             ff_mac(rh, rl, c.x, c.y, carry.x, carry.z);
@@ -1143,17 +1174,17 @@ __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t 
             ff_norm(ih, il);
             carry = ff_rot_step(c, sn, a1, carry);
             // g_i -= R(i, l) y_l
-            float4 gi = gk[i];
+            float4 gi = gk[i * sf];
             float gr = gi.x, grl = gi.z, gim = gi.y, gil = gi.w;
             ff_cmac(gr, grl, gim, gil, make_float4(rh, ih, rl, il), nyf);
             ff_norm(gr, grl);
             ff_norm(gim, gil);
-            gk[i] = make_float4(gr, gim, grl, gil);
+            gk[i * sf] = make_float4(gr, gim, grl, gil);
         }
     }
     for (int e = 0; e < d2; ++e) {
         float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-        for (int l = 0; l < m; ++l) ff_cmac(rh, rl, ih, il, Vf[(int64_t)l * vstride + (int64_t)e * B + b], yk[l]);
+        for (int l = 0; l < m; ++l) ff_cmac(rh, rl, ih, il, Vf[(int64_t)l * vstride + (int64_t)e * B + b], yk[l * sf]);
         x0[k * d2 + e] = cx<double>{(double)rh + (double)rl, (double)ih + (double)il};
     }
 }
@@ -1279,6 +1310,7 @@ static heom_status dcgs_process(heom_hier *h, int64_t B, int64_t S, int mmax, do
     HEOM_CUDA(cudaGetDevice(&dev));
     HEOM_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     HEOM_CUDA(cudaFuncSetAttribute(k_update2_ff, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUpSmem));
+    HEOM_CUDA(cudaFuncSetAttribute(k_dots2_ff_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kD2Smem));
     HEOM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_update2_ff, kDotThreads, kUpSmem));
     std::vector<int> cur((size_t)B);  // original column of each current column
     for (int64_t c = 0; c < B; ++c) cur[(size_t)c] = (int)c;
@@ -1324,7 +1356,7 @@ static heom_status dcgs_process(heom_hier *h, int64_t B, int64_t S, int mmax, do
         Prof pr(HEOM_KC_OTHER, s, (double)nk, (double)nk * mf * 16);
         k_shift_solve_ff<<<(unsigned)((nk + 63) / 64), 64, 0, s>>>(mf, mmax, Bc, nk, d2, bf.Hbf, bf.shift, bf.col_of,
                                                                    bf.rot_cf, bf.rot_sf, bf.rdiag, bf.g, bf.gw, bf.y,
-                                                                   Vc, Lc, bf.x0, klist);
+                                                                   Vc, Lc, bf.x0, klist, S);
         HEOM_CUDA(cudaGetLastError());
         return HEOM_OK;
     };
@@ -1347,9 +1379,9 @@ static heom_status dcgs_process(heom_hier *h, int64_t B, int64_t S, int mmax, do
         {   // one read of the basis for the dots, one for the update
             Prof pr(HEOM_KC_KRYLOV_VECTOR, s, (double)(j + 1) * Lg, (2.0 * j + 6.0) * Lg * 16);
             pr.kernels = 4;
-            k_dots2_ff_tiled<<<dim3((unsigned)((j + 1 + kD2Tile - 1) / kD2Tile), (unsigned)nch), kDotThreads, 0, s>>>(
+            k_dots2_ff_tiled<<<dim3((unsigned)((j + 1 + kD2Tile - 1) / kD2Tile), (unsigned)nch), kDotThreads, kD2Smem, s>>>(
                 Bc, j + 1, Vc, Lc, zf, bf.part, bf.ch);
-            k_reduce_dots2<<<blocks_for((int64_t)(j + 1) * 2 * Bc), 256, 0, s>>>(nch, j + 1, Bc, bf.part, bf.D);
+            k_reduce_dots2<<<(unsigned)(((int64_t)(j + 1) * 2 * Bc + 31) / 32), 256, 0, s>>>(nch, j + 1, Bc, bf.part, bf.D);
             k_dcgs_coef<<<(unsigned)Bc, 256, 0, s>>>(j, mmax, Bc, bf.D, Hc, bf.cfa, bf.cft, bf.rsig);
             k_update2_ff<<<gsu, kDotThreads, kUpSmem, s>>>(Bc, j, Vc, Lc, nullptr, 0, bf.cfa, bf.cft, bf.rsig, bf.uch,
                                                            nuch);
@@ -1365,7 +1397,7 @@ static heom_status dcgs_process(heom_hier *h, int64_t B, int64_t S, int mmax, do
                                                                                           bf.Hbf);
             k_shift_steps<<<(unsigned)((act.size() + 63) / 64), 64, 0, s>>>(
                 j_done, mf, mmax, Bc, (int64_t)act.size(), Hc, bf.shift, bf.col_of, bf.rot_c, bf.rot_s, bf.rdiag, bf.g,
-                bc, bf.res, bf.Hbf, bf.rot_cf, bf.rot_sf, bf.klist);
+                bc, bf.res, bf.Hbf, bf.rot_cf, bf.rot_sf, bf.klist, S);
         }
         j_done = mf;
         HEOM_CUDA(memcpy_counted(hres.data(), bf.res, S * 8, cudaMemcpyDeviceToHost, s));
@@ -1733,7 +1765,7 @@ heom_status shifted_gmres(heom_hier *h, const cx<double> *bvec, int64_t B,
                 Prof pr(HEOM_KC_OTHER, s, (double)S * (mf - j_done), 0.0);
                 k_shift_steps<<<(unsigned)((S + 63) / 64), 64, 0, s>>>(j_done, mf, mmax, B, S, Hb, dsh, dco, rot_c,
                                                                       rot_s, rdiag, g, beta, dres, nullptr, nullptr,
-                                                                      nullptr, nullptr);
+                                                                      nullptr, nullptr, 0);
             }
             j_done = mf;
             HEOM_CUDA(memcpy_counted(hres.data(), dres, S * 8, cudaMemcpyDeviceToHost, s));
