@@ -51,6 +51,22 @@ __global__ void __launch_bounds__(256, Ly::VEC ? 3 : 1) k_apply(DevView<R> v, co
     }
 }
 
+// y = M x for the launches of point_ok: threadIdx.x over columns, threadIdx.y over elements
+template <class R>
+__global__ void __launch_bounds__(256) k_apply_point(DevView<R> v, const cx<R> *__restrict__ x, cx<R> *__restrict__ y,
+                                                     int64_t B, ColSets cps, ApplyMods<R> mods) {
+    const int b = blockIdx.y * blockDim.x + threadIdx.x, rows = (int)v.N * v.d2;
+    const int row = blockIdx.x * blockDim.y + threadIdx.y;
+    if (b >= B || row >= rows) return;
+    const int n = row / v.d2, e = row - n * v.d2, set = cps.set(b);
+    const int64_t i0 = (int64_t)row * B + b;
+    cx<R> x0[1], o[1];
+    if (beyond_cap(v, n, set)) zero_rows<R, 1>(mods.shift ? x + i0 : nullptr, B, x0, o);
+    else o[0] = apply_point(v, x, n, e, b, B, set, x0[0]);
+    apply_mods<R, 1>(mods, v, x, n, e, b, B, x0, o);
+    y[i0] = o[0];
+}
+
 // One column of a large hierarchy of small blocks: 32 ADOs per warp (heom_block.cuh). The warp
 // hands its blocks through shared memory and writes whole lines.
 template <class R, int D, int W>
@@ -147,6 +163,11 @@ cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t 
         return cudaGetLastError();
     }
     const StageGeom sg = stage_geom(v, B);
+    if (point_ok(v, B)) {
+        const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
+        k_apply_point<R><<<g.grid, g.block, 0, s>>>(v, x, y, B, cps, mods);
+        return cudaGetLastError();
+    }
     if (sg.cw && !quad) {
         const bool vec = row_vec<R>(B, x, y);
 #define CALL(CW, BLOCK, W) \

@@ -316,7 +316,60 @@ __device__ __forceinline__ void apply_cols(const DevView<R> &v, const OpRec<R> *
     for (int u = 0; u < RP * D; ++u) s[u] = acc.value(u);
 }
 
+// ---------------------------------------------------------------- small launches
+// y = (M X)[n][e][b] term by term, one element per thread. Most threads and least bookkeeping per thread: the
+// fastest layout while a launch does not fill the chip. Term order as in apply_rows.
+template <class R>
+__device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *__restrict__ X, int64_t n, int e,
+                                             int64_t b, int64_t B, int set, cx<R> &x0) {
+    const int d = v.d, ns = v.n_sets, r = e / d, c = e - r * d;
+    const cx<R> *Xn = X + n * v.d2 * B + b;
+    x0 = ldc(Xn + e * B);
+    const cx<R> dmp = ldc(v.damp + n * ns + set);
+    cx<R> acc{-(dmp.re * x0.re - dmp.im * x0.im), -(dmp.re * x0.im + dmp.im * x0.re)};
+    for (int j = __ldg(v.s_ptr + e), j1 = __ldg(v.s_ptr + e + 1); j < j1; ++j)
+        fma_to(acc, ldc(v.s_val + (int64_t)j * ns + set), ldc(Xn + __ldg(v.s_src + j) * B));
+    const Kept kept(v, set);
+    const int t1 = __ldg(v.row_ptr + n + 1);
+    for (int t = __ldg(v.row_ptr + n); t < t1; ++t) {
+        const int4 raw = __ldg(reinterpret_cast<const int4 *>(v.ent) + t);
+        if (!kept(raw.x)) continue;  // beyond the set's tiers: not in its hierarchy
+        const R ml = R((int16_t)(raw.z >> 16)), mr = R((int16_t)(raw.w & 0xffff));
+        cx<R> cl{R(0), -ml}, cr{R(0), -mr};
+        if ((int16_t)(raw.z & 0xffff) <= 0) {
+            const int64_t pk = (int64_t)(raw.y >> 16) * ns + set;
+            cl = mul_mi(ml * ldc(v.coefL + pk));
+            cr = mul_mi(mr * ldc(v.coefR + pk));
+        }
+        const cx<R> *Xb = X + (int64_t)raw.x * v.d2 * B + b;
+        const int base = (int)(int16_t)(raw.y & 0xffff) * (d + 1);
+        for (int j = __ldg(v.op_rptr + base + r), j1 = __ldg(v.op_rptr + base + r + 1); j < j1; ++j) {
+            const OpRec<R> o = ld_rec(v.op_rrec + j);
+            fma_to(acc, cl * cx<R>{o.re, o.im}, ldc(Xb + (o.idx * d + c) * B));
+        }
+        for (int j = __ldg(v.op_cptr + base + c), j1 = __ldg(v.op_cptr + base + c + 1); j < j1; ++j) {
+            const OpRec<R> o = ld_rec(v.op_crec + j);
+            fma_to(acc, cr * cx<R>{o.re, o.im}, ldc(Xb + (r * d + o.idx) * B));
+        }
+    }
+    return acc;
+}
+
 // ---------------------------------------------------------------- choice
+// Whether a launch runs one element per thread in (32 columns x 8 elements) blocks. FP32, several columns: the
+// wider layouts need enough threads to pay off (d = 4, 16 and more columns: 25 ADOs x 17 columns 17.3 against 24.4
+// us, 2,325 x 16 29.5 against 25.4; fewer columns: 2,325 x 8 23.2 against 27.9, 12,951 x 3 48 against 32);
+// larger blocks have them only where 32-column blocks stand half empty (charge-cavity model, 790 ADOs of
+// 24 x 24: 16 columns 327 against 345 us, 17 columns 627 against 382). FP64: the smallest launches (25 ADOs x 5
+// columns 33.9 against 37.8 us).
+template <class R>
+inline bool point_ok(const DevView<R> &v, int64_t B) {
+    const double el = (double)v.N * v.d2 * (double)B;
+    if (B < 2 || el >= 2147483647.0) return false;
+    if (sizeof(R) == 8) return el < 5e3;
+    if (v.d <= 4) return el < (B >= 16 ? 430e3 : 590e3);
+    return B <= 16 || el < 800e3 || (double)((B + 31) / 32 * 32) < 1.5 * (double)B;
+}
 // Whether the FP32 one-column kernel runs a launch: d a multiple of four, real operators with at
 // most two nonzeros per row and column, 16-byte aligned buffers.
 inline bool quad_ok(const DevView<float> &v, int64_t B, const void *a, const void *b, const void *c = nullptr,
@@ -411,6 +464,23 @@ struct ColsLayout {  // RP rows of a small block, operators in shared memory
     }
 };
 
+template <class R>
+struct PointLayout {  // one element
+    static constexpr int NE = 1;
+    static constexpr bool VEC = false;
+    static __host__ __device__ int per_ado(const DevView<R> &v) { return v.d2; }
+    static __device__ __forceinline__ const OpRec<R> *stage(const DevView<R> &) { return nullptr; }
+    static __device__ __forceinline__ void pos(const DevView<R> &v, int64_t q, bool small, int64_t &n, int &e0) {
+        n = small ? (int64_t)((uint32_t)q / (uint32_t)v.d2) : q / v.d2;
+        e0 = (int)(q - n * v.d2);
+    }
+    static __device__ __forceinline__ void apply(const DevView<R> &v, const OpRec<R> *, const cx<R> *__restrict__ X,
+                                                 int64_t n, int e0, int64_t b, int64_t B, int set, cx<R> (&x0)[1],
+                                                 cx<R> (&y)[1]) {
+        y[0] = apply_point(v, X, n, e0, b, B, set, x0[0]);
+    }
+};
+
 // Layout of a launch: cw > 0 the row layout, quad the FP32 one-column layout, else rows/w of the
 // many-column one.
 struct LayoutPick {
@@ -446,6 +516,10 @@ inline LayoutPick pick_layout(const DevView<R> &v, int64_t B, bool quad = false,
     p.cw = p.ne = row_width(v.N, v.d, B);
     return p;
 }
+// one element per thread: FP64 leaves out the zero halves of coefficients
+template <class R>
+using OneLayout = std::conditional_t<sizeof(R) == 8, RowsLayout<R, 1>, PointLayout<R>>;
+
 // CALL(Layout) of a pick
 #define HEOM_COLS_W(R, D, RP, w, CALL)                                                          \
     do {                                                                                        \
@@ -456,7 +530,7 @@ inline LayoutPick pick_layout(const DevView<R> &v, int64_t B, bool quad = false,
     do {                                                                                        \
         if ((p).cw == 4) { using Ly = RowsLayout<R, 4>; CALL(Ly); }                             \
         else if ((p).cw == 2) { using Ly = RowsLayout<R, 2>; CALL(Ly); }                        \
-        else if ((p).cw == 1) { using Ly = RowsLayout<R, 1>; CALL(Ly); }                        \
+        else if ((p).cw == 1) { using Ly = OneLayout<R>; CALL(Ly); }                            \
         else if ((p).d == 2) HEOM_COLS_W(R, 2, 2, (p).w, CALL);                                 \
         else if ((p).rows == 4) HEOM_COLS_W(R, 4, 4, (p).w, CALL);                              \
         else HEOM_COLS_W(R, 4, 1, (p).w, CALL);                                                 \

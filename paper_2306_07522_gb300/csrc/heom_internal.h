@@ -328,8 +328,9 @@ constexpr int kRangeTerms = 4096;
 constexpr int kRangeSlots = 8192;
 constexpr int kRangeAdos = 64;
 constexpr int kPersistTerms = 6144;  // terms of one persistent range (FP64: 20 B each)
-// one-column layout of small blocks: enough ADOs that every SM sub-partition has a warp of 32
-constexpr int64_t kWarpMinAdos = 32 * 608;
+// FP64 one-column layout of small blocks, two warps of 32 ADOs per SM sub-partition (29,317 ADOs of 4 x 4: 220 us
+// this way, 97 us staged in groups of threads; 396,607 ADOs: 418 us this way)
+constexpr int64_t kWarpMinAdos = 64 * 608;
 constexpr int64_t kArElemWeight = 128;  // persistent Arnoldi: balance weight of one element
 
 // launch geometry shared by every row x column kernel: block (bx, by), grid (gx, gy)

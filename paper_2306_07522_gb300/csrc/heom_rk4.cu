@@ -51,6 +51,20 @@ __global__ void __launch_bounds__(256, Ly::VEC ? 3 : 1) k_rk4_stage(DevView<R> v
     }
 }
 
+// the launches of point_ok: threadIdx.x over columns, threadIdx.y over elements
+template <class R>
+__global__ void __launch_bounds__(256) k_rk4_point(DevView<R> v, const cx<R> *__restrict__ z_in, cx<R> *z_out, cx<R> *y,
+                                                   cx<R> *acc, int64_t B, ColSets cps, R dt, int stage) {
+    const int b = blockIdx.y * blockDim.x + threadIdx.x, rows = (int)v.N * v.d2;
+    const int row = blockIdx.x * blockDim.y + threadIdx.y;
+    if (b >= B || row >= rows) return;
+    const int n = row / v.d2, e = row - n * v.d2, set = cps.set(b);
+    cx<R> x0[1], k[1];
+    if (beyond_cap(v, n, set)) zero_rows<R, 1>(nullptr, B, x0, k);
+    else k[0] = apply_point(v, z_in, n, e, b, B, set, x0[0]);
+    rk4_update<R, 1, false>((int64_t)row * B + b, B, k, z_out, y, acc, dt, stage);
+}
+
 // a few columns: neighbour blocks staged through shared memory (heom_staged.cuh)
 template <class R, int CW, bool BLOCK, int W>
 __global__ void __launch_bounds__(512) k_rk4_staged(DevView<R> v, const cx<R> *__restrict__ z_in, cx<R> *z_out, cx<R> *y, cx<R> *acc,
@@ -74,6 +88,11 @@ cudaError_t launch_rk4_stage(const DevView<R> &v, const cx<R> *z_in, cx<R> *z_ou
     const ColSets cps(B / v.n_sets);
     const bool quad = quad_ok(v, B, z_in, z_out, y, acc);
     const StageGeom sg = stage_geom(v, B);
+    if (point_ok(v, B)) {
+        const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
+        k_rk4_point<R><<<g.grid, g.block, 0, s>>>(v, z_in, z_out, y, acc, B, cps, dt, stage);
+        return cudaGetLastError();
+    }
     if (sg.cw && !quad) {
         const bool vec = row_vec<R>(B, z_in, z_out, y, acc);
 #define CALL(CW, BLOCK, W) \
