@@ -1125,7 +1125,8 @@ __global__ void k_shift_solve_long(int m, int mmax, int64_t B, int64_t S, int d2
 // back substitution's updates of g and x0 = V_0 y from the float-float tier-0 rows of the
 // basis (Vf), for the S shifts klist[0 .. S-1]. Work arrays gw [mmax+1][sf] and y [mmax][sf]
 // (shift fastest, like the split rotations, so that a warp's shifts read whole lines: 33.1 -> 26.3 ms of the
-// solve above; sf = all shifts) hold float-float values.
+// solve above, with the loads of kSsBatch rows in flight 15.0 ms; sf = all shifts) hold float-float values.
+constexpr int kSsBatch = 4;
 __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t B, int64_t S, int d2,
                                                        const float4 *__restrict__ Hbf,
                                                        const cx<double> *__restrict__ shift,
@@ -1157,29 +1158,41 @@ __global__ void __launch_bounds__(64) k_shift_solve_ff(int m, int mmax, int64_t 
             ff_add(carry.x, carry.z, shf.x, shf.z);
             ff_add(carry.y, carry.w, shf.y, shf.w);
         }
-        for (int i = 0; i < l; ++i) {
-            float4 a1 = Hbf[hb_at(i + 1, l, mmax, B, b)];
-            if (i + 1 == l) {
-                ff_add(a1.x, a1.z, shf.x, shf.z);
-                ff_add(a1.y, a1.w, shf.y, shf.w);
+        for (int i0 = 0; i0 < l; i0 += kSsBatch) {  // the loads of kSsBatch rows in flight together
+            float2 cv[kSsBatch];
+            float4 sv[kSsBatch], av[kSsBatch], gv[kSsBatch];
+#pragma unroll
+            for (int u = 0; u < kSsBatch; ++u) {
+                const int i = i0 + u < l ? i0 + u : l - 1;
+                cv[u] = rcf[i * sf];
+                sv[u] = rsf[i * sf];
+                av[u] = Hbf[hb_at(i + 1, l, mmax, B, b)];
+                gv[u] = gk[i * sf];
             }
-            const float2 c = rcf[i * sf];
-            const float4 sn = rsf[i * sf];
-            // R(i, l) = c carry + s a1; carry <- c a1 - conj(s) carry
-            float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
-            ff_mac(rh, rl, c.x, c.y, carry.x, carry.z);
-            ff_mac(ih, il, c.x, c.y, carry.y, carry.w);
-            ff_cmac(rh, rl, ih, il, sn, a1);
-            ff_norm(rh, rl);
-            ff_norm(ih, il);
-            carry = ff_rot_step(c, sn, a1, carry);
-            // g_i -= R(i, l) y_l
-            float4 gi = gk[i * sf];
-            float gr = gi.x, grl = gi.z, gim = gi.y, gil = gi.w;
-            ff_cmac(gr, grl, gim, gil, make_float4(rh, ih, rl, il), nyf);
-            ff_norm(gr, grl);
-            ff_norm(gim, gil);
-            gk[i * sf] = make_float4(gr, gim, grl, gil);
+#pragma unroll
+            for (int u = 0; u < kSsBatch; ++u) {
+                const int i = i0 + u;
+                if (i >= l) break;
+                float4 a1 = av[u];
+                if (i + 1 == l) {
+                    ff_add(a1.x, a1.z, shf.x, shf.z);
+                    ff_add(a1.y, a1.w, shf.y, shf.w);
+                }
+                // R(i, l) = c carry + s a1; carry <- c a1 - conj(s) carry
+                float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+                ff_mac(rh, rl, cv[u].x, cv[u].y, carry.x, carry.z);
+                ff_mac(ih, il, cv[u].x, cv[u].y, carry.y, carry.w);
+                ff_cmac(rh, rl, ih, il, sv[u], a1);
+                ff_norm(rh, rl);
+                ff_norm(ih, il);
+                carry = ff_rot_step(cv[u], sv[u], a1, carry);
+                // g_i -= R(i, l) y_l
+                float gr = gv[u].x, grl = gv[u].z, gim = gv[u].y, gil = gv[u].w;
+                ff_cmac(gr, grl, gim, gil, make_float4(rh, ih, rl, il), nyf);
+                ff_norm(gr, grl);
+                ff_norm(gim, gil);
+                gk[i * sf] = make_float4(gr, gim, grl, gil);
+            }
         }
     }
     for (int e = 0; e < d2; ++e) {
@@ -1262,7 +1275,10 @@ static int64_t make_chunks(const std::vector<int> &acols, int d2, std::vector<Gs
         n = n1;
     }
     for (const GsChunk &c0 : ch) {
-        const int64_t rows_c = c0.row1 - c0.row0, ustep = std::max<int64_t>(1, (rows_c + 7) / 8);
+        // at most eight pieces, each a whole number of the update's passes (kUpRows rows per thread): a piece of 2.8
+        // rows per thread took the time of four
+        const int64_t rows_c = c0.row1 - c0.row0, pass = (int64_t)kUpRows * std::max(1, kDotThreads / c0.acols),
+                      ustep = std::max<int64_t>(1, (rows_c + 8 * pass - 1) / (8 * pass)) * pass;
         for (int64_t r = c0.row0; r < c0.row1; r += ustep)
             uch.push_back(GsChunk{(int32_t)r, (int32_t)std::min<int64_t>(c0.row1, r + ustep), c0.acols, 0});
     }
