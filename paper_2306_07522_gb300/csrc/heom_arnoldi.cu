@@ -50,14 +50,15 @@ struct ArnoldiArgs {
     const double *beta;
     double *res;
     double tol;
-    double *part;      // per CTA: dot partials [2][kArMaxSteps + 2][B] complex, norm [B], res max
+    double *part;      // per CTA: dot partials [2][kArMaxSteps + 2][B] complex
     cx<double> *hred;  // reduced h of the two passes [2][kArMaxSteps + 2][B]
     GridBar *bar;
     long long wait_cycles;  // bound of every grid-barrier wait (SM clock cycles)
     int *out;          // [0] steps done, [1] converged, [2] barrier failure
 };
 
-constexpr int kPartStride = 2 * 2 * (kArMaxSteps + 2) * kArMaxB + kArMaxB + 2;  // doubles per CTA
+constexpr int kPartStride = 2 * 2 * (kArMaxSteps + 2) * kArMaxB;  // doubles per CTA
+static_assert(kArMaxB <= kBarVals, "the norms travel with a barrier");
 
 __device__ __forceinline__ float4 ld_l2_f4(const float4 *p) { return __ldcg(p); }
 
@@ -138,7 +139,7 @@ __device__ void slice_reduce(const ArnoldiArgs &a, int pass, int nv) {
 }
 
 __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
-    unsigned gen = 0;
+    BarState gen;
     const DevView<double> &v = a.v;
     const int d2 = v.d2, B = (int)a.B, G = gridDim.x;
     const int n0 = __ldg(v.pers_ado + blockIdx.x), n1 = __ldg(v.pers_ado + blockIdx.x + 1);
@@ -152,9 +153,11 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
     double *s_red = reinterpret_cast<double *>(s_hf + a.hcap);     // [32][kArMaxB]
     double *s_nrm = s_red + 32 * kArMaxB;                              // [kArMaxB]
     double *s_ib2 = s_nrm + kArMaxB;                                   // [kArMaxB] 1 / beta^2
-    int *s_flag = reinterpret_cast<int *>(s_ib2 + kArMaxB);           // [2 + kArMaxB]
+    double *s_sum = s_ib2 + kArMaxB;                                   // [kBarVals] exchanged by a barrier
+    int *s_flag = reinterpret_cast<int *>(s_sum + kBarVals);           // [2 + kArMaxB]
     ProgSmem<double> ps = prog_layout<double>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
-                                              reinterpret_cast<unsigned char *>(s_flag + 4));
+                                              reinterpret_cast<unsigned char *>(s_flag + 4 + kArMaxB));
+    __shared__ float2 s_nf[kArMaxB];  // 1 / |w| in float-float
     if (threadIdx.x < B) {
         const double bt = a.beta[threadIdx.x];
         s_ib2[threadIdx.x] = bt > 0.0 ? 1.0 / (bt * bt) : 0.0;
@@ -200,9 +203,9 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         __syncthreads();
         // ---- 2. Gram-Schmidt pass 1 (+ |w|^2 as the dot of w with itself, slot j + 1)
         own_dots(a, W, j + 2, e0, nel, mypart);
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
+        if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
         slice_reduce(a, 0, j + 2);
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
+        if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
         for (int p = tid; p < (j + 2) * B; p += bd) {  // written by other CTAs: through L2
             const double2 hv = __ldcg(reinterpret_cast<const double2 *>(a.hred + p));
             const cx<double> h{hv.x, hv.y};
@@ -232,9 +235,9 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         for (int pass = 0; pass < 1 + need2; ++pass) {
             if (pass == 1) {
                 own_dots(a, W, j + 1, e0, nel, mypart + 2 * (kArMaxSteps + 2) * kArMaxB);
-                if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
+                if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
                 slice_reduce(a, 1, j + 1);
-                if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
+                if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
                 for (int p = tid; p < (j + 1) * B; p += bd) {
                     const double2 hv = __ldcg(reinterpret_cast<const double2 *>(
                         a.hred + (int64_t)(kArMaxSteps + 2) * kArMaxB + p));
@@ -292,30 +295,29 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
                 double sacc = lane < (bd >> 5) ? s_red[lane * kArMaxB + warp] : 0.0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) sacc += __shfl_down_sync(0xffffffffu, sacc, o);
-                if (lane == 0) mypart[4 * (kArMaxSteps + 2) * kArMaxB + warp] = sacc;
+                if (lane == 0) s_nrm[warp] = sacc;
             }
+            __syncthreads();
         }
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
-        if (warp < B) {  // warp b adds column b's partials of all CTAs: lane-strided, fixed tree
-            double sacc = 0.0;
-            for (int gi = lane; gi < G; gi += 32)
-                sacc += __ldcg(a.part + (int64_t)gi * kPartStride + 4 * (kArMaxSteps + 2) * kArMaxB + warp);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) sacc += __shfl_down_sync(0xffffffffu, sacc, o);
-            if (lane == 0) {
-                const double n = std::sqrt(sacc);
-                s_nrm[warp] = n > 0.0 ? 1.0 / n : 0.0;  // the inverse, used by every element
-                s_hcol[(j + 1) * B + warp] = cx<double>{n, 0.0};
-            }
+        if (!grid_exchange(a.bar, gen, B, a.wait_cycles, B, tid < B ? s_nrm[tid] : 0.0, s_sum, RedSum{})) { status = 1; break; }
+        if (tid < B) {
+            const double n = std::sqrt(s_sum[tid]);
+            const double inv = n > 0.0 ? 1.0 / n : 0.0;  // used by every element
+            const float ih = (float)inv;
+            s_nf[tid] = make_float2(ih, (float)(inv - (double)ih));
+            s_hcol[(j + 1) * B + tid] = cx<double>{n, 0.0};
         }
         __syncthreads();
         // v_{j+1} = w / |w| in float-float for the next steps; the FP64 copy only of the
         // tier-0 rows (elements below d2 * B), which the final combination x_0 = V_0 y reads,
         // so that the basis held in L2 is the float-float one alone
         for (int idx = tid; idx < nel; idx += bd) {
-            const cx<double> x = s_nrm[idx % B] * ff_join(W[e0 + idx]);  // zero norm: zeros
-            if (e0 + idx < (int64_t)d2 * B) a.V[(int64_t)(j + 1) * a.L + e0 + idx] = x;
-            W[e0 + idx] = ff_split(x);
+            float4 w = W[e0 + idx];
+            const float2 sc = s_nf[idx % B];  // zero norm: zeros
+            ff_scale(w.x, w.z, sc.x, sc.y);
+            ff_scale(w.y, w.w, sc.x, sc.y);
+            W[e0 + idx] = w;
+            if (e0 + idx < (int64_t)d2 * B) a.V[(int64_t)(j + 1) * a.L + e0 + idx] = ff_join(w);
         }
         // Hessenberg column j to global memory (CTA 0); its rows 0 .. j split into float-float
         // for the rotation chains (s_hf is free again: the Gram-Schmidt update has used it)
@@ -392,24 +394,17 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         float *s_redf = reinterpret_cast<float *>(s_red);
         if (lane == 0) s_redf[warp] = rmax;
         __syncthreads();
+        double mx = 0.0;
         if (warp == 0) {
-            float mx = lane < (bd >> 5) ? s_redf[lane] : 0.f;
+            float m = lane < (bd >> 5) ? s_redf[lane] : 0.f;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-            if (lane == 0) mypart[4 * (kArMaxSteps + 2) * kArMaxB + kArMaxB] = (double)mx;
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_down_sync(0xffffffffu, m, o));
+            mx = (double)m;
         }
         steps = j + 1;
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = 1; break; }
-        if (warp == 0) {  // largest residual estimate over all CTAs
-            float mx = 0.f;
-            for (int gi = lane; gi < G; gi += 32)
-                mx = fmaxf(mx, (float)__ldcg(a.part + (int64_t)gi * kPartStride + 4 * (kArMaxSteps + 2) * kArMaxB + kArMaxB));
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_down_sync(0xffffffffu, mx, o));
-            if (lane == 0) s_flag[1] = mx <= (float)(a.tol * a.tol);
-        }
-        __syncthreads();
-        if (s_flag[1]) { converged = 1; break; }
+        // largest residual estimate over all CTAs
+        if (!grid_exchange(a.bar, gen, B, a.wait_cycles, 1, mx, s_sum, RedMax{})) { status = 1; break; }
+        if ((float)s_sum[0] <= (float)(a.tol * a.tol)) { converged = 1; break; }
     }
     // the last basis vector in FP64 as a whole: the step-by-step continuation starts from it
     if (!status)
@@ -424,7 +419,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
 
 size_t arnoldi_smem(const DevView<double> &v, int hcap) {
     return (size_t)hcap * (sizeof(cx<double>) + sizeof(float4)) +
-           32 * kArMaxB * sizeof(double) + 2 * kArMaxB * sizeof(double) + (2 + kArMaxB) * sizeof(int) +
+           32 * kArMaxB * sizeof(double) + (2 * kArMaxB + kBarVals) * sizeof(double) + (2 + kArMaxB) * sizeof(int) +
            prog_smem_bytes<double>(v.pers_terms, v.pers_slots, v.pers_ados, v.d2) + 64;
 }
 
@@ -444,7 +439,7 @@ DevView<double> arnoldi_view(const heom_hier *h) {
 bool arnoldi_persistent_ok(const heom_hier *h, int64_t B, int max_steps) {
     // the resident term programs carry one parameter set's coefficients
     if (h->n_sets != 1 || h->has_caps) return false;
-    if (h->ar_ranges < 1 || B < 1 || B > kArMaxB || (32 % B) != 0 || (kArThreads % B) != 0) return false;
+    if (h->ar_ranges < 1 || h->ar_ranges > kBarMaxGrid || B < 1 || B > kArMaxB || (32 % B) != 0 || (kArThreads % B) != 0) return false;
     const int steps = std::min(max_steps, kArMaxSteps);
     return arnoldi_smem(arnoldi_view(h), (steps + 2) * (int)B) <= 200 * 1024;
 }
@@ -463,7 +458,7 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
     const int G = h->ar_ranges;
     const size_t part_bytes = (size_t)G * kPartStride * sizeof(double);
     const size_t hred_bytes = (size_t)2 * (kArMaxSteps + 2) * kArMaxB * sizeof(cx<double>);
-    heom_status st = ensure_ws(h->ws_pers, part_bytes + hred_bytes + 512);
+    heom_status st = ensure_ws(h->ws_pers, part_bytes + hred_bytes + 128 + grid_bar_bytes(G, (int)B));
     if (st != HEOM_OK) return st;
     char *base = (char *)h->ws_pers.p;
     ArnoldiArgs a{};
@@ -490,10 +485,11 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
     a.tol = tol;
     a.part = (double *)base;
     a.hred = (cx<double> *)(base + part_bytes);
-    a.bar = (GridBar *)(base + part_bytes + hred_bytes);
-    a.out = (int *)(base + part_bytes + hred_bytes + 256);
+    a.out = (int *)(base + part_bytes + hred_bytes);
+    a.bar = (GridBar *)(base + part_bytes + hred_bytes + 128);
     a.wait_cycles = wait_limit_cycles();
-    HEOM_CUDA(cudaMemsetAsync(a.bar, 0, 512, s));
+    HEOM_CUDA(cudaMemsetAsync(a.out, 0, 128, s));
+    HEOM_CUDA(grid_bar_reset(a.bar, G, (int)B, s));
     const size_t sm = arnoldi_smem(a.v, a.hcap);
     HEOM_CUDA(cudaFuncSetAttribute(k_arnoldi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     void *args[] = {&a};

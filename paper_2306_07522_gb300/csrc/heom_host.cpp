@@ -491,7 +491,7 @@ void free_all(heom_hier *h) {
                     &h->d_sdiag32, &h->d_tdval64, &h->d_floor64, &h->d_floor32, &h->ws,
                     &h->ws_small,
                     &h->d_t_ptr, &h->d_t_src, &h->d_t_val64, &h->d_t_val32, &h->d_cta_ado,
-                    &h->d_pers_ado, &h->d_ar_ado, &h->d_dense32, &h->ws_pers, &h->ws_res, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
+                    &h->d_pers_ado, &h->d_ar_ado, &h->d_dense32, &h->ws_pers, &h->ws_res, &h->ws_rhs, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
                     &h->d_op_rvalff, &h->d_op_cvalff, &h->d_svalff, &h->d_coefLff, &h->d_coefRff,
                     &h->d_rateff};
     for (DBuf *b : bufs) heom::dfree(*b);

@@ -3,9 +3,8 @@
 // Eq. HEOM in shared memory once (from the neighbour tables, never stored elsewhere) and
 // keeps them for every iteration. Vector updates touch only the CTA's own rows; the apply
 // reads neighbour rows of the whole vector after a grid-wide barrier. Dot products are
-// block sums written to per-block slots, added in a fixed order by every CTA after the next
-// barrier, so every CTA derives the same Krylov scalars and the same convergence decision
-// without any host round trip. Five grid barriers per iteration; the host reads the result
+// block sums exchanged by the barriers and added in a fixed order by every CTA, so every CTA
+// derives the same Krylov scalars and the same convergence decision without any host round trip. Five grid barriers per iteration; the host reads the result
 // once, at the end. In the FP64 solve the two applies of an iteration run in float-float (the
 // Krylov vectors, dot products and scalars stay FP64).
 #include <algorithm>
@@ -27,26 +26,30 @@ struct PersistOut {
 template <class R>
 struct PersistArgs {
     DevView<R> v;
-    const cx<R> *b;
+    const cx<R> *b;  // columns col of [rows][B]
     cx<R> *x;
+    int64_t B, col;
+    int set;         // the column's parameter set
     int x_zero;
     const cx<R> *shift;  // [1] or null
     R aug;
     int precond;
-    cx<R> *r, *rh, *p, *vv, *ph, *sh, *t;
+    cx<R> *r, *rh, *p, *vv, *ph, *sh, *t, *xw;
     float4 *phf, *shf;  // FP64 solve: float-float copies of ph and sh (the apply operands)
-    double *part;  // [kSlots][G][4]
     GridBar *bar;
     long long wait_cycles;  // bound of every grid-barrier wait (SM clock cycles)
     double tol;
     int max_iter, stall_iters;
+    int local;         // own rows of the vectors in shared memory, local_off bytes from its start
+    int local_off;
     PersistOut *out;
 };
 
 namespace {
 
 constexpr int kPersThreads = 512;
-constexpr int kSlots = 4;
+constexpr size_t kPersSmem = 224 * 1024;  // of 227 KB: the kernel has static arrays too
+constexpr int kPersVals = 3;  // numbers a barrier exchanges
 
 // Load written earlier in this launch by another CTA: through L2 (ld.global.cg), never the
 // non-coherent read-only path.
@@ -110,46 +113,30 @@ __device__ __forceinline__ cx<double> prog_apply_ff(const ProgSmem<double> &ps, 
     return cx<double>{(double)rh + (double)rl, (double)ih + (double)il};
 }
 
-// Grid-wide sum of NV doubles: block sums to part[slot][block], grid barrier, then in every
-// block warp k adds value k over all blocks (lane-strided loads through L2, then a fixed
-// shuffle tree; lane 0's result is used), so every block derives bit-identical totals. Only
-// the first nw warps hold values (the warps past the block's elements add nothing), so only
-// they run the FP64 shuffle trees.
+// Grid-wide sum of NV doubles: block sums, exchanged by the barrier. Only the first nw warps hold
+// values. One warp per value adds them (each FP64 addition of a warp occupies its sub-partition's pipe for
+// 64 cycles: a shuffle tree in every warp took more of them than everything else here).
 template <int NV>
-__device__ __forceinline__ bool grid_sum(double (&val)[NV], double *part, int slot, double *s_red,
-                                         double *s_tot, GridBar *bar, unsigned &gen, int nw,
-                                         long long limit) {
+__device__ __forceinline__ bool grid_sum(double (&val)[NV], double *s_red, double *s_tot, GridBar *bar, BarState &gen,
+                                         int nw, long long limit) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp < nw) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double x = val[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-            if (lane == 0) s_red[warp * 4 + k] = x;
-        }
+        for (int k = 0; k < NV; ++k) s_red[k * kPersThreads + threadIdx.x] = val[k];
     }
     __syncthreads();
-    if (threadIdx.x < NV) {
-        double x = 0.0;
-        for (int w = 0; w < nw; ++w) x += s_red[w * 4 + threadIdx.x];
-        part[((size_t)slot * gridDim.x + blockIdx.x) * 4 + threadIdx.x] = x;
-    }
-    if (!grid_barrier(bar, gen, limit)) return false;
-    if (warp < NV) {
-        // written by the other CTAs since this CTA last read the slot: through L2, so that
-        // no line of an earlier iteration cached in L1 is reused
-        double x = 0.0;
-        for (unsigned g = lane; g < gridDim.x; g += 32)
-            x += __ldcg(part + ((size_t)slot * gridDim.x + g) * 4 + warp);
+    double mine = 0.0;
+    if (warp < NV) {  // warp k adds value k: its warps' values lane by lane, then the lanes
+        for (int w = 0; w < nw; ++w) mine += s_red[warp * kPersThreads + w * 32 + lane];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if (lane == 0) s_tot[warp] = x;
+        for (int o = 16; o > 0; o >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, o);
+        if (lane == 0) s_tot[warp] = mine;
     }
     __syncthreads();
+    mine = threadIdx.x < NV ? s_tot[threadIdx.x] : 0.0;
+    if (!grid_exchange(bar, gen, kPersVals, limit, NV, mine, s_tot, RedSum{})) return false;
 #pragma unroll
     for (int k = 0; k < NV; ++k) val[k] = s_tot[k];
-    __syncthreads();
     return true;
 }
 
@@ -175,22 +162,22 @@ __device__ __forceinline__ bool finite_c(cx<double> a) { return isfinite(a.re) &
 
 template <class R>
 __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a) {
-    unsigned gen = 0;  // barriers this block has passed (the barrier starts zeroed)
+    BarState gen;
     // Krylov scalars are computed once per CTA by thread 0 and broadcast (every CTA derives
     // the same values from the same grid sums); redundant FP64 divisions in all 16 warps
     // would queue on the FP64 pipe
-    __shared__ double s_sc[8];
+    __shared__ double s_sc[9];
     const DevView<R> &v = a.v;
     const int d2 = v.d2;
     const int n0 = __ldg(v.pers_ado + blockIdx.x), n1 = __ldg(v.pers_ado + blockIdx.x + 1);
     extern __shared__ __align__(16) unsigned char smem[];
-    double *s_red = reinterpret_cast<double *>(smem);   // [32 warps][4]
-    double *s_tot = s_red + 32 * 4;                     // [4]
+    double *s_red = reinterpret_cast<double *>(smem);   // [kPersVals][threads]
+    double *s_tot = s_red + kPersVals * kPersThreads;   // [4]
     cx<R> *s_pinv = reinterpret_cast<cx<R> *>(s_tot + 4);
     ProgSmem<R> ps = prog_layout<R>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
                                     reinterpret_cast<unsigned char *>(s_pinv + (size_t)v.pers_ados * d2));
-    build_programs<R>(v, ps, n0, n1, a.aug, 0);
-    const cx<R> shift = a.shift ? a.shift[0] : cx<R>{R(0), R(0)};
+    build_programs<R>(v, ps, n0, n1, a.aug, a.set);
+    const cx<R> shift = a.shift ? a.shift[a.col] : cx<R>{R(0), R(0)};
     const int items = (n1 - n0) * d2;
     const int64_t row0 = (int64_t)n0 * d2;
     // warps that hold elements (thread t takes items t, t + blockDim.x, ...)
@@ -198,10 +185,19 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
         const int pp = it / d2, e = it - pp * d2;
         const int64_t n = n0 + pp;
-        s_pinv[it] = a.precond ? precond_inv(v, n, e, 0, damping_of(v, n, 0), shift)
+        s_pinv[it] = a.precond ? precond_inv(v, n, e, a.set, damping_of(v, n, a.set), shift)
                                : cx<R>{R(1), R(0)};
     }
     __syncthreads();
+
+    // The CTA's own rows of the vectors: in shared memory where they fit (a.local), so that the updates wait
+    // for no load from L2; the operands of the applies, which other CTAs read, are global too.
+    cx<R> *const loc = reinterpret_cast<cx<R> *>(smem + a.local_off);
+    const auto own = [&](int k, cx<R> *g) { return a.local ? loc + (size_t)k * v.pers_ados * d2 : g + row0; };
+    cx<R> *const r = own(0, a.r), *const rh = own(1, a.rh), *const p = own(2, a.p), *const vv = own(3, a.vv),
+                *const t = own(4, a.t), *const x = own(5, a.xw),
+                *const ph = sizeof(R) == 8 ? own(6, a.ph) : a.ph + row0,
+                *const sh = sizeof(R) == 8 ? own(7, a.sh) : a.sh + row0;
 
     // ---- r = b - A x, rh = r, p = v = 0
     double val2[2] = {0.0, 0.0};
@@ -209,12 +205,13 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
         const int64_t i = row0 + it;
         cx<R> ax{R(0), R(0)};
         if (!a.x_zero) ax = prog_apply(ps, it, a.x, shift);
-        const cx<R> bi = a.b[i];
+        x[it] = a.x_zero ? cx<R>{R(0), R(0)} : a.x[i];
+        const cx<R> bi = a.b[i * a.B + a.col];
         const cx<R> ri = bi - ax;
-        a.r[i] = ri;
-        a.rh[i] = ri;
-        a.p[i] = cx<R>{R(0), R(0)};
-        a.vv[i] = cx<R>{R(0), R(0)};
+        r[it] = ri;
+        rh[it] = ri;
+        p[it] = cx<R>{R(0), R(0)};
+        vv[it] = cx<R>{R(0), R(0)};
         val2[0] += (double)norm2(ri);
         val2[1] += (double)norm2(bi);
     }
@@ -232,44 +229,54 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
         for (int t = threadIdx.x; t < ps.item[items]; t += blockDim.x) cf[t] = ff_split(ps.coef[t]);
         __syncthreads();
     }
-    const bool started = grid_sum<2>(val2, a.part, 0, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles);
+    const bool started = grid_sum<2>(val2, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles);
+    // Thread 0 holds the scalars and takes the decisions, the same ones in every CTA (redundant FP64 operations of
+    // 16 warps queue on the FP64 pipe); s_st < 0: go on
+    __shared__ int s_st;
     double nr = val2[0];
-    const double bn = val2[1], tol2 = a.tol * a.tol;
+    const double bn = val2[1], stop2 = a.tol * a.tol * bn;
     cx<double> rho{nr, 0.0}, rho_old{1.0, 0.0}, alpha{1.0, 0.0}, omega{1.0, 0.0};
-    int status = !started ? HEOM_ETIMEOUT : (nr <= tol2 * bn) ? 0 : -1, it_done = 0;
     double best = nr, rhn = nr;  // rhn = ||rh||^2
-    int best_it = 0;
-    for (int iter = 1; status < 0 && iter <= a.max_iter; ++iter) {
-        // ---- restart when rh has become nearly orthogonal to r: rh = r, p = r;
-        // beta = (rho / rho_old)(alpha / omega)
-        if (threadIdx.x == 0) {
-            const bool rs = iter > 1 && norm2(rho) < kRestartTau2 * rhn * nr;
-            const cx<double> rr = rs ? cx<double>{nr, 0.0} : rho;
-            const cx<double> bb = cplx_div(rr, rho_old) * cplx_div(alpha, omega);
-            s_sc[0] = rs ? 1.0 : 0.0;
-            s_sc[1] = bb.re;
-            s_sc[2] = bb.im;
-        }
-        __syncthreads();
-        const bool restart = s_sc[0] != 0.0;
-        const cx<double> beta{s_sc[1], s_sc[2]};
-        if (restart) {
+    int best_it = 0, it_done = 0;
+    // restart when rh has become nearly orthogonal to r: rh = r, p = r; beta = (rho / rho_old)(alpha / omega)
+    const auto next_scalars = [&](int iter) {
+        const bool rs = iter > 1 && norm2(rho) < kRestartTau2 * rhn * nr;
+        if (rs) {
             rho = cx<double>{nr, 0.0};
             rhn = nr;
         }
+        const cx<double> bb = cplx_div(rho, rho_old) * cplx_div(alpha, omega), bo = bb * omega;
+        s_sc[0] = rs ? 1.0 : 0.0;
+        s_sc[1] = bb.re;
+        s_sc[2] = bb.im;
+        s_sc[3] = -bo.re;
+        s_sc[4] = -bo.im;
+    };
+    if (threadIdx.x == 0) {
+        s_st = !started ? HEOM_ETIMEOUT : nr <= stop2 ? 0 : -1;
+        if (s_st < 0) next_scalars(1);
+    }
+    __syncthreads();
+    int status = s_st;
+    for (int iter = 1; status < 0 && iter <= a.max_iter; ++iter) {
+        const bool restart = __double2hiint(s_sc[0]) != 0;
         // ---- p = r + beta (p - omega v), ph = P^-1 p
-        const cx<R> bt = cast<R>(beta), om = cast<R>(omega);
+        const cx<R> bt{R(s_sc[1]), R(s_sc[2])}, nbo{R(s_sc[3]), R(s_sc[4])};
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
             const int64_t i = row0 + it;
-            const cx<R> ri = a.r[i];
-            const cx<R> pi = restart ? ri : ri + bt * (a.p[i] - om * a.vv[i]);
-            if (restart) a.rh[i] = ri;
-            a.p[i] = pi;
+            const cx<R> ri = r[it];
+            cx<R> pi = ri;
+            if (!restart) {
+                fma_to(pi, bt, p[it]);
+                fma_to(pi, nbo, vv[it]);
+            }
+            if (restart) rh[it] = ri;
+            p[it] = pi;
             const cx<R> phi = pi * s_pinv[it];
-            a.ph[i] = phi;
+            ph[it] = phi;
             if constexpr (sizeof(R) == 8) a.phf[i] = ff_split(phi);
         }
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
+        if (!grid_barrier(a.bar, gen, kPersVals, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         // ---- v = A ph, (rh, v)
         double d1[2] = {0.0, 0.0};
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
@@ -277,32 +284,32 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
             cx<R> y;
             if constexpr (sizeof(R) == 8) y = prog_apply_ff(ps, it, a.phf);
             else y = prog_apply(ps, it, a.ph, shift);
-            a.vv[i] = y;
-            const cx<double> yd = cast<double>(y), wd = cast<double>(a.rh[i]);
-            d1[0] += wd.re * yd.re + wd.im * yd.im;
-            d1[1] += wd.re * yd.im - wd.im * yd.re;
+            vv[it] = y;
+            const cx<double> yd = cast<double>(y), wd = cast<double>(rh[it]);
+            d1[0] = fma(wd.re, yd.re, fma(wd.im, yd.im, d1[0]));
+            d1[1] = fma(wd.re, yd.im, fma(-wd.im, yd.re, d1[1]));
         }
-        if (!grid_sum<2>(d1, a.part, 1, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
-        const cx<double> rv{d1[0], d1[1]};
-        if (norm2(rv) == 0.0) { status = HEOM_EBREAKDOWN; it_done = iter; break; }
+        if (!grid_sum<2>(d1, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         if (threadIdx.x == 0) {
-            const cx<double> al0 = cplx_div(rho, rv);
-            s_sc[3] = al0.re;
-            s_sc[4] = al0.im;
+            const cx<double> rv{d1[0], d1[1]};
+            s_st = norm2(rv) == 0.0 ? HEOM_EBREAKDOWN : -1;
+            alpha = cplx_div(rho, rv);
+            s_sc[5] = alpha.re;
+            s_sc[6] = alpha.im;
         }
         __syncthreads();
-        alpha = cx<double>{s_sc[3], s_sc[4]};
-        // ---- s = r - alpha v (in r), sh = P^-1 s
-        const cx<R> al = cast<R>(alpha);
+        if (s_st >= 0) { status = s_st; it_done = iter; break; }
+        const cx<R> al{R(s_sc[5]), R(s_sc[6])}, nal{-al.re, -al.im};
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
             const int64_t i = row0 + it;
-            const cx<R> si = a.r[i] - al * a.vv[i];
-            a.r[i] = si;
+            cx<R> si = r[it];
+            fma_to(si, nal, vv[it]);
+            r[it] = si;
             const cx<R> shi = si * s_pinv[it];
-            a.sh[i] = shi;
+            sh[it] = shi;
             if constexpr (sizeof(R) == 8) a.shf[i] = ff_split(shi);
         }
-        if (!grid_barrier(a.bar, gen, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
+        if (!grid_barrier(a.bar, gen, kPersVals, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         // ---- t = A sh, (t, s), (t, t)
         double d2v[3] = {0.0, 0.0, 0.0};
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
@@ -310,61 +317,82 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
             cx<R> y;
             if constexpr (sizeof(R) == 8) y = prog_apply_ff(ps, it, a.shf);
             else y = prog_apply(ps, it, a.sh, shift);
-            a.t[i] = y;
-            const cx<double> yd = cast<double>(y), wd = cast<double>(a.r[i]);
-            d2v[0] += yd.re * wd.re + yd.im * wd.im;
-            d2v[1] += yd.re * wd.im - yd.im * wd.re;
-            d2v[2] += yd.re * yd.re + yd.im * yd.im;
+            t[it] = y;
+            const cx<double> yd = cast<double>(y), wd = cast<double>(r[it]);
+            d2v[0] = fma(yd.re, wd.re, fma(yd.im, wd.im, d2v[0]));
+            d2v[1] = fma(yd.re, wd.im, fma(-yd.im, wd.re, d2v[1]));
+            d2v[2] = fma(yd.re, yd.re, fma(yd.im, yd.im, d2v[2]));
         }
-        if (!grid_sum<3>(d2v, a.part, 2, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
+        if (!grid_sum<3>(d2v, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         if (threadIdx.x == 0) {
             const double it2 = d2v[2] == 0.0 ? 0.0 : nr_rcp(d2v[2]);
-            s_sc[5] = d2v[0] * it2;
-            s_sc[6] = d2v[1] * it2;
+            omega = cx<double>{d2v[0] * it2, d2v[1] * it2};
+            s_st = finite_c(omega) && finite_c(alpha) ? -1 : HEOM_EBREAKDOWN;
+            s_sc[7] = omega.re;
+            s_sc[8] = omega.im;
         }
         __syncthreads();
-        omega = cx<double>{s_sc[5], s_sc[6]};
-        if (!finite_c(omega) || !finite_c(alpha)) { status = HEOM_EBREAKDOWN; it_done = iter; break; }
+        if (s_st >= 0) { status = s_st; it_done = iter; break; }
         // ---- x += alpha ph + omega sh, r = s - omega t, (rh, r), ||r||^2
-        const cx<R> omr = cast<R>(omega);
+        const cx<R> omr{R(s_sc[7]), R(s_sc[8])}, nomr{-omr.re, -omr.im};
         double d3[3] = {0.0, 0.0, 0.0};
         for (int it = threadIdx.x; it < items; it += blockDim.x) {
             const int64_t i = row0 + it;
-            a.x[i] = a.x[i] + al * a.ph[i] + omr * a.sh[i];
-            const cx<R> ri = a.r[i] - omr * a.t[i];
-            a.r[i] = ri;
-            const cx<double> rd = cast<double>(ri), hd = cast<double>(a.rh[i]);
-            d3[0] += hd.re * rd.re + hd.im * rd.im;
-            d3[1] += hd.re * rd.im - hd.im * rd.re;
-            d3[2] += rd.re * rd.re + rd.im * rd.im;
+            cx<R> xi = x[it], ri = r[it];
+            fma_to(xi, al, ph[it]);
+            fma_to(xi, omr, sh[it]);
+            x[it] = xi;
+            fma_to(ri, nomr, t[it]);
+            r[it] = ri;
+            const cx<double> rd = cast<double>(ri), hd = cast<double>(rh[it]);
+            d3[0] = fma(hd.re, rd.re, fma(hd.im, rd.im, d3[0]));
+            d3[1] = fma(hd.re, rd.im, fma(-hd.im, rd.re, d3[1]));
+            d3[2] = fma(rd.re, rd.re, fma(rd.im, rd.im, d3[2]));
         }
-        if (!grid_sum<3>(d3, a.part, 3, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
-        rho_old = rho;
-        rho = cx<double>{d3[0], d3[1]};
-        nr = d3[2];
+        if (!grid_sum<3>(d3, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         it_done = iter;
-        if (!isfinite(nr)) { status = HEOM_EBREAKDOWN; break; }
-        if (nr <= tol2 * bn) { status = 0; break; }
-        // no new minimum for stall_iters iterations: stalled (or diverging); the result is
-        // usable if it still improved on the start. Single large transients (a near
-        // breakdown just after a restart) are allowed: the recursion often recovers.
-        if (nr < best) { best = nr; best_it = iter; }
-        else if (iter - best_it >= a.stall_iters) {
-            status = nr < bn ? HEOM_ENOCONV : HEOM_EBREAKDOWN;
-            break;
+        if (threadIdx.x == 0) {
+            rho_old = rho;
+            rho = cx<double>{d3[0], d3[1]};
+            nr = d3[2];
+            int next = -1;
+            if (!isfinite(nr)) next = HEOM_EBREAKDOWN;
+            else if (nr <= stop2) next = 0;
+            // no new minimum for stall_iters iterations: stalled (or diverging); the result is
+            // usable if it still improved on the start. Single large transients (a near
+            // breakdown just after a restart) are allowed: the recursion often recovers.
+            else if (nr < best) { best = nr; best_it = iter; }
+            else if (iter - best_it >= a.stall_iters) next = nr < bn ? HEOM_ENOCONV : HEOM_EBREAKDOWN;
+            s_st = next;
+            if (next < 0) next_scalars(iter + 1);
         }
+        __syncthreads();
+        status = s_st;
     }
+    for (int it = threadIdx.x; it < items; it += blockDim.x) a.x[(row0 + it) * a.B + a.col] = x[it];
     if (status < 0) status = HEOM_ENOCONV;
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = PersistOut{it_done, status, nr, bn};
 }
 
-template <class R> DevView<R> view_of_p(const heom_hier *h);
-template <> DevView<double> view_of_p<double>(const heom_hier *h) { return h->view64(); }
-template <> DevView<float> view_of_p<float>(const heom_hier *h) { return h->view32(); }
+// The view with ADO ranges balanced on terms + 128 d^2 per ADO: most of an iteration is FP64 vector work, which
+// follows a range's elements (balanced on terms alone the ranges of the tier-3 Anderson model hold 80 to 400
+// of them, and 400 cost 10,500 cycles in the first update alone).
+template <class R>
+DevView<R> view_of_p(const heom_hier *h) {
+    DevView<R> v;
+    if constexpr (sizeof(R) == 8) v = h->view64();
+    else v = h->view32();
+    v.pers_ado = (const int32_t *)h->d_ar_ado.p;
+    v.pers_ranges = h->ar_ranges;
+    v.pers_terms = h->ar_terms;
+    v.pers_slots = h->ar_slots;
+    v.pers_ados = h->ar_ados;
+    return v;
+}
 
 template <class R>
 size_t persist_smem(const DevView<R> &v) {
-    return 32 * 4 * sizeof(double) + 4 * sizeof(double) + (size_t)v.pers_ados * v.d2 * sizeof(cx<R>) +
+    return kPersVals * kPersThreads * sizeof(double) + 4 * sizeof(double) + (size_t)v.pers_ados * v.d2 * sizeof(cx<R>) +
            prog_smem_bytes<R>(v.pers_terms, v.pers_slots, v.pers_ados, v.d2) + 64;
 }
 
@@ -372,25 +400,26 @@ size_t persist_smem(const DevView<R> &v) {
 
 template <class R>
 bool persist_ok(const heom_hier *h) {
-    if (h->pers_ranges < 1 || h->n_sets != 1 || h->has_caps) return false;
+    if (h->ar_ranges < 1 || h->ar_ranges > kBarMaxGrid) return false;
     const DevView<R> v = view_of_p<R>(h);
     return persist_smem(v) <= 200 * 1024;
 }
 template bool persist_ok<double>(const heom_hier *);
 template bool persist_ok<float>(const heom_hier *);
 
-// One persistent BiCGStab solve of (M + shift + aug e00 tr) x = b for a single column.
+// One persistent BiCGStab solve of (M + shift + aug e00 tr) x = b for column col of b and x ([rows][B]; a starting
+// vector other than zero only with B = 1).
 template <class R>
-heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, bool x_zero,
+heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col, bool x_zero,
                                 const cx<R> *shift, R aug, double tol, int max_iter,
                                 int stall_iters, int *iters, int *status, double *rel_res,
                                 cudaStream_t s) {
     const DevView<R> v = view_of_p<R>(h);
     const int64_t rows = h->N * h->d2;
-    const int G = h->pers_ranges;
+    const int G = h->ar_ranges;
     const size_t vec = ((size_t)rows * sizeof(cx<R>) + 255) & ~size_t(255);
     const size_t fvec = sizeof(R) == 8 ? (((size_t)rows * sizeof(float4) + 255) & ~size_t(255)) : 0;
-    const size_t bytes = 7 * vec + 2 * fvec + (size_t)kSlots * G * 4 * sizeof(double) + 512;
+    const size_t bytes = 8 * vec + 2 * fvec + 128 + grid_bar_bytes(G, kPersVals);
     heom_status st = ensure_ws(h->ws_pers, bytes);
     if (st != HEOM_OK) return st;
     char *base = (char *)h->ws_pers.p;
@@ -398,26 +427,33 @@ heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, bool x_z
     a.v = v;
     a.b = b;
     a.x = x;
-    a.x_zero = x_zero ? 1 : 0;
+    a.B = B;
+    a.col = col;
+    a.set = (int)(col / (B / h->n_sets));
+    a.x_zero = x_zero || B > 1 ? 1 : 0;
     a.shift = shift;
     a.aug = aug;
     a.precond = 1;
-    cx<R> **vecs[7] = {&a.r, &a.rh, &a.p, &a.vv, &a.ph, &a.sh, &a.t};
-    for (int i = 0; i < 7; ++i) *vecs[i] = (cx<R> *)(base + i * vec);
+    cx<R> **vecs[8] = {&a.r, &a.rh, &a.p, &a.vv, &a.ph, &a.sh, &a.t, &a.xw};
+    for (int i = 0; i < 8; ++i) *vecs[i] = (cx<R> *)(base + i * vec);
     if (fvec) {
-        a.phf = (float4 *)(base + 7 * vec);
-        a.shf = (float4 *)(base + 7 * vec + fvec);
+        a.phf = (float4 *)(base + 8 * vec);
+        a.shf = (float4 *)(base + 8 * vec + fvec);
     }
-    a.part = (double *)(base + 7 * vec + 2 * fvec);
-    a.out = (PersistOut *)((char *)a.part + (size_t)kSlots * G * 4 * sizeof(double));
+    a.out = (PersistOut *)(base + 8 * vec + 2 * fvec);
     a.bar = (GridBar *)((char *)a.out + 128);
-    HEOM_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(GridBar), s));
+    HEOM_CUDA(grid_bar_reset(a.bar, G, kPersVals, s));
     a.tol = tol;
     a.max_iter = max_iter;
     a.stall_iters = stall_iters;
     a.wait_cycles = wait_limit_cycles();
-    if (x_zero) HEOM_CUDA(cudaMemsetAsync(x, 0, rows * sizeof(cx<R>), s));
-    const size_t sm = persist_smem(v);
+    size_t sm = persist_smem(v);
+    const size_t loc = (size_t)8 * v.pers_ados * v.d2 * sizeof(cx<R>), off = (sm + 15) & ~size_t(15);
+    if (off + loc <= kPersSmem) {
+        a.local = 1;
+        a.local_off = (int)off;
+        sm = off + loc;
+    }
     HEOM_CUDA(cudaFuncSetAttribute(k_persist_bicg<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     void *args[] = {&a};
     {
@@ -440,10 +476,10 @@ heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, bool x_z
     return HEOM_OK;
 }
 
-template heom_status bicgstab_persistent<double>(heom_hier *, const cx<double> *, cx<double> *, bool,
+template heom_status bicgstab_persistent<double>(heom_hier *, const cx<double> *, cx<double> *, int64_t, int64_t, bool,
                                                  const cx<double> *, double, double, int, int, int *,
                                                  int *, double *, cudaStream_t);
-template heom_status bicgstab_persistent<float>(heom_hier *, const cx<float> *, cx<float> *, bool,
+template heom_status bicgstab_persistent<float>(heom_hier *, const cx<float> *, cx<float> *, int64_t, int64_t, bool,
                                                 const cx<float> *, float, double, int, int, int *,
                                                 int *, double *, cudaStream_t);
 

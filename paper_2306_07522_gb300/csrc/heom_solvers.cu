@@ -1055,14 +1055,16 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
         const double inner_tol = plain ? std::max(0.5 * tol / worst, 1e-10) : 1e-4;
         inner_max = std::min(inner_max, plain ? kInnerCap64 : kInnerCap);
         SolveOut o;
-        if (B == 1 && !strict && persist_ok<RI>(h)) {
-            // one column: the whole BiCGStab solve is one cooperative launch
-            o.iters.assign(1, 0);
-            o.status.assign(1, HEOM_OK);
-            o.res.assign(1, 0.0);
-            stt = bicgstab_persistent<RI>(h, rhs, dv, true, shift64 ? shift_in : nullptr, (RI)aug,
-                                          inner_tol, inner_max, kStallIters, &o.iters[0],
-                                          &o.status[0], &o.res[0], s);
+        if (B <= kPersistMaxB && !strict && persist_ok<RI>(h)) {
+            // few columns: the whole BiCGStab solve of a column is one cooperative launch
+            o.iters.assign(B, 0);
+            o.status.assign(B, HEOM_OK);
+            o.res.assign(B, 0.0);
+            for (int64_t b = 0; b < B && stt == HEOM_OK; ++b)
+                if (active[b])
+                    stt = bicgstab_persistent<RI>(h, rhs, dv, B, b, true, shift64 ? shift_in : nullptr, (RI)aug,
+                                                  inner_tol, std::min(inner_max, std::max(1, max_iter - res.iters[b])),
+                                                  kStallIters, &o.iters[b], &o.status[b], &o.res[b], s);
         } else {
             stt = bicgstab<RI>(h, rhs, dv, B, shift64 ? shift_in : nullptr, (RI)aug, inner_tol,
                                inner_max, active, w, st, d_map, d_lmap, shift_c, d_reg, reg_cap, o, s);
@@ -1311,6 +1313,9 @@ extern "C" heom_status heom_evolve_td(heom_hier *h, void *ados, int64_t batch, d
                               (cx<float> *)rho_traj, f, (cudaStream_t)s);
 }
 
+// a buffer of the hierarchy's own, allocated anew only when it is too small
+static heom_status keep_buf(DBuf &b, size_t bytes) { return b.p && b.bytes >= bytes ? HEOM_OK : dalloc(b, bytes); }
+
 static void fill_stats(heom_solve_stats *stats, const Solve &r, int64_t off, int64_t n) {
     if (!stats) return;
     for (int64_t b = 0; b < n; ++b) {
@@ -1334,11 +1339,11 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
     HEOM_DEVICE(h->device);
     cudaStream_t st = (cudaStream_t)s;
     const int64_t rows = h->N * h->d2, L = rows * batch;
-    // the right-hand side e_(0,(0,0)) lives behind the solver workspace in ws_small's sibling
-    DBuf bbuf;
-    heom_status stt = dalloc(bbuf, L * sizeof(cx<double>));
+    // the right-hand side e_(0,(0,0)), the columns' factors and norms: a workspace of their own, kept like
+    // the solvers' (a cudaMalloc and a cudaFree, which waits for the device, cost as much as an iteration or more)
+    heom_status stt = keep_buf(h->ws_rhs, (size_t)L * sizeof(cx<double>) + batch * (sizeof(cx<double>) + 2 * sizeof(double)));
     if (stt != HEOM_OK) return stt;
-    cx<double> *b64 = (cx<double> *)bbuf.p, *x = (cx<double> *)x_out;
+    cx<double> *b64 = (cx<double> *)h->ws_rhs.p, *x = (cx<double> *)x_out;
     { Prof pr(HEOM_KC_OTHER, st, (double)L);
       k_set_e00<double><<<flat_blocks(L), 256, 0, st>>>(L, b64, batch); }
     if (x0) {
@@ -1347,7 +1352,6 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
     // drive ||b - A x|| below tol/10: then ||M x|| / ||x|| <= tol for ||x|| >= 0.2
     Solve r;
     stt = solve_system(h, b64, x, batch, nullptr, 1.0, x0 == nullptr, 0.1 * tol, max_iter, prec, r, st);
-    dfree(bbuf);
     if (stt != HEOM_OK) return stt;
     // normalise Tr rho_sys = 1 and measure r_ss = ||M x|| / ||x||
     std::vector<cx<double>> top((size_t)h->d2 * batch);
@@ -1359,10 +1363,7 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
         for (int i = 0; i < h->d; ++i) tr = tr + top[(size_t)(i * h->d + i) * batch + b];
         fac[b] = (tr.re == 0.0 && tr.im == 0.0) ? cx<double>{1.0, 0.0} : cdiv(cx<double>{1.0, 0.0}, tr);
     }
-    DBuf tmp;
-    stt = dalloc(tmp, batch * (sizeof(cx<double>) + 2 * sizeof(double)));
-    if (stt != HEOM_OK) return stt;
-    cx<double> *dfac = (cx<double> *)tmp.p;
+    cx<double> *dfac = b64 + L;
     double *norms = (double *)(dfac + batch);
     HEOM_CUDA(memcpy_counted(dfac, fac.data(), batch * sizeof(cx<double>), cudaMemcpyHostToDevice, st));
     { Prof pr(HEOM_KC_OTHER, st, (double)L);
@@ -1384,7 +1385,6 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
     std::vector<double> hn(2 * batch);
     HEOM_CUDA(memcpy_counted(hn.data(), norms, hn.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
     HEOM_CUDA(cudaStreamSynchronize(st));
-    dfree(tmp);
     heom_status ret = HEOM_OK;
     for (int64_t b = 0; b < batch; ++b) {
         // r_ss = ||M x|| / ||x||; a zero iterate (a solve that never started) has none
@@ -1408,10 +1408,9 @@ static heom_status spectrum_shifted(heom_hier *odd, const void *ss_ados, const h
     const int d = odd->d;
     const int64_t ns = odd->n_sets, B = 2 * ns;
     const int64_t rows = odd->N * odd->d2, L = rows * B;
-    DBuf buf;
-    heom_status stt = dalloc(buf, L * sizeof(cx<double>) + 2 * d * d * sizeof(cx<double>));
+    heom_status stt = keep_buf(odd->ws_rhs, (size_t)(L + 2 * d * d) * sizeof(cx<double>));
     if (stt != HEOM_OK) return stt;
-    cx<double> *b64 = (cx<double> *)buf.p, *ops = b64 + L;
+    cx<double> *b64 = (cx<double> *)odd->ws_rhs.p, *ops = b64 + L;
     std::vector<cx<double>> hops(2 * d * d);
     for (int r = 0; r < d; ++r)
         for (int c = 0; c < d; ++c) {
@@ -1437,7 +1436,6 @@ static heom_status spectrum_shifted(heom_hier *odd, const void *ss_ados, const h
     int steps = 0;
     stt = shifted_gmres(odd, b64, B, shift, col_of, 0.5 * tol, std::max(1, std::min(max_iter, 2000)),
                         x0, res, &steps, st);
-    dfree(buf);
     if (stt == HEOM_ETIMEOUT) {  // a device wait ran out: no solution, every frequency flagged
         for (int64_t k = 0; k < ns * n_omega; ++k) A_out[k] = NAN;
         if (stats)

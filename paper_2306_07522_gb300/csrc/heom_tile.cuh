@@ -83,7 +83,7 @@ __device__ inline ProgSmem<R> prog_layout(int terms, int slots, int ados, int d2
     s.off = s.src + terms;                       // [triples]
     s.item = s.off + slots;                      // [items] program start of (p, e)
     s.nb = s.item + items;                       // [pairs]
-    s.op = s.nb + pairs;                         // [pairs] op slot / -1 H / -2 trace / -3 damping
+    s.op = s.nb + pairs;                         // [pairs] op slot / -1 H / -2 trace / -3 damping / -4 none
     s.pb = s.op + pairs;                         // [ados + 2] first pair of ADO p
     s.scan = s.pb + ados + 2;                    // [<= 1024 threads] scan scratch
     return s;
@@ -165,6 +165,8 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
             nb = 0;
             cl = cx<R>{aug, R(0)};
         }
+        // beyond the set's truncation an ADO and its couplings are not in the hierarchy
+        if (v.set_cap && op >= -2 && (beyond_cap(v, n, set) || beyond_cap(v, nb, set))) op = -4;
         s_nb[q] = nb;
         s_op[q] = op;
         s_cl[q] = cl;
@@ -182,6 +184,7 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
         if (op >= 0) len = __ldg(v.t_ptr + op * d2 + e + 1) - __ldg(v.t_ptr + op * d2 + e);
         else if (op == -1) len = __ldg(v.s_ptr + e + 1) - __ldg(v.s_ptr + e);
         else if (op == -3) len = 1;
+        else if (op == -4) len = 0;
         else len = (e == 0 && n0 + p == 0 && aug != R(0)) ? d : 0;
         s_off[z] = len;
     }
@@ -249,7 +252,7 @@ __device__ void build_programs(const DevView<R> &v, ProgSmem<R> &ps, int n0, int
             const cx<R> dmp = damping_of(v, (int64_t)(n0 + p), set);
             s_src[pos] = (n0 + p) * d2 + e;
             s_coef[pos] = cx<R>{-dmp.re, -dmp.im};
-        } else if (e == 0 && n0 + p == 0 && aug != R(0)) {
+        } else if (op == -2 && e == 0 && n0 + p == 0 && aug != R(0)) {
             for (int i = 0; i < d; ++i, ++pos) {
                 s_src[pos] = i * d + i;
                 s_coef[pos] = s_cl[q];
