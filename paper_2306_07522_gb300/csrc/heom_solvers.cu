@@ -93,6 +93,7 @@ struct ColRegion {
     int32_t ado0, ado1, col0, acols;
 };
 constexpr int kRegThreads = 256;
+constexpr int kRegPieces = 32;  // pieces the regions are cut into, about
 
 #define REGION_PROLOGUE                                                                           \
     const ColRegion rg = regions[blockIdx.y];                                                     \
@@ -681,6 +682,34 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
             c0 += w;
         }
         if (regs.empty()) regs.push_back(ColRegion{0, 0, 0, 1});
+        // Pieces of about equal work, so that the blocks, dealt evenly over them, have equal work too: an
+        // ADO counts its neighbour entries and four for its own rows
+        {
+            const auto upto = [&](int64_t n) { return (double)h->row_ptr[(size_t)n] + 4.0 * (double)n; };
+            double all = 0.0;
+            for (const ColRegion &r : regs) all += (upto(r.ado1) - upto(r.ado0)) * r.acols;
+            std::vector<ColRegion> cut;
+            for (const ColRegion &r : regs) {
+                const double w0 = upto(r.ado0), w = upto(r.ado1) - w0;
+                const int k = std::max(1, (int)std::lround(w * r.acols / std::max(all, 1.0) * kRegPieces));
+                int32_t at = r.ado0;
+                for (int i = 1; i <= k; ++i) {
+                    int32_t to = r.ado1;
+                    if (i < k) {
+                        int32_t lo = at, hi = r.ado1;
+                        while (lo < hi) {
+                            const int32_t mid = lo + (hi - lo) / 2;
+                            if (upto(mid) - w0 < w * i / k) lo = mid + 1;
+                            else hi = mid;
+                        }
+                        to = lo;
+                    }
+                    if (to > at || r.ado1 == r.ado0) cut.push_back(ColRegion{at, to, r.col0, r.acols});
+                    at = to;
+                }
+            }
+            regs.swap(cut);
+        }
         if ((int64_t)regs.size() > reg_cap) {
             set_error("BiCGStab: region table overflow");
             return HEOM_EINVAL;
@@ -695,9 +724,10 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
             }
             return dim3((unsigned)std::min(need, std::max<int64_t>(1, most / nr)), (unsigned)nr, 1);
         };
+        // vector updates: one wave -- a block's start-up forms its columns' scalars with FP64 divisions, 2 to 3 us
         ga = grid(lp.ne, 152 * 12);
-        gd = grid(1, 152 * 12);
-        gv = grid(1, 152 * 64);
+        gd = grid(1, 152 * 8);
+        gv = grid(1, 152 * 8);
         gi = make_geom(rows, Bc, std::max<int64_t>(1, 4096 / ((Bc + 31) / 32)));
         return HEOM_OK;
     };
@@ -947,8 +977,8 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
     heom_status stt = ensure_ws(h->ws, bytes);
     if (stt != HEOM_OK) return stt;
     // regions of the working layout: per group of columns at most one more than the different
-    // depths of its sets
-    const int64_t reg_cap = (B + 31) / 32 + std::min<int64_t>(B, h->n_sets) + 1;
+    // depths of its sets, cut into about kRegPieces pieces (rounding adds at most one per region)
+    const int64_t reg_cap = 2 * ((B + 31) / 32 + std::min<int64_t>(B, h->n_sets) + 1) + kRegPieces;
     stt = ensure_ws(h->ws_small, align_up(2 * B * sizeof(ColState)) + 3 * align_up(B * sizeof(int)) +
                                      align_up(reg_cap * sizeof(ColRegion)));
     if (stt != HEOM_OK) return stt;
