@@ -30,6 +30,7 @@ namespace heom {
 namespace {
 
 constexpr int kArThreads = 512;
+constexpr size_t kArSmem = 224 * 1024;  // of 227 KB: the kernel has static arrays too
 constexpr int kArMaxSteps = 192;  // Hessenberg column held in shared memory
 constexpr int kArMaxB = 8;        // columns (B divides 32)
 constexpr double kArKeep2 = 0.05 * 0.05;
@@ -38,6 +39,9 @@ struct ArnoldiArgs {
     DevView<double> v;
     int64_t B, L, S;
     int mmax, max_steps;
+    int w_off;    // shared memory from this byte on holds the own rows of w (-1: they stay in global memory)
+    int rot_off;  // and from this one on the split rotations 0 .. rcap - 1 of the CTA's nsh shifts
+    int rcap, nsh;
     int hcap;  // (max_steps + 2) * B: entries of the shared-memory Hessenberg column
     float4 *Vf;
     cx<double> *V, *Hb;
@@ -63,33 +67,29 @@ static_assert(kArMaxB <= kBarVals, "the norms travel with a barrier");
 __device__ __forceinline__ float4 ld_l2_f4(const float4 *p) { return __ldcg(p); }
 
 
-// Partial dot products conj(V_i) w over the CTA's own elements for i < nv (w is V_nv-1 +1
-// slot when self is wanted), into this CTA's slot of part: warp per i, lanes over own
+// Partial dot products conj(V_i) w over the CTA's own elements (Wo: the own rows of w) for i < nv, into this CTA's slot of part: warp per i, lanes over own
 // elements (element = row * B + b; B divides 32, so a lane always sees the same column).
-__device__ void own_dots(const ArnoldiArgs &a, const float4 *W, int nv, int64_t e0, int nel,
+__device__ void own_dots(const ArnoldiArgs &a, const float4 *Wo, int nv, int64_t e0, int nel,
                          double *mypart) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int B = (int)a.B;
     for (int i = warp; i < nv; i += nw) {
         const float4 *Vi = a.Vf + (int64_t)i * a.L + e0;
-        const float4 *Wo = W + e0;
         // float-float accumulation over the lane's elements, one conversion to FP64 at the end
         // (GB300's FP64 pipe is the scarce one)
         float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
         int t = lane;
-        for (; t + 96 < nel; t += 128) {  // four elements per lane, eight loads in flight
-            float4 x[4], y[4];
+        for (; t + 224 < nel; t += 256) {  // eight elements per lane, their loads in flight together
+            float4 x[8];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                x[u] = Vi[t + 32 * u];
-                y[u] = Wo[t + 32 * u];
-            }
+            for (int u = 0; u < 8; ++u) x[u] = Vi[t + 32 * u];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                ff_mac(rh, rl, x[u].x, x[u].z, y[u].x, y[u].z);
-                ff_mac(rh, rl, x[u].y, x[u].w, y[u].y, y[u].w);
-                ff_mac(ih, il, x[u].x, x[u].z, y[u].y, y[u].w);
-                ff_mac(ih, il, -x[u].y, -x[u].w, y[u].x, y[u].z);
+            for (int u = 0; u < 8; ++u) {
+                const float4 y = Wo[t + 32 * u];
+                ff_mac(rh, rl, x[u].x, x[u].z, y.x, y.z);
+                ff_mac(rh, rl, x[u].y, x[u].w, y.y, y.w);
+                ff_mac(ih, il, x[u].x, x[u].z, y.y, y.w);
+                ff_mac(ih, il, -x[u].y, -x[u].w, y.x, y.z);
             }
         }
         for (; t < nel; t += 32) {
@@ -113,6 +113,26 @@ __device__ void own_dots(const ArnoldiArgs &a, const float4 *W, int nv, int64_t 
             mypart[2 * (i * B + lane)] = (double)rh + (double)rl;
             mypart[2 * (i * B + lane) + 1] = (double)ih + (double)il;
         }
+    }
+}
+
+// |w|^2 per column over the CTA's own elements, as own_dots leaves it (one warp)
+__device__ void own_norm(int B, const float4 *Wo, int nel, double *out) {
+    const int lane = threadIdx.x & 31;
+    float h = 0.f, l = 0.f;
+    for (int t = lane; t < nel; t += 32) {
+        const float4 y = Wo[t];
+        ff_mac(h, l, y.x, y.z, y.x, y.z);
+        ff_mac(h, l, y.y, y.w, y.y, y.w);
+    }
+    ff_norm(h, l);
+    for (int o = 16; o >= B; o >>= 1) {
+        const float a0 = __shfl_down_sync(0xffffffffu, h, o), a1 = __shfl_down_sync(0xffffffffu, l, o);
+        ff_add(h, l, a0, a1);
+    }
+    if (lane < B) {
+        out[2 * lane] = (double)h + (double)l;
+        out[2 * lane + 1] = 0.0;
     }
 }
 
@@ -158,6 +178,9 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
     ProgSmem<double> ps = prog_layout<double>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
                                               reinterpret_cast<unsigned char *>(s_flag + 4 + kArMaxB));
     __shared__ float2 s_nf[kArMaxB];  // 1 / |w| in float-float
+    float4 *const s_w = a.w_off >= 0 ? reinterpret_cast<float4 *>(smem + a.w_off) : nullptr;
+    float4 *const s_rs = reinterpret_cast<float4 *>(smem + a.rot_off);
+    float2 *const s_rc = reinterpret_cast<float2 *>(s_rs + (size_t)a.rcap * a.nsh);
     if (threadIdx.x < B) {
         const double bt = a.beta[threadIdx.x];
         s_ib2[threadIdx.x] = bt > 0.0 ? 1.0 / (bt * bt) : 0.0;
@@ -180,6 +203,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
     for (int j = 0; j < a.max_steps; ++j) {
         const float4 *Vj = a.Vf + (int64_t)j * a.L;
         float4 *W = a.Vf + (int64_t)(j + 1) * a.L;
+        float4 *wl = s_w ? s_w : W + e0;  // the own rows of w
         // ---- 1. w = M v_j on the own elements
         for (int idx = tid; idx < nel; idx += bd) {
             const int it = idx / B, b = idx - it * B;
@@ -198,11 +222,12 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
             }
             ff_norm(rh, rl);
             ff_norm(ih, il);
-            W[e0 + idx] = make_float4(rh, ih, rl, il);
+            wl[idx] = make_float4(rh, ih, rl, il);
         }
         __syncthreads();
         // ---- 2. Gram-Schmidt pass 1 (+ |w|^2 as the dot of w with itself, slot j + 1)
-        own_dots(a, W, j + 2, e0, nel, mypart);
+        own_dots(a, wl, j + 1, e0, nel, mypart);
+        if (warp == 0) own_norm(B, wl, nel, mypart + 2 * (j + 1) * B);
         if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
         slice_reduce(a, 0, j + 2);
         if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
@@ -234,7 +259,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         for (int b = 0; b < B; ++b) need2 |= s_flag[2 + b];
         for (int pass = 0; pass < 1 + need2; ++pass) {
             if (pass == 1) {
-                own_dots(a, W, j + 1, e0, nel, mypart + 2 * (kArMaxSteps + 2) * kArMaxB);
+                own_dots(a, wl, j + 1, e0, nel, mypart + 2 * (kArMaxSteps + 2) * kArMaxB);
                 if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
                 slice_reduce(a, 1, j + 1);
                 if (!grid_barrier(a.bar, gen, B, a.wait_cycles)) { status = 1; break; }
@@ -250,7 +275,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
             // w -= sum_{i <= j} v_i h_i on the own elements
             for (int idx = tid; idx < nel; idx += bd) {
                 const int b = idx % B;
-                const float4 w0 = W[e0 + idx];
+                const float4 w0 = wl[idx];
                 float rh = w0.x, rl = w0.z, ih = w0.y, il = w0.w;
                 for (int i0 = 0; i0 <= j; i0 += 8) {  // 8 basis loads in flight
                     float4 vv[8];
@@ -269,7 +294,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
                 }
                 ff_norm(rh, rl);
                 ff_norm(ih, il);
-                W[e0 + idx] = make_float4(rh, ih, rl, il);
+                wl[idx] = make_float4(rh, ih, rl, il);
             }
             __syncthreads();
         }
@@ -280,7 +305,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
             // a thread's elements all have column tid % B when B | bd
             float ah = 0.f, al = 0.f;
             for (int idx = tid; idx < nel; idx += bd) {
-                const float4 x = W[e0 + idx];
+                const float4 x = wl[idx];
                 ff_mac(ah, al, x.x, x.z, x.x, x.z);
                 ff_mac(ah, al, x.y, x.w, x.y, x.w);
             }
@@ -312,7 +337,7 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         // tier-0 rows (elements below d2 * B), which the final combination x_0 = V_0 y reads,
         // so that the basis held in L2 is the float-float one alone
         for (int idx = tid; idx < nel; idx += bd) {
-            float4 w = W[e0 + idx];
+            float4 w = wl[idx];
             const float2 sc = s_nf[idx % B];  // zero norm: zeros
             ff_scale(w.x, w.z, sc.x, sc.y);
             ff_scale(w.y, w.w, sc.x, sc.y);
@@ -347,7 +372,18 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
                 ff_add(h.x, h.z, shf.x, shf.z);
                 ff_add(h.y, h.w, shf.y, shf.w);
             }
-            for (int i0 = 0; i0 < j; i0 += 8) {  // the rotations, 8 loads in flight
+            const auto step = [&](int i, float2 cr, float4 sr) {
+                float4 hi1 = s_hf[(i + 1) * B + b];
+                if (i + 1 == j) {
+                    ff_add(hi1.x, hi1.z, shf.x, shf.z);
+                    ff_add(hi1.y, hi1.w, shf.y, shf.w);
+                }
+                h = ff_rot_step(cr, sr, hi1, h);
+            };
+            const int in_smem = min(j, a.rcap);
+#pragma unroll 4
+            for (int i = 0; i < in_smem; ++i) step(i, s_rc[i * a.nsh + tid], s_rs[i * a.nsh + tid]);
+            for (int i0 = in_smem; i0 < j; i0 += 8) {  // the others, 8 loads in flight
                 float2 cr[8];
                 float4 sr[8];
 #pragma unroll
@@ -358,14 +394,8 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
-                    const int i = i0 + u;
-                    if (i >= j) break;
-                    float4 hi1 = s_hf[(i + 1) * B + b];
-                    if (i + 1 == j) {
-                        ff_add(hi1.x, hi1.z, shf.x, shf.z);
-                        ff_add(hi1.y, hi1.w, shf.y, shf.w);
-                    }
-                    h = ff_rot_step(cr[u], sr[u], hi1, h);
+                    if (i0 + u >= j) break;
+                    step(i0 + u, cr[u], sr[u]);
                 }
             }
             const cx<double> hj = ff_join(h);
@@ -377,8 +407,15 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
             rs[j] = sn;
             {
                 const float ch = __double2float_rn(c);
-                rcf[j] = make_float2(ch, __double2float_rn(c - (double)ch));
-                rsf[j] = ff_split(sn);
+                const float2 cf = make_float2(ch, __double2float_rn(c - (double)ch));
+                const float4 sf = ff_split(sn);
+                if (j < a.rcap) {
+                    s_rc[j * a.nsh + tid] = cf;
+                    s_rs[j * a.nsh + tid] = sf;
+                } else {
+                    rcf[j] = cf;
+                    rsf[j] = sf;
+                }
             }
             a.rdiag[k * a.mmax + j] = r;
             const cx<double> gj = gk[j];
@@ -490,7 +527,24 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
     a.wait_cycles = wait_limit_cycles();
     HEOM_CUDA(cudaMemsetAsync(a.out, 0, 128, s));
     HEOM_CUDA(grid_bar_reset(a.bar, G, (int)B, s));
-    const size_t sm = arnoldi_smem(a.v, a.hcap);
+    // on top, where they fit: the own rows of w (the dots read them for every basis vector) and as many of the
+    // split rotations as there is room for (a shift's chain walks all of them in every step: from L2 24,000 of
+    // the 123,000 cycles of a step at 55 basis vectors, on one warp while the others wait; 1,024 frequencies of 2,325
+    // ADOs: 8.28 -> 8.17 ms)
+    size_t sm = (arnoldi_smem(a.v, a.hcap) + 15) & ~size_t(15);
+    const size_t wb = (size_t)a.v.pers_ados * a.v.d2 * B * sizeof(float4);
+    a.w_off = -1;
+    if (sm + wb <= kArSmem) {
+        a.w_off = (int)sm;
+        sm += wb;
+    }
+    a.rot_off = (int)sm;
+    a.nsh = (int)((S + G - 1) / G);
+    a.rcap = 0;
+    if (a.nsh <= kArThreads && sm < kArSmem) {
+        a.rcap = (int)std::min<size_t>((size_t)a.max_steps, (kArSmem - sm) / ((size_t)a.nsh * (sizeof(float4) + sizeof(float2))));
+        sm += (size_t)a.rcap * a.nsh * (sizeof(float4) + sizeof(float2));
+    }
     HEOM_CUDA(cudaFuncSetAttribute(k_arnoldi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     void *args[] = {&a};
     {

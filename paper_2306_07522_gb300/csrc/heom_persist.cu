@@ -89,9 +89,9 @@ __device__ __forceinline__ cx<R> prog_apply(const ProgSmem<R> &ps, int it, const
 // already folded into each item's first term) and a float-float copy of X, so that the
 // multiply-adds run on the FP32 pipe instead of GB300's 1/64-rate FP64 pipe; about 48
 // significant bits per product and sum.
-__device__ __forceinline__ cx<double> prog_apply_ff(const ProgSmem<double> &ps, int it, const float4 *X) {
+// Terms from j0 on, up to j1, of an item; unevaluated {re hi, im hi, re lo, im lo}.
+__device__ __forceinline__ float4 prog_apply_ff(const ProgSmem<double> &ps, int j0, int j1, const float4 *X) {
     const float4 *coef = reinterpret_cast<const float4 *>(ps.coef);
-    const int j0 = ps.item[it], j1 = ps.item[it + 1];
     float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
     for (int jj = j0; jj < j1; jj += 8) {
         float4 c[8], x[8];
@@ -110,7 +110,40 @@ __device__ __forceinline__ cx<double> prog_apply_ff(const ProgSmem<double> &ps, 
             ff_mac(ih, il, c[u].y, c[u].w, x[u].x, x[u].z);
         }
     }
-    return cx<double>{(double)rh + (double)rl, (double)ih + (double)il};
+    return make_float4(rh, ih, rl, il);
+}
+
+// body(it, y) for every item of the block with y = its apply to X, the FP64 solve's in float-float. Where the block
+// has two threads per item, each takes half of its terms (an item of a low tier has 25 and more, each load
+// a trip to L2: the ranges that hold them set the pace of the whole grid).
+template <class R, class F>
+__device__ __forceinline__ void apply_items(const ProgSmem<R> &ps, int items, const cx<R> *X, const float4 *Xf, cx<R> shift,
+                                            float4 *s_half, F &&body) {
+    if constexpr (sizeof(R) == 8) {
+        if (2 * items <= (int)blockDim.x) {
+            const int half = blockDim.x / 2, hf = threadIdx.x >= half, it = threadIdx.x - hf * half;
+            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (it < items) {
+                const int j0 = ps.item[it], j1 = ps.item[it + 1], mid = (j0 + j1 + 1) / 2;
+                q = hf ? prog_apply_ff(ps, mid, j1, Xf) : prog_apply_ff(ps, j0, mid, Xf);
+                if (hf) s_half[it] = q;
+            }
+            __syncthreads();
+            if (!hf && it < items) {
+                const float4 o = s_half[it];
+                ff_norm(q.x, q.z);
+                ff_norm(q.y, q.w);
+                ff_add(q.x, q.z, o.x, o.z);
+                ff_add(q.y, q.w, o.y, o.w);
+                body(it, ff_join(q));
+            }
+            return;
+        }
+        for (int it = threadIdx.x; it < items; it += blockDim.x)
+            body(it, ff_join(prog_apply_ff(ps, ps.item[it], ps.item[it + 1], Xf)));
+    } else {
+        for (int it = threadIdx.x; it < items; it += blockDim.x) body(it, prog_apply(ps, it, X, shift));
+    }
 }
 
 // Grid-wide sum of NV doubles: block sums, exchanged by the barrier. Only the first nw warps hold
@@ -173,7 +206,8 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
     extern __shared__ __align__(16) unsigned char smem[];
     double *s_red = reinterpret_cast<double *>(smem);   // [kPersVals][threads]
     double *s_tot = s_red + kPersVals * kPersThreads;   // [4]
-    cx<R> *s_pinv = reinterpret_cast<cx<R> *>(s_tot + 4);
+    float4 *s_half = reinterpret_cast<float4 *>(s_tot + 4);  // [threads / 2]
+    cx<R> *s_pinv = reinterpret_cast<cx<R> *>(s_half + kPersThreads / 2);
     ProgSmem<R> ps = prog_layout<R>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
                                     reinterpret_cast<unsigned char *>(s_pinv + (size_t)v.pers_ados * d2));
     build_programs<R>(v, ps, n0, n1, a.aug, a.set);
@@ -279,16 +313,12 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
         if (!grid_barrier(a.bar, gen, kPersVals, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         // ---- v = A ph, (rh, v)
         double d1[2] = {0.0, 0.0};
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
-            const int64_t i = row0 + it;
-            cx<R> y;
-            if constexpr (sizeof(R) == 8) y = prog_apply_ff(ps, it, a.phf);
-            else y = prog_apply(ps, it, a.ph, shift);
+        apply_items<R>(ps, items, a.ph, a.phf, shift, s_half, [&](int it, cx<R> y) {
             vv[it] = y;
             const cx<double> yd = cast<double>(y), wd = cast<double>(rh[it]);
             d1[0] = fma(wd.re, yd.re, fma(wd.im, yd.im, d1[0]));
             d1[1] = fma(wd.re, yd.im, fma(-wd.im, yd.re, d1[1]));
-        }
+        });
         if (!grid_sum<2>(d1, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         if (threadIdx.x == 0) {
             const cx<double> rv{d1[0], d1[1]};
@@ -312,17 +342,13 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
         if (!grid_barrier(a.bar, gen, kPersVals, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         // ---- t = A sh, (t, s), (t, t)
         double d2v[3] = {0.0, 0.0, 0.0};
-        for (int it = threadIdx.x; it < items; it += blockDim.x) {
-            const int64_t i = row0 + it;
-            cx<R> y;
-            if constexpr (sizeof(R) == 8) y = prog_apply_ff(ps, it, a.shf);
-            else y = prog_apply(ps, it, a.sh, shift);
+        apply_items<R>(ps, items, a.sh, a.shf, shift, s_half, [&](int it, cx<R> y) {
             t[it] = y;
             const cx<double> yd = cast<double>(y), wd = cast<double>(r[it]);
             d2v[0] = fma(yd.re, wd.re, fma(yd.im, wd.im, d2v[0]));
             d2v[1] = fma(yd.re, wd.im, fma(-yd.im, wd.re, d2v[1]));
             d2v[2] = fma(yd.re, yd.re, fma(yd.im, yd.im, d2v[2]));
-        }
+        });
         if (!grid_sum<3>(d2v, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles)) { status = HEOM_ETIMEOUT; break; }
         if (threadIdx.x == 0) {
             const double it2 = d2v[2] == 0.0 ? 0.0 : nr_rcp(d2v[2]);
@@ -392,7 +418,7 @@ DevView<R> view_of_p(const heom_hier *h) {
 
 template <class R>
 size_t persist_smem(const DevView<R> &v) {
-    return kPersVals * kPersThreads * sizeof(double) + 4 * sizeof(double) + (size_t)v.pers_ados * v.d2 * sizeof(cx<R>) +
+    return kPersVals * kPersThreads * sizeof(double) + 4 * sizeof(double) + kPersThreads / 2 * sizeof(float4) + (size_t)v.pers_ados * v.d2 * sizeof(cx<R>) +
            prog_smem_bytes<R>(v.pers_terms, v.pers_slots, v.pers_ados, v.d2) + 64;
 }
 
