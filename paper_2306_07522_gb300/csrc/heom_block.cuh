@@ -404,7 +404,7 @@ inline size_t warp_launch_smem(const DevView<R> &v) {
 // (ADO n, elements e0 .. e0 + NE - 1) of one column, and the function that forms it.
 template <class R, int CW>
 struct RowsLayout {  // runs of a row, operator lists from global memory
-    static constexpr int NE = CW;
+    static constexpr int NE = CW, MINB = 1;
     static constexpr bool VEC = false;
     static __host__ __device__ int per_ado(const DevView<R> &v) { return v.d2 / CW; }
     static __device__ __forceinline__ const OpRec<R> *stage(const DevView<R> &) { return nullptr; }
@@ -445,6 +445,9 @@ struct QuadLayout {  // FP32, one column: four elements, branch-free
 template <class R, int D, int RP, int W>
 struct ColsLayout {  // RP rows of a small block, operators in shared memory
     static constexpr int NE = RP * D, PA = D / RP;
+    // blocks of 256 per SM that kernels with per-column sums are compiled for: the FP32 row waits for loads and
+    // wants the warps (32 sets of uneven depth, 12,951 ADOs: stationary states 111 -> 98 ms)
+    static constexpr int MINB = sizeof(R) == 4 && RP == 1 ? 3 : 1;
     static constexpr bool VEC = false;
     static __host__ __device__ int per_ado(const DevView<R> &) { return PA; }
     static __device__ __forceinline__ const OpRec<R> *stage(const DevView<R> &v) {
@@ -466,7 +469,7 @@ struct ColsLayout {  // RP rows of a small block, operators in shared memory
 
 template <class R>
 struct PointLayout {  // one element
-    static constexpr int NE = 1;
+    static constexpr int NE = 1, MINB = 1;
     static constexpr bool VEC = false;
     static __host__ __device__ int per_ado(const DevView<R> &v) { return v.d2; }
     static __device__ __forceinline__ const OpRec<R> *stage(const DevView<R> &) { return nullptr; }

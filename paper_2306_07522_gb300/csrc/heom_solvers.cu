@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) k_bicg_p(DevView<R> v, const cx<R> *__res
 //   mode 0 (v = A ph):  acc_rv += (rh, v)
 //   mode 1 (t = A sh):  acc_ts += (t, s), acc_tt += (t, t)
 template <class R, class Ly>
-__global__ void __launch_bounds__(256) k_bicg_apply(DevView<R> v, const cx<R> *__restrict__ in,
+__global__ void __launch_bounds__(256, Ly::MINB) k_bicg_apply(DevView<R> v, const cx<R> *__restrict__ in,
                                                     cx<R> *__restrict__ out,
                                                     const cx<R> *__restrict__ w, int64_t B,
                                                     ColSets cps, ApplyMods<R> mods, int mode,
