@@ -955,6 +955,35 @@ struct Solve {
 constexpr int kInnerCap = 400;     // FP32 BiCGStab iterations per refinement sweep
 constexpr int kInnerCap64 = 1500;  // FP64 BiCGStab iterations per sweep (plain path)
 
+// |r|^2 and |b|^2 of the active columns, one block per column, in a fixed order: the norms scale the next
+// sweep's right-hand side, so that a solve of few columns gives the same bits every time (the atomics of
+// k_residual64 add the blocks' sums in the order they arrive)
+__global__ void __launch_bounds__(1024) k_resid_norms(int64_t rows, int64_t B, const cx<double> *__restrict__ r,
+                                                      const cx<double> *__restrict__ bb, ColState *st) {
+    const int64_t b = blockIdx.x;
+    if (!st[b].active) return;
+    __shared__ double sr[1024], sb[1024];
+    double nr = 0.0, nb = 0.0;
+    for (int64_t i = threadIdx.x; i < rows; i += 1024) {
+        nr += norm2(r[i * B + b]);
+        nb += norm2(bb[i * B + b]);
+    }
+    sr[threadIdx.x] = nr;
+    sb[threadIdx.x] = nb;
+    __syncthreads();
+    for (int k = 512; k > 0; k >>= 1) {
+        if ((int)threadIdx.x < k) {
+            sr[threadIdx.x] += sr[threadIdx.x + k];
+            sb[threadIdx.x] += sb[threadIdx.x + k];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        st[b].acc_nr = sr[0];
+        st[b].bnorm2 = sb[0];
+    }
+}
+
 // flagged columns: x = 0, r = b
 __global__ void k_reset_cols(int64_t total, int64_t B, const int *flags, const cx<double> *b,
                              cx<double> *x, cx<double> *r) {
@@ -1037,6 +1066,10 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
               HEOM_LAYOUT_DISPATCH(double, lp, CALL);
 #undef CALL
           } }
+        if (B <= kPersistMaxB) {
+            Prof pr(HEOM_KC_OTHER, s, (double)rows * n_on, 2.0 * rows * n_on * sizeof(cx<double>));
+            k_resid_norms<<<(unsigned)B, 1024, 0, s>>>(rows, B, r64, b64, st_out);
+        }
         HEOM_CUDA(cudaGetLastError());
         HEOM_CUDA(memcpy_counted(hs.data(), st_out, B * sizeof(ColState), cudaMemcpyDeviceToHost, s));
         HEOM_CUDA(cudaStreamSynchronize(s));
