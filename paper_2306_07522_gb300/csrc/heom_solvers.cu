@@ -17,9 +17,10 @@
 namespace heom {
 
 // ------------------------------------------------------------------ block reduction
+// The block's sums per column, added to dst (add) or stored there: a place of the block's own.
 template <int NV>
 __device__ __forceinline__ void reduce_add(double (&val)[NV], double *const (&dst)[NV],
-                                           bool valid) {
+                                           bool valid, bool add = true) {
     __shared__ double sh[NV][256];
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
 #pragma unroll
@@ -34,8 +35,11 @@ __device__ __forceinline__ void reduce_add(double (&val)[NV], double *const (&ds
     }
     if (threadIdx.y == 0 && valid) {
 #pragma unroll
-        for (int i = 0; i < NV; ++i)
-            if (dst[i]) atomicAdd(dst[i], sh[i][threadIdx.x]);
+        for (int i = 0; i < NV; ++i) {
+            if (!dst[i]) continue;
+            if (add) atomicAdd(dst[i], sh[i][threadIdx.x]);
+            else *dst[i] = sh[i][threadIdx.x];
+        }
     }
 }
 
@@ -407,13 +411,14 @@ __global__ void __launch_bounds__(256) k_bicg_x(DevView<R> v, cx<R> *x, const cx
 }
 
 // ------------------------------------------------------------------ refinement helpers
-// r64 = b - A x64 in FP64 with |r|^2 -> acc_nr and |b|^2 -> bnorm2 of the outer state
+// r64 = b - A x64 in FP64 with |r|^2 -> acc_nr and |b|^2 -> bnorm2 of the outer state, or with the
+// block's sums of both -> part[block][2][B] (k_resid_norms adds those in a fixed order)
 template <class Ly>
 __global__ void __launch_bounds__(256) k_residual64(DevView<double> v, const cx<double> *__restrict__ bb,
                                                     const cx<double> *__restrict__ x,
                                                     cx<double> *__restrict__ r, int64_t B,
                                                     ColSets cps, ApplyMods<double> mods,
-                                                    ColState *st) {
+                                                    ColState *st, double *part) {
     constexpr int NE = Ly::NE;
     const OpRec<double> *s_ops = Ly::stage(v);
     COLUMN_PROLOGUE
@@ -439,8 +444,9 @@ __global__ void __launch_bounds__(256) k_residual64(DevView<double> v, const cx<
         }
     }
     double val[2] = {nr, nb};
-    double *const dst[2] = {act ? &st[b].acc_nr : nullptr, act ? &st[b].bnorm2 : nullptr};
-    reduce_add<2>(val, dst, act);
+    double *const own = part ? part + (int64_t)blockIdx.x * 2 * B + b : nullptr;
+    double *const dst[2] = {!act ? nullptr : own ? own : &st[b].acc_nr, !act ? nullptr : own ? own + B : &st[b].bnorm2};
+    reduce_add<2>(val, dst, act, !part);
 }
 
 // rin = r64 / ||r64|| per active column, in the inner solver's precision
@@ -955,23 +961,24 @@ struct Solve {
 constexpr int kInnerCap = 400;     // FP32 BiCGStab iterations per refinement sweep
 constexpr int kInnerCap64 = 1500;  // FP64 BiCGStab iterations per sweep (plain path)
 
-// |r|^2 and |b|^2 of the active columns, one block per column, in a fixed order: the norms scale the next
-// sweep's right-hand side, so that a solve of few columns gives the same bits every time (the atomics of
-// k_residual64 add the blocks' sums in the order they arrive)
-__global__ void __launch_bounds__(1024) k_resid_norms(int64_t rows, int64_t B, const cx<double> *__restrict__ r,
-                                                      const cx<double> *__restrict__ bb, ColState *st) {
+// |r|^2 and |b|^2 of the active columns from the nparts block sums of k_residual64, one block per column,
+// in a fixed order. The norms scale the next sweep's right-hand side, so that a solve whose columns
+// run one by one (bicgstab_persistent) gives the same bits every time; the atomics of k_residual64 add the
+// blocks' sums in the order they arrive. (Read from r and b themselves by this one block they took 77 us of an
+// SM's FP64 pipe at 207,216 elements and 2.1 ms on average at 6.3 million, where the residual takes 69 and 620 us.)
+__global__ void __launch_bounds__(256) k_resid_norms(int nparts, int64_t B, const double *__restrict__ part, ColState *st) {
     const int64_t b = blockIdx.x;
     if (!st[b].active) return;
-    __shared__ double sr[1024], sb[1024];
+    __shared__ double sr[256], sb[256];
     double nr = 0.0, nb = 0.0;
-    for (int64_t i = threadIdx.x; i < rows; i += 1024) {
-        nr += norm2(r[i * B + b]);
-        nb += norm2(bb[i * B + b]);
+    for (int i = threadIdx.x; i < nparts; i += 256) {
+        nr += part[(int64_t)i * 2 * B + b];
+        nb += part[(int64_t)i * 2 * B + B + b];
     }
     sr[threadIdx.x] = nr;
     sb[threadIdx.x] = nb;
     __syncthreads();
-    for (int k = 512; k > 0; k >>= 1) {
+    for (int k = 128; k > 0; k >>= 1) {
         if ((int)threadIdx.x < k) {
             sr[threadIdx.x] += sr[threadIdx.x + k];
             sb[threadIdx.x] += sb[threadIdx.x + k];
@@ -1008,8 +1015,14 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
     // regions of the working layout: per group of columns at most one more than the different
     // depths of its sets, cut into about kRegPieces pieces (rounding adds at most one per region)
     const int64_t reg_cap = 2 * ((B + 31) / 32 + std::min<int64_t>(B, h->n_sets) + 1) + kRegPieces;
+    const DevView<double> v64 = h->view64();
+    const LayoutPick lp = pick_layout(v64, B);
+    const Geom ga = make_geom(rows / lp.ne, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
+    // few columns: the whole BiCGStab solve of a column is one cooperative launch
+    const bool one_by_one = B <= kPersistMaxB && !strict && persist_ok<RI>(h);
     stt = ensure_ws(h->ws_small, align_up(2 * B * sizeof(ColState)) + 3 * align_up(B * sizeof(int)) +
-                                     align_up(reg_cap * sizeof(ColRegion)));
+                                     align_up(reg_cap * sizeof(ColRegion)) +
+                                     (one_by_one ? (size_t)ga.grid.x * 2 * B * sizeof(double) : 0));
     if (stt != HEOM_OK) return stt;
     ColState *st = (ColState *)h->ws_small.p;
     ColState *st_out = st + B;
@@ -1017,6 +1030,7 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
     int *d_map = (int *)((char *)d_flags + align_up(B * sizeof(int)));
     int *d_lmap = (int *)((char *)d_map + align_up(B * sizeof(int)));
     ColRegion *d_reg = (ColRegion *)((char *)d_lmap + align_up(B * sizeof(int)));
+    double *d_part = one_by_one ? (double *)((char *)d_reg + align_up(reg_cap * sizeof(ColRegion))) : nullptr;
     res.iters.assign(B, 0);
     res.refine.assign(B, 0);
     res.status.assign(B, HEOM_OK);
@@ -1033,11 +1047,8 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
         Prof pr(HEOM_KC_OTHER, s, (double)B);
         k_convert<RI, double><<<flat_blocks(B), 256, 0, s>>>(B, shift64, shift_in);
     }
-    const DevView<double> v64 = h->view64();
     const int64_t cps = B / h->n_sets;
     const Geom gd = make_geom(rows, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
-    const LayoutPick lp = pick_layout(v64, B);
-    const Geom ga = make_geom(rows / lp.ne, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
     ApplyMods<double> m64{shift64, aug};
     std::vector<ColState> hs(B);
     std::vector<int> breakdowns(B, 0);
@@ -1062,13 +1073,13 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
               ta.st = st_out; ta.B = B;
               HEOM_CUDA((launch_tile<double, TM_RESID>(ta, s)));
           } else {
-#define CALL(Ly) k_residual64<Ly><<<ga.grid, ga.block, lp.smem, s>>>(v64, b64, x64, r64, B, cps, m64, st_out)
+#define CALL(Ly) k_residual64<Ly><<<ga.grid, ga.block, lp.smem, s>>>(v64, b64, x64, r64, B, cps, m64, st_out, d_part)
               HEOM_LAYOUT_DISPATCH(double, lp, CALL);
 #undef CALL
           } }
-        if (B <= kPersistMaxB) {
-            Prof pr(HEOM_KC_OTHER, s, (double)rows * n_on, 2.0 * rows * n_on * sizeof(cx<double>));
-            k_resid_norms<<<(unsigned)B, 1024, 0, s>>>(rows, B, r64, b64, st_out);
+        if (d_part) {
+            Prof pr(HEOM_KC_OTHER, s, (double)B, 2.0 * ga.grid.x * B * sizeof(double));
+            k_resid_norms<<<(unsigned)B, 256, 0, s>>>((int)ga.grid.x, B, d_part, st_out);
         }
         HEOM_CUDA(cudaGetLastError());
         HEOM_CUDA(memcpy_counted(hs.data(), st_out, B * sizeof(ColState), cudaMemcpyDeviceToHost, s));
@@ -1118,8 +1129,7 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
         const double inner_tol = plain ? std::max(0.5 * tol / worst, 1e-10) : 1e-4;
         inner_max = std::min(inner_max, plain ? kInnerCap64 : kInnerCap);
         SolveOut o;
-        if (B <= kPersistMaxB && !strict && persist_ok<RI>(h)) {
-            // few columns: the whole BiCGStab solve of a column is one cooperative launch
+        if (one_by_one) {
             o.iters.assign(B, 0);
             o.status.assign(B, HEOM_OK);
             o.res.assign(B, 0.0);
