@@ -387,12 +387,11 @@ heom_status shifted_gmres(heom_hier *h, const cx<double> *bvec, int64_t B,
                           double tol, int mmax, std::vector<cx<double>> &x0,
                           std::vector<double> &res, int *steps, cudaStream_t s);
 
-// cooperative persistent BiCGStab for one column of b and x (heom_persist.cu); from kPersistMaxB columns on they
-// run together in launches per step instead: 2 columns of 301 ADOs of 4 x 4, mixed precision, 28 against 6 ms,
-// 8 columns 45 against 25 ms, 16 columns 44 against 50 ms
-constexpr int64_t kPersistMaxB = 8;
+// cooperative persistent BiCGStab for one column of b and x (heom_persist.cu)
 template <class R>
 bool persist_ok(const heom_hier *h);
+template <class R>
+int64_t persist_max_cols(const heom_hier *h);  // up to this many columns run one after another
 template <class R>
 heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col, bool x_zero,
                                 const cx<R> *shift, R aug, double tol, int max_iter,

@@ -433,6 +433,23 @@ bool persist_ok(const heom_hier *h) {
 template bool persist_ok<double>(const heom_hier *);
 template bool persist_ok<float>(const heom_hier *);
 
+// A persistent iteration takes 25 to 45 us a column whatever the hierarchy (its barriers), a batched one 70 us and
+// more for all columns together (five launches, two of them waiting for the longest chain of neighbour entries), so the
+// line follows the entries: 6 an ADO in the spin-boson model, 15 in the small charge-cavity model, 24 in the Anderson
+// model. Stationary states, ms, one by one against together (FP64; mixed):
+//   35 ADOs of 2 x 2:          2 columns 3.0 / 2.8, 3 4.3 / 2.8, 8 11.0 / 3.4; 2 5.5 / 9.6, 3 8.2 / 9.7, 8 21 / 9.7
+//   charge-cavity, 60 iter.:   2 4.0 / 5.2, 5 9.6 / 5.4; 2 3.2 / 3.6, 5 7.5 / 3.7
+//   25 ADOs of 4 x 4:          3 1.1 / 1.3, 4 1.3 / 1.5, 5 1.7 / 1.5, 8 2.5 / 1.5; 5 4.0 / 5.8, 6 4.8 / 5.8, 8 6.4 / 5.8
+//   301 ADOs:                  3 5.2 / 6.8, 4 7.2 / 7.3, 5 8.6 / 8.2, 8 13.2 / 7.3; 5 14.2 / 33, 8 23 / 47
+//   2,325 ADOs, uneven depths: 4 9.3 / 12.3, 8 20.6 / 16.2; 5 24.5 / 28.9, 8 29.9 / 36.5
+template <class R>
+int64_t persist_max_cols(const heom_hier *h) {
+    if (h->max_entries < 20) return 2;
+    return sizeof(R) == 8 ? 4 : h->N < 100 ? 5 : 8;
+}
+template int64_t persist_max_cols<double>(const heom_hier *);
+template int64_t persist_max_cols<float>(const heom_hier *);
+
 // One persistent BiCGStab solve of (M + shift + aug e00 tr) x = b for column col of b and x ([rows][B]; a starting
 // vector other than zero only with B = 1).
 template <class R>
