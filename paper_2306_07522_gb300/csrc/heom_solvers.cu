@@ -307,6 +307,49 @@ __global__ void __launch_bounds__(256, Ly::MINB) k_bicg_apply(DevView<R> v, cons
     }
 }
 
+// The same for the FP32 launches of bicg_point: one element per thread in (32 columns x 8 elements) blocks, as in
+// k_apply_point. A thread has one element or a few, so its dot products are formed in FP64.
+template <class R>
+__global__ void __launch_bounds__(256) k_bicg_apply_point(DevView<R> v, const cx<R> *__restrict__ in,
+                                                          cx<R> *__restrict__ out, const cx<R> *__restrict__ w,
+                                                          int64_t B, ColSets cps, ApplyMods<R> mods, int mode,
+                                                          ColState *st) {
+    COLUMN_PROLOGUE
+    const bool act = inb && st[b].active;
+    double c_re = 0, c_im = 0, tt = 0;
+    if (act) {
+        for (int64_t row = (int64_t)blockIdx.x * blockDim.y + threadIdx.y; row < rows;
+             row += (int64_t)gridDim.x * blockDim.y) {
+            const int64_t n = ado_of(row, v.d2, rows), i = row * B + b;
+            const int e = (int)(row - n * v.d2);
+            if (beyond_cap(v, n, set)) continue;  // zero there, and nothing reads it
+            cx<R> x0[1], y[1];
+            y[0] = apply_point(v, in, n, e, b, B, set, x0[0]);
+            apply_mods<R, 1>(mods, v, in, n, e, b, B, x0, y);
+            out[i] = y[0];
+            const cx<double> yd = cast<double>(y[0]), wd = cast<double>(w[i]);
+            const cx<double> p = mode == 0 ? wd : yd, q = mode == 0 ? yd : wd;  // sum conj(p) q
+            c_re += p.re * q.re + p.im * q.im;
+            c_im += p.re * q.im - p.im * q.re;
+            if (mode) tt += norm2(yd);
+        }
+    }
+    if (mode == 0) {
+        double val[2] = {c_re, c_im};
+        double *const dst[2] = {act ? &st[b].acc_rv.re : nullptr, act ? &st[b].acc_rv.im : nullptr};
+        reduce_add<2>(val, dst, act);
+    } else {
+        double val[3] = {c_re, c_im, tt};
+        double *const dst[3] = {act ? &st[b].acc_ts.re : nullptr, act ? &st[b].acc_ts.im : nullptr,
+                                act ? &st[b].acc_tt.re : nullptr};
+        reduce_add<3>(val, dst, act);
+        if (act && blockIdx.x == 0 && threadIdx.y == 0) {
+            st[b].acc_rr = {0.0, 0.0};
+            st[b].acc_nr = 0.0;
+        }
+    }
+}
+
 // alpha = rho / (rh, v); s = r - alpha v (in place in r); sh = P^-1 s
 template <class R>
 __global__ void __launch_bounds__(256) k_bicg_s(DevView<R> v, cx<R> *r, const cx<R> *__restrict__ vv,
@@ -606,6 +649,23 @@ struct SolveOut {
     std::vector<double> res;  // final relative residual sqrt(acc_nr / bnorm2)
 };
 
+// Whether the FP32 apply of an iteration runs one element per thread (k_bicg_apply_point): small vectors, where the
+// row kernel's longer chains and its sums over up to 256 threads a column cost more than its decoding saves. us per
+// launch against the row kernel: 400 elements x 8 to 64 columns 23 / 33, 4,816 x 5 26 / 35, x 64 28 / 34, 37,200 x 8
+// 32 / 37, x 9 50 / 39, 207,216 x 2 44 / 47, x 3 68 / 48; one column: 207,216 30 / 43, 469,072 58 / 81, 6.3 million
+// 526 / 330. (B: the columns of the whole solve, so that the rounding does not change as columns converge.)
+template <class R>
+inline bool bicg_point(const DevView<R> &v, int64_t B) {
+    return sizeof(R) == 4 && (double)v.N * v.d2 * (double)B < (B == 1 ? 1e6 : 320e3);
+}
+// Columns from which the row kernel's lanes hold neighbouring columns (a warp then has the rows of few ADOs). FP64
+// vectors below 16,000 elements stay with one element per thread, us per launch: 660 elements x 5 columns 17 / 26,
+// 400 x 8 29 / 43, x 32 25 / 35.
+template <class R>
+inline int64_t bicg_cols_min(const DevView<R> &v, int64_t B) {
+    return sizeof(R) == 8 && (double)v.N * v.d2 * (double)B < 16e3 ? INT64_MAX : 4;
+}
+
 constexpr int kStallIters = 96;
 
 // Batched right-preconditioned BiCGStab on A x = b, A = M + diag(shift) (+ trace aug), from
@@ -665,9 +725,11 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
     LayoutPick lp;
     std::vector<ColRegion> regs;
     dim3 ga, gd, gv;
-    Geom gi;  // start-up: every row of every column
+    Geom gi;  // every row of every column: start-up, one element per thread
+    bool point = false;
     auto geoms = [&]() -> heom_status {
-        lp = pick_layout(v, Bc, false, 4);  // a warp holds the rows of few ADOs from 4 columns on
+        lp = pick_layout(v, Bc, false, bicg_cols_min(v, B));
+        point = bicg_point(v, B);
         regs.clear();
         for (int64_t c0 = 0; c0 < Bc;) {
             const int64_t w = Bc - c0 <= 64 ? Bc - c0 : 32;
@@ -844,27 +906,29 @@ heom_status bicgstab(heom_hier *h, const cx<R> *bvec, cx<R> *x, int64_t B, const
         const double u_vec = (double)rows * Bc;
         const double sz = sizeof(cx<R>), e_vec = u_vec * sz;
         // one iteration: five kernels on stream q (event brackets when accounting is on)
+        auto apply = [&](const cx<R> *in, cx<R> *o, const cx<R> *wv, int mode, cudaStream_t q) {
+            if constexpr (sizeof(R) == 4)
+                if (point) {
+                    k_bicg_apply_point<R><<<gi.grid, gi.block, 0, q>>>(v, in, o, wv, Bc, cps, mods, mode, st);
+                    return;
+                }
+#define CALL(Ly) k_bicg_apply<R, Ly><<<ga, kRegThreads, lp.smem, q>>>(v, in, o, wv, Bc, cps, mods, mode, d_reg, st)
+            HEOM_LAYOUT_DISPATCH(R, lp, CALL);
+#undef CALL
+        };
         auto launch_iter = [&](cudaStream_t q, bool prof, bool set_attr) -> cudaError_t {
             cudaError_t e = cudaSuccess;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 5.0 * e_vec); pr.on = pr.on && prof;
               k_bicg_p<R><<<gv, kRegThreads, 0, q>>>(v, r, p, vv, ph, rh, Bc, cps, shc, 1, d_reg, st); }
             { Prof pr(kc_apply, q, u_app, 3.0 * e_vec); pr.on = pr.on && prof;
               if (tiled) { ta.x = ph; ta.out = vv; ta.w = rh; e = launch_tile<R, TM_BICG_V>(ta, q, set_attr); }
-              else {
-#define CALL(Ly) k_bicg_apply<R, Ly><<<ga, kRegThreads, lp.smem, q>>>(v, ph, vv, rh, Bc, cps, mods, 0, d_reg, st)
-                  HEOM_LAYOUT_DISPATCH(R, lp, CALL);
-#undef CALL
-              } }
+              else apply(ph, vv, rh, 0, q); }
             if (e != cudaSuccess) return e;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 4.0 * e_vec); pr.on = pr.on && prof;
               k_bicg_s<R><<<gv, kRegThreads, 0, q>>>(v, r, vv, sh, Bc, cps, shc, 1, d_reg, st); }
             { Prof pr(kc_apply, q, u_app, 3.0 * e_vec); pr.on = pr.on && prof;
               if (tiled) { ta.x = sh; ta.out = t; ta.w = r; e = launch_tile<R, TM_BICG_T>(ta, q, set_attr); }
-              else {
-#define CALL(Ly) k_bicg_apply<R, Ly><<<ga, kRegThreads, lp.smem, q>>>(v, sh, t, r, Bc, cps, mods, 1, d_reg, st)
-                  HEOM_LAYOUT_DISPATCH(R, lp, CALL);
-#undef CALL
-              } }
+              else apply(sh, t, r, 1, q); }
             if (e != cudaSuccess) return e;
             { Prof pr(HEOM_KC_KRYLOV_VECTOR, q, u_vec, 8.0 * e_vec); pr.on = pr.on && prof;
               k_bicg_x<R><<<gd, kRegThreads, 0, q>>>(v, xw, ph, sh, r, t, rh, Bc, cps, d_reg, st); }
