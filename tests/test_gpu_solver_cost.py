@@ -45,3 +45,18 @@ def test_columns_run_together_where_that_is_faster(prec, cols):
     applies = pr["krylov_apply_fp64" if prec == "FP64" else "krylov_apply_fp32"]["launches"]
     assert applies <= cols * sweeps if cols <= 2 else applies > 8 * sweeps
     assert float((x.reshape(g.n_ado, 2, 2, cols)[0, 0, 0] + x.reshape(g.n_ado, 2, 2, cols)[0, 1, 1] - 1).abs().max()) < 1e-9
+
+
+@pytest.mark.parametrize("tier,cols,prec,one_by_one", [
+    (1, 4, "FP64", True), (1, 5, "FP64", False), (1, 5, "MIXED", True), (1, 6, "MIXED", False),
+    (2, 8, "MIXED", True), (2, 9, "MIXED", False), (3, 6, "FP64", True), (3, 7, "FP64", False)])
+def test_columns_of_long_neighbour_lists(tier, cols, prec, one_by_one):
+    """24 entries an ADO: the last number of columns that run one by one and the first that runs together."""
+    import torch
+    import paper_2306_07522_gb300 as heom
+    g = heom.build_hierarchy(heom.problem_from_model(W.siam_model(tier=tier)))
+    x = torch.zeros((g.n_ado, 4, 4, cols), dtype=torch.complex128, device="cuda")
+    pr = _accounted(heom, lambda: heom.steady(g, x, tol=1e-10, max_iter=4000, prec=getattr(heom, prec)))
+    applies = pr["krylov_apply_fp64" if prec == "FP64" else "krylov_apply_fp32"]["launches"]
+    assert (applies <= cols * pr["residual_fp64"]["launches"]) == one_by_one
+    assert float((torch.diagonal(x[0]).sum(-1) - 1).abs().max()) < 1e-9
