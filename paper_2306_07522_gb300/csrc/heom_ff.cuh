@@ -123,7 +123,8 @@ __device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
 // Sum of products of FP32 values to more than FP64's precision on the FP32 pipe, two sums at a
 // time: each product split exactly by an FMA (p + e), each addition exactly by Knuth's two-sum,
 // the errors of the first level summed in a second level with its own exact additions and those
-// of the second in a third, so a sum's relative error is about 2^-70. GB300's FP64 pipe would
+// of the second in a third, so a sum's relative error is about 2^-70 as long as the products stay between
+// 2^-101 and 2^127 / (their number); beyond that it is inf or NaN and the caller has to look. GB300's FP64 pipe would
 // spend 64 cycles of a sub-partition on every converted operand and every multiply-add; a
 // product here takes about 20 packed instructions.
 struct Sum3 {

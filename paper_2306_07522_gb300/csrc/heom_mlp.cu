@@ -259,8 +259,9 @@ __global__ void k_destandardise(int64_t M, int n, const float *__restrict__ y, c
 }
 
 // g = 2 (y - ts) / (M n) with ts the standardised targets (t - mean) / sd; per-block partial sums
-// of (y - ts)^2 into part[block] (exact FP32 sums, see Sum3: an FP64 multiply-add per element
-// would take longer than the rest)
+// of (y - ts)^2 into part[block] (FP32 sums of more bits than FP64's, see Sum3: an FP64 multiply-add per
+// element would take longer than the rest). Where a thread's sum leaves the range in which those are exact -- a
+// diverging network, or one that fits to the last bits -- it is formed again in FP64.
 __global__ void __launch_bounds__(256) k_mse_grad(int64_t total, int n, const float *__restrict__ y,
                                                   const float *__restrict__ t, const float *__restrict__ mean,
                                                   const float *__restrict__ sd, float *__restrict__ g,
@@ -275,7 +276,17 @@ __global__ void __launch_bounds__(256) k_mse_grad(int64_t total, int n, const fl
         g[i] = scale * dlt;
         acc.mac(make_float2(dlt, 0.f), make_float2(dlt, 0.f));
     }
-    sh[threadIdx.x] = acc.x();
+    double sum = acc.x();
+    if (!(sum >= 0x1p-60 && isfinite(sum))) {
+        sum = 0.0;
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+             i += (int64_t)gridDim.x * blockDim.x) {
+            const int c = (int)(i % n);
+            const double dlt = (double)(y[i] - (t[i] - mean[c]) / sd[c]);
+            sum += dlt * dlt;
+        }
+    }
+    sh[threadIdx.x] = sum;
     __syncthreads();
     for (int s = 128; s > 0; s >>= 1) {
         if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];

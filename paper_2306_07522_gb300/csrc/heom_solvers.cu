@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "heom_block.cuh"
+#include "heom_dots.cuh"
 #include "heom_tile.cuh"
 
 namespace heom {
@@ -49,38 +50,6 @@ __device__ __forceinline__ void reduce_add(double (&val)[NV], double *const (&ds
     const int64_t rows = v.N * v.d2;                                       \
     const int set = inb ? cps.set(b) : 0;                                  \
     (void)set; (void)rows;
-
-// Per-column dot products of a thread over its entries: c = sum conj(a) b and n = sum |b|^2. FP64
-// vectors in FP64; FP32 vectors in exact FP32 sums (Sum3).
-template <class R>
-struct ColDots;
-template <>
-struct ColDots<double> {
-    double re = 0, im = 0, nn = 0;
-    __device__ __forceinline__ void cross(cx<double> a, cx<double> b) {
-        re += a.re * b.re + a.im * b.im;
-        im += a.re * b.im - a.im * b.re;
-    }
-    __device__ __forceinline__ void norm(cx<double> b) { nn += norm2(b); }
-    __device__ __forceinline__ double c_re() const { return re; }
-    __device__ __forceinline__ double c_im() const { return im; }
-    __device__ __forceinline__ double n() const { return nn; }
-};
-template <>
-struct ColDots<float> {
-    Sum3 c, q;
-    __device__ __forceinline__ void cross(cx<float> a, cx<float> b) {
-        c.mac(make_float2(a.re, a.re), make_float2(b.re, b.im));
-        c.mac(make_float2(a.im, a.im), make_float2(b.im, -b.re));
-    }
-    __device__ __forceinline__ void norm(cx<float> b) {
-        const float2 x = make_float2(b.re, b.im);
-        q.mac(x, x);
-    }
-    __device__ __forceinline__ double c_re() const { return c.x(); }
-    __device__ __forceinline__ double c_im() const { return c.y(); }
-    __device__ __forceinline__ double n() const { return q.x() + q.y(); }
-};
 
 // ADO of a row, by a 32-bit division where the vector allows it
 __device__ __forceinline__ int64_t ado_of(int64_t row, int d2, int64_t rows) {
@@ -291,12 +260,33 @@ __global__ void __launch_bounds__(256, Ly::MINB) k_bicg_apply(DevView<R> v, cons
             }
         }
     }
+    DotVals sum(dots);
+    if (dots.overflowed()) {  // again from what has been stored, in FP64
+        ColDots<double> wide;
+        REGION_RUNS(Ly) {
+            int64_t n;
+            int e0;
+            Ly::pos(v, q, small, n, e0);
+            if (beyond_cap(v, n, set)) continue;
+            for (int u = 0; u < NE; ++u) {
+                const int64_t i = (n * v.d2 + e0 + u) * B + b;
+                const cx<double> y = cast<double>(out[i]), wv = cast<double>(w[i]);
+                if (mode == 0) {
+                    wide.cross(wv, y);
+                } else {
+                    wide.cross(y, wv);
+                    wide.norm(y);
+                }
+            }
+        }
+        sum = DotVals(wide);
+    }
     if (mode == 0) {
-        double val[2] = {dots.c_re(), dots.c_im()};
+        double val[2] = {sum.re, sum.im};
         double *const dst[2] = {act ? &st[b].acc_rv.re : nullptr, act ? &st[b].acc_rv.im : nullptr};
         region_add<2>(rg, val, dst, act);
     } else {
-        double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
+        double val[3] = {sum.re, sum.im, sum.n};
         double *const dst[3] = {act ? &st[b].acc_ts.re : nullptr, act ? &st[b].acc_ts.im : nullptr,
                                 act ? &st[b].acc_tt.re : nullptr};
         region_add<3>(rg, val, dst, act);
@@ -433,7 +423,7 @@ __global__ void __launch_bounds__(256) k_bicg_x(DevView<R> v, cx<R> *x, const cx
     if (act) {
         const cx<R> al = c.a, om = c.b;
         const Kept kept(v, set);
-    REGION_ROWS {
+        REGION_ROWS {
             if (!kept(ado_of(row, v.d2, v.N * v.d2))) continue;
             const int64_t i = row * B + b;
             x[i] = x[i] + al * ph[i] + om * sh[i];
@@ -443,7 +433,19 @@ __global__ void __launch_bounds__(256) k_bicg_x(DevView<R> v, cx<R> *x, const cx
             dots.norm(ri);
         }
     }
-    double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
+    DotVals sum(dots);
+    if (dots.overflowed()) {  // again from what has been stored, in FP64
+        ColDots<double> wide;
+        const Kept kept(v, set);
+        REGION_ROWS {
+            if (!kept(ado_of(row, v.d2, v.N * v.d2))) continue;
+            const cx<double> rd = cast<double>(r[row * B + b]);
+            wide.cross(cast<double>(rh[row * B + b]), rd);
+            wide.norm(rd);
+        }
+        sum = DotVals(wide);
+    }
+    double val[3] = {sum.re, sum.im, sum.n};
     double *const dst[3] = {act ? &st[b].acc_rr.re : nullptr, act ? &st[b].acc_rr.im : nullptr,
                             act ? &st[b].acc_nr : nullptr};
     region_add<3>(rg, val, dst, act);
