@@ -177,7 +177,6 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
     int *s_flag = reinterpret_cast<int *>(s_sum + kBarVals);           // [2 + kArMaxB]
     ProgSmem<double> ps = prog_layout<double>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
                                               reinterpret_cast<unsigned char *>(s_flag + 4 + kArMaxB));
-    __shared__ float2 s_nf[kArMaxB];  // 1 / |w| in float-float
     float4 *const s_w = a.w_off >= 0 ? reinterpret_cast<float4 *>(smem + a.w_off) : nullptr;
     float4 *const s_rs = reinterpret_cast<float4 *>(smem + a.rot_off);
     float2 *const s_rc = reinterpret_cast<float2 *>(s_rs + (size_t)a.rcap * a.nsh);
@@ -327,22 +326,17 @@ __global__ void __launch_bounds__(kArThreads, 1) k_arnoldi(ArnoldiArgs a) {
         if (!grid_exchange(a.bar, gen, B, a.wait_cycles, B, tid < B ? s_nrm[tid] : 0.0, s_sum, RedSum{})) { status = 1; break; }
         if (tid < B) {
             const double n = std::sqrt(s_sum[tid]);
-            const double inv = n > 0.0 ? 1.0 / n : 0.0;  // used by every element
-            const float ih = (float)inv;
-            s_nf[tid] = make_float2(ih, (float)(inv - (double)ih));
+            s_nrm[tid] = n > 0.0 ? 1.0 / n : 0.0;  // the inverse, used by every element
             s_hcol[(j + 1) * B + tid] = cx<double>{n, 0.0};
         }
         __syncthreads();
-        // v_{j+1} = w / |w| in float-float for the next steps; the FP64 copy only of the
+        // v_{j+1} = w / |w| in FP64, rounded to float-float for the next steps; the FP64 copy only of the
         // tier-0 rows (elements below d2 * B), which the final combination x_0 = V_0 y reads,
         // so that the basis held in L2 is the float-float one alone
         for (int idx = tid; idx < nel; idx += bd) {
-            float4 w = wl[idx];
-            const float2 sc = s_nf[idx % B];  // zero norm: zeros
-            ff_scale(w.x, w.z, sc.x, sc.y);
-            ff_scale(w.y, w.w, sc.x, sc.y);
-            W[e0 + idx] = w;
-            if (e0 + idx < (int64_t)d2 * B) a.V[(int64_t)(j + 1) * a.L + e0 + idx] = ff_join(w);
+            const cx<double> x = s_nrm[idx % B] * ff_join(wl[idx]);  // zero norm: zeros
+            if (e0 + idx < (int64_t)d2 * B) a.V[(int64_t)(j + 1) * a.L + e0 + idx] = x;
+            W[e0 + idx] = ff_split(x);
         }
         // Hessenberg column j to global memory (CTA 0); its rows 0 .. j split into float-float
         // for the rotation chains (s_hf is free again: the Gram-Schmidt update has used it)
