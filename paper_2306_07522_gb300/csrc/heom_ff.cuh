@@ -145,6 +145,14 @@ struct Sum3 {
         two_sum2(m, e, w);
         l = f2_add(l, f2_add(u, w));
     }
+    // += the float-float values hi + lo
+    __device__ __forceinline__ void add(float2 hi, float2 lo) {
+        float2 t, u, w;
+        two_sum2(h, hi, t);
+        two_sum2(m, t, u);
+        two_sum2(m, lo, w);
+        l = f2_add(l, f2_add(u, w));
+    }
     __device__ __forceinline__ double x() const { return ((double)h.x + (double)m.x) + (double)l.x; }
     __device__ __forceinline__ double y() const { return ((double)h.y + (double)m.y) + (double)l.y; }
 };

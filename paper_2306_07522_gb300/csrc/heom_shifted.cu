@@ -438,9 +438,9 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // Each thread streams its rows through a ring of kD2Depth stages in shared memory filled by asynchronous
 // copies, so the loads of the next rows are in flight while it computes: bytes and
 // float-float arithmetic take about the same time here and have to overlap. The sums over a column's
-// threads are formed in float-float by all threads of the block (by one thread per column in FP64 they
-// took a third of a block's time at 32 columns). 16 sets of uneven depth, 12,951 ADOs, 140 steps: 143.6 -> 76.8 ms
-// of the solve's 336, now at the rate of the update (k_update2_ff, 85.9 ms).
+// threads are formed by all threads of the block, in FP32 sums of more bits than FP64's (by one thread per column in
+// FP64 they took a third of a block's time at 32 columns). 16 sets of uneven depth, 12,951 ADOs, 140 steps: 143.6 ->
+// 76.8 ms of the solve's 336, now at the rate of the update (k_update2_ff).
 constexpr int kD2Tile = 6, kD2Depth = 3;
 constexpr size_t kD2Smem = (size_t)kD2Depth * (kD2Tile + 2) * kDotThreads * sizeof(float4);
 static_assert(kD2Depth * (kD2Tile + 2) >= 2 * kD2Tile, "the ring holds the block's sums at the end");
@@ -519,14 +519,13 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_dots2_ff_tiled(int64_t B, in
     const int per = kDotThreads / max(ch.acols, 1);
     for (int t = threadIdx.x; t < nt * 2 * (int)B; t += kDotThreads) {
         const int kr = t / (int)B, cl = t - kr * (int)B;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        Sum3 acc;  // (re, im)
         if (cl < ch.acols)
             for (int q = 0; q < per; ++q) {
                 const float4 x = dring[kr * kDotThreads + cl + q * ch.acols];
-                ff_add(acc.x, acc.z, x.x, x.z);
-                ff_add(acc.y, acc.w, x.y, x.w);
+                acc.add(make_float2(x.x, x.y), make_float2(x.z, x.w));
             }
-        part[((int64_t)c * nv + i0) * 2 * B + t] = ff_join(acc);
+        part[((int64_t)c * nv + i0) * 2 * B + t] = cx<double>{acc.x(), acc.y()};
     }
 }
 
