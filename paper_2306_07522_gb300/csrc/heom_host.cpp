@@ -139,7 +139,7 @@ void ws_release(DBuf &b, int device) {
     if (evict.buf.p) free_on_device(evict);
 }
 
-heom_status ensure_ws(DBuf &b, size_t bytes) {
+heom_status ensure_ws(DBuf &b, size_t bytes, size_t most) {
     if (b.bytes >= bytes && b.p) return HEOM_OK;
     g_ws_takes.fetch_add(1);
     int dev = 0;
@@ -149,7 +149,7 @@ heom_status ensure_ws(DBuf &b, size_t bytes) {
         std::lock_guard<std::mutex> lk(g_ws_mu);
         size_t best = g_ws_cache.size();
         for (size_t i = 0; i < g_ws_cache.size(); ++i)
-            if (g_ws_cache[i].device == dev && g_ws_cache[i].buf.bytes >= bytes &&
+            if (g_ws_cache[i].device == dev && g_ws_cache[i].buf.bytes >= bytes && g_ws_cache[i].buf.bytes <= most &&
                 (best == g_ws_cache.size() || g_ws_cache[i].buf.bytes < g_ws_cache[best].buf.bytes))
                 best = i;
         if (best < g_ws_cache.size()) {
@@ -1441,6 +1441,7 @@ extern "C" void heom_destroy(heom_hier *h) {
     heom::ws_release(h->ws_small, h->device);
     heom::ws_release(h->ws_pers, h->device);
     heom::ws_release(h->ws_res, h->device);
+    heom::ws_release(h->ws_rhs, h->device);
     free_all(h);
     delete h;
 }

@@ -321,7 +321,8 @@ struct DeviceScope {
 heom_status dalloc(DBuf &b, size_t bytes);  // the library's only cudaMalloc (counted)
 long long wait_limit_cycles();               // bound of device-side waits (heom_set_wait_limit)
 void dfree(DBuf &b);
-heom_status ensure_ws(DBuf &b, size_t bytes);  // grows b, from the workspace cache when it can
+// grows b, from the workspace cache when that has a buffer of bytes .. most
+heom_status ensure_ws(DBuf &b, size_t bytes, size_t most = SIZE_MAX);
 void ws_release(DBuf &b, int device);           // hands b to the workspace cache
 size_t ws_cached_total(int device);             // bytes of the cached workspaces on a device
 void ws_release_all();

@@ -1452,9 +1452,6 @@ extern "C" heom_status heom_evolve_td(heom_hier *h, void *ados, int64_t batch, d
                               (cx<float> *)rho_traj, f, (cudaStream_t)s);
 }
 
-// a buffer of the hierarchy's own, allocated anew only when it is too small
-static heom_status keep_buf(DBuf &b, size_t bytes) { return b.p && b.bytes >= bytes ? HEOM_OK : dalloc(b, bytes); }
-
 static void fill_stats(heom_solve_stats *stats, const Solve &r, int64_t off, int64_t n) {
     if (!stats) return;
     for (int64_t b = 0; b < n; ++b) {
@@ -1479,8 +1476,10 @@ extern "C" heom_status heom_steady(heom_hier *h, const void *x0, void *x_out, in
     cudaStream_t st = (cudaStream_t)s;
     const int64_t rows = h->N * h->d2, L = rows * batch;
     // the right-hand side e_(0,(0,0)), the columns' factors and norms: a workspace of their own, kept like
-    // the solvers' (a cudaMalloc and a cudaFree, which waits for the device, cost as much as an iteration or more)
-    heom_status stt = keep_buf(h->ws_rhs, (size_t)L * sizeof(cx<double>) + batch * (sizeof(cx<double>) + 2 * sizeof(double)));
+    // the solvers' (a cudaMalloc and a cudaFree, which waits for the device, cost as much as an iteration or more). No
+    // cached buffer of more than twice its size: the solver's own, asked for next, is 8 to 16 times as large.
+    const size_t rhs_bytes = (size_t)L * sizeof(cx<double>) + batch * (sizeof(cx<double>) + 2 * sizeof(double));
+    heom_status stt = ensure_ws(h->ws_rhs, rhs_bytes, 2 * rhs_bytes);
     if (stt != HEOM_OK) return stt;
     cx<double> *b64 = (cx<double> *)h->ws_rhs.p, *x = (cx<double> *)x_out;
     { Prof pr(HEOM_KC_OTHER, st, (double)L);
@@ -1547,7 +1546,8 @@ static heom_status spectrum_shifted(heom_hier *odd, const void *ss_ados, const h
     const int d = odd->d;
     const int64_t ns = odd->n_sets, B = 2 * ns;
     const int64_t rows = odd->N * odd->d2, L = rows * B;
-    heom_status stt = keep_buf(odd->ws_rhs, (size_t)(L + 2 * d * d) * sizeof(cx<double>));
+    const size_t rhs_bytes = (size_t)(L + 2 * d * d) * sizeof(cx<double>);
+    heom_status stt = ensure_ws(odd->ws_rhs, rhs_bytes, 2 * rhs_bytes);
     if (stt != HEOM_OK) return stt;
     cx<double> *b64 = (cx<double> *)odd->ws_rhs.p, *ops = b64 + L;
     std::vector<cx<double>> hops(2 * d * d);
