@@ -370,14 +370,14 @@ heom_status heom_psd(heom_hier *even, const void *ss_ados, const heom_c64 *op_a,
 
 /* Autotuner of the apply for one batch width (measurement of this GPU; the paper has no
  * counterpart). Times heom_apply on a library-allocated test vector of `batch` columns in
- * precision prec with the per-element kernel and with the tiled kernel at 1..5 ADO ranges
- * per SM -- in FP32 each with every kernel variant (columns per lane / terms per item in
+ * precision prec without the tiled kernel (per-element kernels, or block products for dense
+ * FP32 operators) and with the tiled kernel at 1..5 ADO ranges per SM -- in FP32 each with every kernel variant (columns per lane / terms per item in
  * flight / items per warp in flight / CTAs per SM the registers are sized for -- 0: 2/4/1/3;
  * 1: 2/4/1/4; 2: 2/3/1/4; 3: 2/2/1/5; 4: 2/6/1/3; 5: 4/4/1/2) -- and keeps the fastest in h: the tiled granularity and variant for every later
- * batched apply and solve, or, when the per-element kernel wins, the per-element kernel for
- * batches up to `batch` columns. candidates_us: host [6] or NULL (index 0 per-element,
+ * batched apply and solve, or, when the first wins, no tiling for
+ * batches up to `batch` columns. candidates_us: host [6] or NULL (index 0 untiled,
  * p = 1..5 the fastest variant of the tiled kernel with p ranges per SM, -1 where not
- * applicable); tiled, ctas_per_sm, best_us, variant (-1 when the per-element kernel won):
+ * applicable); tiled, ctas_per_sm, best_us, variant (-1 when the untiled kernel won):
  * host or NULL. Results do not depend on the granularity (the same terms, summed in the
  * same order); the tiled and per-element kernels agree to rounding. Allocates two vectors
  * of N d^2 batch elements for the duration of the call. Synchronises s. */
@@ -386,8 +386,8 @@ heom_status heom_autotune(heom_hier *h, int64_t batch, int prec, double *candida
                           heom_stream s);
 
 /* Pin the configuration the autotuner would choose (the paper has no counterpart): the
- * tiled kernel for every batch of 16 or more columns, at ctas_per_sm ADO ranges per SM
- * (1..5) and FP32 variant `variant` (0..5, as listed for heom_autotune; FP64 ignores it). For
+ * tiled kernel for every batch of 16 or more columns that it can take -- applies, solvers and
+ * RK4 alike, before any other kernel --, at ctas_per_sm ADO ranges per SM (1..5) and FP32 variant `variant` (0..5, as listed for heom_autotune; FP64 ignores it). For
  * reproducible timings and for tests of each variant. Results agree with every other
  * configuration to rounding. Errors: HEOM_EINVAL for arguments out of range. */
 heom_status heom_set_tile_config(heom_hier *h, int ctas_per_sm, int variant);

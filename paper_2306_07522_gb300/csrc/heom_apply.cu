@@ -130,10 +130,12 @@ __global__ void __launch_bounds__(512) k_apply_staged(DevView<R> v, const cx<R> 
 template <class R>
 cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t B,
                          const ApplyMods<R> &mods, cudaStream_t s) {
-    if constexpr (sizeof(R) == 4)
-        if (!mods.shift && mods.aug == 0.f && dense_ok(v, B)) return launch_apply_dense(v, x, y, B, s);
     // the tiled kernel reads and writes 16-byte vectors: both buffers must be 16-byte aligned
-    if (tile_ok(v, B) && (((uintptr_t)x | (uintptr_t)y) & 15) == 0) {
+    const bool tiled = tile_ok(v, B) && (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
+    if constexpr (sizeof(R) == 4)
+        if (!(tiled && v.tile_pinned) && !mods.shift && mods.aug == 0.f && dense_ok(v, B))
+            return launch_apply_dense(v, x, y, B, s);
+    if (tiled) {
         TileArgs<R> a{};
         a.v = v;
         a.x = x;
@@ -313,9 +315,9 @@ heom_status autotune(heom_hier *h, int64_t B, double *cand, int *tiled, int *per
     if (st != HEOM_OK) return st;
     cx<R> *x = (cx<R> *)buf.p, *y = x + total;
     k_tune_fill<R><<<(unsigned)std::min<int64_t>((total + 255) / 256, 152 * 16), 256, 0, s>>>(total, x);
-    const int per_sm0 = h->tile_per_sm, var0 = h->tile_var;
+    const int per_sm0 = h->tile_per_sm, var0 = h->tile_var, pinned0 = h->tile_pinned;
     const int64_t min_b0 = h->tile_min_b;
-    // candidate 0: the row kernel (tiled kernel switched off)
+    // candidate 0: what runs with the tiled kernel switched off
     h->tile_min_b = INT64_MAX;
     double t0 = 0.0;
     st = tune_time<R>(h, x, y, B, s, &t0);
@@ -331,6 +333,7 @@ heom_status autotune(heom_hier *h, int64_t B, double *cand, int *tiled, int *per
         if (!tile_possible) continue;
         if ((st = set_tile_partition(h, p)) != HEOM_OK) break;
         h->tile_min_b = 16;
+        h->tile_pinned = 1;
         for (int var = 0; var < n_var && st == HEOM_OK; ++var) {
             h->tile_var = var;
             bool ok;
@@ -348,11 +351,13 @@ heom_status autotune(heom_hier *h, int64_t B, double *cand, int *tiled, int *per
         set_tile_partition(h, per_sm0);
         h->tile_min_b = min_b0;
         h->tile_var = var0;
+        h->tile_pinned = pinned0;
         return st;
     }
-    // keep the winner: tiled with best_p ranges per SM and variant best_v, or the per-element
-    // kernel for batches up to this width (wider batches keep the tiled kernel at its default
-    // granularity)
+    // keep the winner: tiled with best_p ranges per SM and variant best_v, or no tiling
+    // for batches up to this width (wider batches keep the tiled kernel at its default
+    // granularity). The dense kernel is FP32's.
+    h->tile_pinned = sizeof(R) == 4 ? (best_p > 0 ? 1 : 0) : std::min(pinned0, 1);
     if (best_p > 0) {
         st = set_tile_partition(h, best_p);
         h->tile_min_b = 16;
@@ -406,5 +411,6 @@ extern "C" heom_status heom_set_tile_config(heom_hier *h, int ctas_per_sm, int v
     if (st != HEOM_OK) return st;
     h->tile_var = variant;
     h->tile_min_b = 16;
+    h->tile_pinned = 2;
     return HEOM_OK;
 }

@@ -437,7 +437,7 @@ heom::DevView<double> heom_hier::view64() const {
     v.max_terms = max_terms; v.max_entries = max_entries;
     v.cta_ado = (const int32_t *)d_cta_ado.p; v.n_ranges = n_ranges; v.range_terms = range_terms;
     v.range_slots = range_slots; v.range_ados = range_ados; v.tile_min_b = tile_min_b;
-    v.tile_var = tile_var;
+    v.tile_var = tile_var; v.tile_pinned = tile_pinned;
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
     v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;
@@ -471,7 +471,7 @@ heom::DevView<float> heom_hier::view32() const {
     v.max_terms = max_terms; v.max_entries = max_entries;
     v.cta_ado = (const int32_t *)d_cta_ado.p; v.n_ranges = n_ranges; v.range_terms = range_terms;
     v.range_slots = range_slots; v.range_ados = range_ados; v.tile_min_b = tile_min_b;
-    v.tile_var = tile_var;
+    v.tile_var = tile_var; v.tile_pinned = tile_pinned;
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
     v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;

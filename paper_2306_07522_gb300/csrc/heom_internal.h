@@ -132,6 +132,7 @@ struct DevView {
     int n_ranges;
     int64_t tile_min_b;       // smallest batch that takes the tiled kernel (autotuned, >= 16)
     int tile_var;             // FP32 variant of the tiled kernel (kTileVariant, autotuned)
+    int tile_pinned;          // the tiled kernel goes before the dense one (1: tuned) and before every other (2: set)
     int range_terms;          // largest program of one range (terms)
     int range_slots;          // largest sum over a range of d2 * (entries + 3)
     int range_ados;           // largest number of ADOs in a range
@@ -254,6 +255,7 @@ struct heom_hier {
     int tile_per_sm = 2;        // tiled kernel: ADO ranges per SM (autotuned)
     int64_t tile_min_b = 16;    // tiled kernel from this batch on (autotuned)
     int tile_var = 0;           // FP32 tiled-kernel variant (autotuned)
+    int tile_pinned = 0;        // see DevView
     int pers_ranges = 0, pers_terms = 0, pers_slots = 0, pers_ados = 0;
     heom::DBuf d_ar_ado;        // ADO ranges of the persistent Arnoldi (elements weighted)
     int ar_ranges = 0, ar_terms = 0, ar_slots = 0, ar_ados = 0;

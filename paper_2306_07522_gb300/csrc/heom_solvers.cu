@@ -1343,8 +1343,8 @@ heom_status evolve_impl(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t n_
         }
         return HEOM_OK;
     };
-    // small hierarchies: whole columns in shared memory
-    if (n_steps > 0 && resident_ok(h, B, (int)sizeof(cx<R>))) {
+    // small hierarchies: whole columns in shared memory, unless the caller has pinned the tiled kernel
+    if (n_steps > 0 && !(tiled && v.tile_pinned == 2) && resident_ok(h, B, (int)sizeof(cx<R>))) {
         bool done = true;
         const int64_t chunk = td ? (kTdChunk - 1) / 2 : n_steps;
         for (int64_t n = 0; n < n_steps && done && st == HEOM_OK; n += chunk) {
