@@ -703,9 +703,10 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     }
     std::vector<float> fl32(fl.begin(), fl.end());
     h->nS = nS;
+    // the term program of the shared-memory RK4 holds the system terms' pattern, not their values
+    if (h->s_ptr != sptr || h->s_src != ssrc) h->res = heom::ResPlan{};
     h->s_ptr = sptr;
     h->s_src = ssrc;
-    h->res = heom::ResPlan{};  // its program follows the system terms
     // largest term program of one ADO: damping (1 per element) + system terms + neighbour
     // terms + trace row
     {
