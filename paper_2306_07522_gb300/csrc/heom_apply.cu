@@ -204,8 +204,10 @@ __global__ void k_damping(int64_t N, int n_sets, const int32_t *__restrict__ occ
 
 heom_status fill_damping(heom_hier *h, int n_sets, cudaStream_t s) {
     const int64_t total = h->N * n_sets;
-    heom_status st = dalloc(h->d_damp64, total * sizeof(cx<double>));
-    if (st == HEOM_OK) st = dalloc(h->d_damp32, total * sizeof(cx<float>));
+    heom_status st = HEOM_OK;
+    // tables of the same size stay (the uploads before this have waited for the device)
+    if (h->d_damp64.bytes != total * sizeof(cx<double>)) st = dalloc(h->d_damp64, total * sizeof(cx<double>));
+    if (st == HEOM_OK && h->d_damp32.bytes != total * sizeof(cx<float>)) st = dalloc(h->d_damp32, total * sizeof(cx<float>));
     if (st != HEOM_OK) return st;
     const Geom g = flat_geom(std::min<int64_t>(total, 152 * 16 * 256));
     k_damping<<<g.grid, g.block, 0, s>>>(h->N, n_sets, (const int32_t *)h->d_occ_ptr.p, (const OccEntry *)h->d_occ.p,

@@ -455,24 +455,15 @@ size_t arnoldi_smem(const DevView<double> &v, int hcap) {
 }
 
 // The FP64 view with the Arnoldi's own ADO ranges in place of the persistent solver's.
-DevView<double> arnoldi_view(const heom_hier *h) {
-    DevView<double> v = h->view64();
-    v.pers_ado = (const int32_t *)h->d_ar_ado.p;
-    v.pers_ranges = h->ar_ranges;
-    v.pers_terms = h->ar_terms;
-    v.pers_slots = h->ar_slots;
-    v.pers_ados = h->ar_ados;
-    return v;
-}
 
 }  // namespace
 
 bool arnoldi_persistent_ok(const heom_hier *h, int64_t B, int max_steps) {
     // the resident term programs carry one parameter set's coefficients
     if (h->n_sets != 1 || h->has_caps) return false;
-    if (h->ar_ranges < 1 || h->ar_ranges > kBarMaxGrid || B < 1 || B > kArMaxB || (32 % B) != 0 || (kArThreads % B) != 0) return false;
+    if (h->pers_ranges < 1 || h->pers_ranges > kBarMaxGrid || B < 1 || B > kArMaxB || (32 % B) != 0 || (kArThreads % B) != 0) return false;
     const int steps = std::min(max_steps, kArMaxSteps);
-    return arnoldi_smem(arnoldi_view(h), (steps + 2) * (int)B) <= 200 * 1024;
+    return arnoldi_smem(h->view64(), (steps + 2) * (int)B) <= 200 * 1024;
 }
 
 int arnoldi_max_steps() { return kArMaxSteps; }
@@ -486,14 +477,14 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
                                double *rot_c, cx<double> *rot_s, cx<double> *rdiag, cx<double> *g,
                                float2 *rot_cf, float4 *rot_sf, const double *beta, double *res,
                                double tol, int *steps, bool *converged, cudaStream_t s) {
-    const int G = h->ar_ranges;
+    const int G = h->pers_ranges;
     const size_t part_bytes = (size_t)G * kPartStride * sizeof(double);
     const size_t hred_bytes = (size_t)2 * (kArMaxSteps + 2) * kArMaxB * sizeof(cx<double>);
     heom_status st = ensure_ws(h->ws_pers, part_bytes + hred_bytes + 128 + grid_bar_bytes(G, (int)B));
     if (st != HEOM_OK) return st;
     char *base = (char *)h->ws_pers.p;
     ArnoldiArgs a{};
-    a.v = arnoldi_view(h);
+    a.v = h->view64();
     a.B = B;
     a.L = h->N * h->d2 * B;
     a.S = S;

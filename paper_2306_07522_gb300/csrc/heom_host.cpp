@@ -430,7 +430,7 @@ heom::DevView<double> heom_hier::view64() const {
     v.s_ptr = (const int32_t *)d_s_ptr.p; v.s_src = (const int32_t *)d_s_src.p;
     v.s_val = (const cx<double> *)d_sval64.p; v.sdiag = (const cx<double> *)d_sdiag64.p;
     v.coefL = (const cx<double> *)d_coefL64.p; v.coefR = (const cx<double> *)d_coefR64.p;
-    v.rate = (const cx<double> *)d_rate64.p; v.damp = (const cx<double> *)d_damp64.p;
+    v.damp = (const cx<double> *)d_damp64.p;
     v.floor = (const double *)d_floor64.p;
     v.t_ptr = (const int32_t *)d_t_ptr.p; v.t_src = (const int32_t *)d_t_src.p;
     v.t_val = (const cx<double> *)d_t_val64.p;
@@ -441,8 +441,8 @@ heom::DevView<double> heom_hier::view64() const {
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
     v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;
-    v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_ranges = pers_ranges;
-    v.pers_terms = pers_terms; v.pers_slots = pers_slots; v.pers_ados = pers_ados;
+    v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_terms = pers_terms; v.pers_slots = pers_slots;
+    v.pers_ados = pers_ados;
     v.op_rvalf = (const float4 *)d_op_rvalff.p; v.op_cvalf = (const float4 *)d_op_cvalff.p;
     v.s_valf = (const float4 *)d_svalff.p; v.coefLf = (const float4 *)d_coefLff.p;
     v.coefRf = (const float4 *)d_coefRff.p; v.ratef = (const float4 *)d_rateff.p;
@@ -464,7 +464,7 @@ heom::DevView<float> heom_hier::view32() const {
     v.s_ptr = (const int32_t *)d_s_ptr.p; v.s_src = (const int32_t *)d_s_src.p;
     v.s_val = (const cx<float> *)d_sval32.p; v.sdiag = (const cx<float> *)d_sdiag32.p;
     v.coefL = (const cx<float> *)d_coefL32.p; v.coefR = (const cx<float> *)d_coefR32.p;
-    v.rate = (const cx<float> *)d_rate32.p; v.damp = (const cx<float> *)d_damp32.p;
+    v.damp = (const cx<float> *)d_damp32.p;
     v.floor = (const float *)d_floor32.p;
     v.t_ptr = (const int32_t *)d_t_ptr.p; v.t_src = (const int32_t *)d_t_src.p;
     v.t_val = (const cx<float> *)d_t_val32.p;
@@ -475,8 +475,8 @@ heom::DevView<float> heom_hier::view32() const {
     v.ado_tier = has_caps ? (const int32_t *)d_ado_tier.p : nullptr;
     v.set_cap = has_caps ? (const int32_t *)d_set_cap.p : nullptr;
     v.set_end = has_caps && cap_prefix ? (const int32_t *)d_set_end.p : nullptr;
-    v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_ranges = pers_ranges;
-    v.pers_terms = pers_terms; v.pers_slots = pers_slots; v.pers_ados = pers_ados;
+    v.pers_ado = (const int32_t *)d_pers_ado.p; v.pers_terms = pers_terms; v.pers_slots = pers_slots;
+    v.pers_ados = pers_ados;
     return v;
 }
 
@@ -487,11 +487,11 @@ void free_all(heom_hier *h) {
                     &h->d_op_rcol, &h->d_op_cptr, &h->d_op_crow, &h->d_op_rrec64,
                     &h->d_op_crec64, &h->d_op_rrec32, &h->d_op_crec32, &h->d_op_ell64, &h->d_op_ell32, &h->d_perm, &h->d_damp64, &h->d_damp32, &h->d_s_ptr,
                     &h->d_s_src, &h->d_sval64, &h->d_sval32, &h->d_coefL64, &h->d_coefL32,
-                    &h->d_coefR64, &h->d_coefR32, &h->d_rate64, &h->d_rate32, &h->d_sdiag64,
+                    &h->d_coefR64, &h->d_coefR32, &h->d_rate64, &h->d_sdiag64,
                     &h->d_sdiag32, &h->d_tdval64, &h->d_floor64, &h->d_floor32, &h->ws,
                     &h->ws_small,
                     &h->d_t_ptr, &h->d_t_src, &h->d_t_val64, &h->d_t_val32, &h->d_cta_ado,
-                    &h->d_pers_ado, &h->d_ar_ado, &h->d_dense32, &h->ws_pers, &h->ws_res, &h->ws_rhs, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
+                    &h->d_pers_ado, &h->d_dense32, &h->ws_pers, &h->ws_res, &h->ws_rhs, &h->d_ado_tier, &h->d_set_cap, &h->d_set_end,
                     &h->d_op_rvalff, &h->d_op_cvalff, &h->d_svalff, &h->d_coefLff, &h->d_coefRff,
                     &h->d_rateff};
     for (DBuf *b : bufs) heom::dfree(*b);
@@ -724,7 +724,7 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     // bounded for shared memory. Tiled kernel: tile_per_sm CTAs per SM (two unless the
     // autotuner chose otherwise), all resident at once. Cooperative persistent solvers: one
     // range per SM.
-    std::vector<int32_t> ranges, pranges, arranges;
+    std::vector<int32_t> ranges, pranges;
     {
         RangeCosts rc = range_costs(h);
         int n_sm = 152;
@@ -735,38 +735,25 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
         h->range_terms = (int)std::min<int64_t>(rt, INT32_MAX);
         h->range_slots = (int)std::min<int64_t>(rs, INT32_MAX);
         h->range_ados = (int)rn;
-        const bool pfit = partition_ranges(h, rc, n_sm, heom::kPersistTerms, pranges, rt, rs, rn);
-        h->pers_ranges = (pfit && rt <= heom::kPersistTerms && rs <= heom::kRangeSlots) ? (int)pranges.size() - 1 : 0;
-        h->pers_terms = (int)std::min<int64_t>(rt, INT32_MAX);
-        h->pers_slots = (int)std::min<int64_t>(rs, INT32_MAX);
-        h->pers_ados = (int)rn;
-        // The persistent Arnoldi's Gram-Schmidt work grows with the elements a range owns
-        // (about 2 (j + 1) float-float multiply-adds per element and step), the apply with its
-        // terms: its ranges balance terms + kArElemWeight * d2 per ADO. Without a fitting
-        // partition it keeps the one above.
+        // Much of a persistent solver's work is per element a range owns (the Arnoldi's Gram-Schmidt about 2 (j + 1)
+        // float-float multiply-adds per element and step, the BiCGStab's FP64 vectors: balanced on terms alone the
+        // ranges of the tier-3 Anderson model hold 80 to 400 elements, and 400 cost 10,500 cycles in the first
+        // update), the apply's is per term: the ranges balance terms + kArElemWeight * d2 per ADO, terms alone where
+        // that does not fit.
         std::vector<int64_t> w(h->N);
         int64_t wt = 0;
         for (int64_t i = 0; i < h->N; ++i) { w[i] = rc.terms[i] + heom::kArElemWeight * h->d2; wt += w[i]; }
-        std::vector<int32_t> ar;
-        const bool afit = partition_ranges(h, rc, n_sm, heom::kPersistTerms, ar, rt, rs, rn, &w, wt) &&
-                          rt <= heom::kPersistTerms && rs <= heom::kRangeSlots;
-        if (afit) {
-            arranges = ar;
-            h->ar_ranges = (int)ar.size() - 1;
-            h->ar_terms = (int)rt;
-            h->ar_slots = (int)rs;
-            h->ar_ados = (int)rn;
-        } else {
-            arranges = pranges;
-            h->ar_ranges = h->pers_ranges;
-            h->ar_terms = h->pers_terms;
-            h->ar_slots = h->pers_slots;
-            h->ar_ados = h->pers_ados;
-        }
+        const auto fits = [&](bool part) { return part && rt <= heom::kPersistTerms && rs <= heom::kRangeSlots; };
+        const bool fit = fits(partition_ranges(h, rc, n_sm, heom::kPersistTerms, pranges, rt, rs, rn, &w, wt)) ||
+                         fits(partition_ranges(h, rc, n_sm, heom::kPersistTerms, pranges, rt, rs, rn));
+        h->pers_ranges = fit ? (int)pranges.size() - 1 : 0;
+        h->pers_terms = (int)std::min<int64_t>(rt, INT32_MAX);
+        h->pers_slots = (int)std::min<int64_t>(rs, INT32_MAX);
+        h->pers_ados = (int)rn;
     }
     heom_status st;
 #define UP(buf, vec) if ((st = upload(h->buf, vec)) != HEOM_OK) return st
-    UP(d_cta_ado, ranges); UP(d_pers_ado, pranges); UP(d_ar_ado, arranges);
+    UP(d_cta_ado, ranges); UP(d_pers_ado, pranges);
     UP(d_s_ptr, sptr); UP(d_s_src, ssrc);
     UP(d_sval64, to_cx<double>(sval)); UP(d_sval32, to_cx<float>(sval)); UP(d_svalff, to_ff(sval));
     UP(d_coefLff, to_ff(cl)); UP(d_coefRff, to_ff(cr)); UP(d_rateff, to_ff(rt));
@@ -774,7 +761,7 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     UP(d_tdval64, to_cx<double>(tdval));
     UP(d_coefL64, to_cx<double>(cl)); UP(d_coefL32, to_cx<float>(cl));
     UP(d_coefR64, to_cx<double>(cr)); UP(d_coefR32, to_cx<float>(cr));
-    UP(d_rate64, to_cx<double>(rt)); UP(d_rate32, to_cx<float>(rt));
+    UP(d_rate64, to_cx<double>(rt));
     UP(d_floor64, fl); UP(d_floor32, fl32);
     // dense apply: blocks of 8 to 32 with at least a quarter of the operators' entries non-zero (term
     // by term an entry costs about four times what it costs in a block product, zero or not)

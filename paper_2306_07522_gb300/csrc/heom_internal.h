@@ -105,7 +105,6 @@ struct DevView {
     // hold neighbouring columns (and so neighbouring sets), read one contiguous run.
     const cx<R> *coefL;       // [K][n_sets]
     const cx<R> *coefR;       // [K][n_sets]
-    const cx<R> *rate;        // [K][n_sets]
     const cx<R> *damp;        // [N][n_sets]  sum_k count_k rate_k of every ADO
     const R *floor;           // [n_sets]      damping floor for undamped ADOs (preconditioner)
     // ADO-local system superoperator L_s X = -i (H X - X H) + sum_k gamma_k J(F_k)[X] (the
@@ -139,7 +138,7 @@ struct DevView {
     // ADO ranges of the cooperative persistent solvers: one range per SM, programs of the
     // whole hierarchy resident in shared memory (pers_ranges = 0 when they do not fit)
     const int32_t *pers_ado;  // [pers_ranges + 1]
-    int pers_ranges, pers_terms, pers_slots, pers_ados;
+    int pers_terms, pers_slots, pers_ados;
     // Per-set truncation (heom_set_truncation; both null when unused): ADO n has fermionic
     // tier ado_tier[n] & 0xffff and bosonic tier ado_tier[n] >> 16; parameter set s keeps
     // the ADOs with fermionic tier <= set_cap[s] & 0xffff and bosonic tier <= set_cap[s] >> 16
@@ -257,11 +256,9 @@ struct heom_hier {
     int tile_var = 0;           // FP32 tiled-kernel variant (autotuned)
     int tile_pinned = 0;        // see DevView
     int pers_ranges = 0, pers_terms = 0, pers_slots = 0, pers_ados = 0;
-    heom::DBuf d_ar_ado;        // ADO ranges of the persistent Arnoldi (elements weighted)
-    int ar_ranges = 0, ar_terms = 0, ar_slots = 0, ar_ados = 0;
     // device parameters (per set), both precisions and float-float
     heom::DBuf d_sval64, d_sval32, d_coefL64, d_coefL32, d_coefR64, d_coefR32, d_rate64,
-        d_rate32, d_damp64, d_damp32, d_sdiag64, d_sdiag32, d_floor64, d_floor32, d_svalff, d_coefLff, d_coefRff,
+        d_damp64, d_damp32, d_sdiag64, d_sdiag32, d_floor64, d_floor32, d_svalff, d_coefLff, d_coefRff,
         d_rateff;
     // solver workspace (grown on demand)
     heom::DBuf ws;
@@ -337,7 +334,7 @@ constexpr int kPersistTerms = 6144;  // terms of one persistent range (FP64: 20 
 // FP64 one-column layout of small blocks, two warps of 32 ADOs per SM sub-partition (29,317 ADOs of 4 x 4: 220 us
 // this way, 97 us staged in groups of threads; 396,607 ADOs: 418 us this way)
 constexpr int64_t kWarpMinAdos = 64 * 608;
-constexpr int64_t kArElemWeight = 128;  // persistent Arnoldi: balance weight of one element
+constexpr int64_t kArElemWeight = 128;  // persistent solvers: balance weight of one element
 
 // launch geometry shared by every row x column kernel: block (bx, by), grid (gx, gy)
 struct Geom {

@@ -400,20 +400,10 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.out = PersistOut{it_done, status, nr, bn};
 }
 
-// The view with ADO ranges balanced on terms + 128 d^2 per ADO: most of an iteration is FP64 vector work, which
-// follows a range's elements (balanced on terms alone the ranges of the tier-3 Anderson model hold 80 to 400
-// of them, and 400 cost 10,500 cycles in the first update alone).
 template <class R>
 DevView<R> view_of_p(const heom_hier *h) {
-    DevView<R> v;
-    if constexpr (sizeof(R) == 8) v = h->view64();
-    else v = h->view32();
-    v.pers_ado = (const int32_t *)h->d_ar_ado.p;
-    v.pers_ranges = h->ar_ranges;
-    v.pers_terms = h->ar_terms;
-    v.pers_slots = h->ar_slots;
-    v.pers_ados = h->ar_ados;
-    return v;
+    if constexpr (sizeof(R) == 8) return h->view64();
+    else return h->view32();
 }
 
 template <class R>
@@ -426,7 +416,7 @@ size_t persist_smem(const DevView<R> &v) {
 
 template <class R>
 bool persist_ok(const heom_hier *h) {
-    if (h->ar_ranges < 1 || h->ar_ranges > kBarMaxGrid) return false;
+    if (h->pers_ranges < 1 || h->pers_ranges > kBarMaxGrid) return false;
     const DevView<R> v = view_of_p<R>(h);
     return persist_smem(v) <= 200 * 1024;
 }
@@ -459,7 +449,7 @@ heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t 
                                 cudaStream_t s) {
     const DevView<R> v = view_of_p<R>(h);
     const int64_t rows = h->N * h->d2;
-    const int G = h->ar_ranges;
+    const int G = h->pers_ranges;
     const size_t vec = ((size_t)rows * sizeof(cx<R>) + 255) & ~size_t(255);
     const size_t fvec = sizeof(R) == 8 ? (((size_t)rows * sizeof(float4) + 255) & ~size_t(255)) : 0;
     const size_t bytes = 8 * vec + 2 * fvec + 128 + grid_bar_bytes(G, kPersVals);
