@@ -202,16 +202,22 @@ cudaError_t launch_bt(const DevView<float> &v, const cx<float> *x, cx<float> *y,
 
 }  // namespace
 
+// columns of a CTA
+static int dense_columns(int d, int64_t B) { return B > 4 && d < 32 ? 8 : 4; }
+
 bool dense_ok(const DevView<float> &v, int64_t B) {
-    return v.dense && v.n_sets == 1 && !v.set_cap && v.max_entries <= kDenseMaxEntries &&
-           (double)v.N * (double)((B + 3) / 4) < 2147483647.0;
+    if (!v.dense || v.n_sets != 1 || v.set_cap || v.max_entries > kDenseMaxEntries) return false;
+    const int bt = dense_columns(v.d, B);
+    const double ctas = (double)v.N * (double)((B + bt - 1) / bt);
+    return ctas >= v.dense_min && ctas < 2147483647.0;
 }
 
 cudaError_t launch_apply_dense(const DevView<float> &v, const cx<float> *x, cx<float> *y, int64_t B, cudaStream_t s) {
+    const bool wide = dense_columns(v.d, B) == 8;
     switch (v.d) {
-    case 8: return B > 4 ? launch_bt<8, 8>(v, x, y, B, s) : launch_bt<8, 4>(v, x, y, B, s);
-    case 16: return B > 4 ? launch_bt<16, 8>(v, x, y, B, s) : launch_bt<16, 4>(v, x, y, B, s);
-    case 24: return B > 4 ? launch_bt<24, 8>(v, x, y, B, s) : launch_bt<24, 4>(v, x, y, B, s);
+    case 8: return wide ? launch_bt<8, 8>(v, x, y, B, s) : launch_bt<8, 4>(v, x, y, B, s);
+    case 16: return wide ? launch_bt<16, 8>(v, x, y, B, s) : launch_bt<16, 4>(v, x, y, B, s);
+    case 24: return wide ? launch_bt<24, 8>(v, x, y, B, s) : launch_bt<24, 4>(v, x, y, B, s);
     default: return launch_bt<32, 4>(v, x, y, B, s);
     }
 }

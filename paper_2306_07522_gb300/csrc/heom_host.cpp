@@ -452,6 +452,7 @@ heom::DevView<double> heom_hier::view64() const {
 heom::DevView<float> heom_hier::view32() const {
     heom::DevView<float> v{};
     v.dense = has_dense ? (const heom::cx<float> *)d_dense32.p : nullptr;
+    v.dense_min = dense_min;
     v.N = N; v.d = d; v.d2 = d2; v.K = K; v.n_sets = n_sets; v.nS = nS;
     v.n_ops = n_ops; v.op_width = op_width; v.op_real = op_real; v.perm = (const int32_t *)d_perm.p;
     v.row_ptr = (const int32_t *)d_row_ptr.p; v.ent = (const NbEntry *)d_ent.p;
@@ -763,11 +764,17 @@ heom_status upload_params(heom_hier *h, int n_sets, const heom_c64 *H, const heo
     UP(d_coefR64, to_cx<double>(cr)); UP(d_coefR32, to_cx<float>(cr));
     UP(d_rate64, to_cx<double>(rt));
     UP(d_floor64, fl); UP(d_floor32, fl32);
-    // dense apply: blocks of 8 to 32 with at least a quarter of the operators' entries non-zero (term
-    // by term an entry costs about four times what it costs in a block product, zero or not)
+    // Dense apply: blocks of 8 to 32 with at least a quarter of the operators' entries non-zero (term
+    // by term an entry costs about four times what it costs in a block product, zero or not). With less than half
+    // of them and large blocks a few CTAs take longer than the many threads of the term by term kernels: from half a
+    // wave on (76 CTAs). 27 ADOs, us, block products against term by term: d = 24, a quarter non-zero, 8 / 16 columns (27 / 54
+    // CTAs) 49 / 51 against 34 / 38, 33 columns (135) 55 against 105, half non-zero, 16 columns 51 against 61;
+    // d = 32, 1 / 8 columns (27 / 54) 51 / 53 against 34 / 47, 16 columns (108) 57 against 76; d = 16, 1 to 16 columns
+    // 24 to 26 against 23 to 26, 0.3 non-zero 24 to 26 against 26 to 28; d = 8 13 to 14 against 17 to 47.
     size_t nnz = 0;
     for (const heom_c64 &o : h->ops) nnz += o.re != 0.0 || o.im != 0.0;
     h->has_dense = n_sets == 1 && n_lind == 0 && d % 8 == 0 && d <= 32 && 4 * nnz >= h->ops.size() && h->n_ops > 0;
+    h->dense_min = 2 * nnz >= h->ops.size() || d < 24 ? 0 : 76;
     if (h->has_dense) {
         std::vector<heom_c64> dn(h->ops);
         dn.insert(dn.end(), H, H + d2);

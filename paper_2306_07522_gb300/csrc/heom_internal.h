@@ -87,6 +87,7 @@ struct DevView {
     // operators and H without zeros as [n_ops + 1][d2], H last (FP32 view; null unless one parameter
     // set, no Lindblad terms and a block size the dense kernel takes: heom_dense.cu)
     const cx<R> *dense;
+    int dense_min;            // CTAs from which a launch takes the dense kernel
     int op_real;              // 1 when every operator is real
     // ADO order of the one-column layout (heom_block.cuh): ADOs whose neighbour entries use the
     // same operators one after another are neighbours (null: none)
@@ -265,6 +266,7 @@ struct heom_hier {
     heom::DBuf ws_small;
     heom::DBuf d_dense32;       // operators and H for the dense apply
     bool has_dense = false;
+    int dense_min = 0;
     std::vector<int32_t> s_ptr, s_src;   // system terms (host copies of d_s_ptr, d_s_src)
     heom::ResPlan res;                   // shared-memory RK4: program, and its device copy
     heom::DBuf ws_res;
