@@ -8,12 +8,14 @@
 // thread forms RT = d / 4 rows of one block column for four batch columns, so a step of the
 // inner loop is 4 RT complex multiply-adds on packed FP32 pairs for RT + 2 (left) or 2 RT + 1 (right)
 // 16-byte shared-memory loads, most of them broadcasts. Real and imaginary parts lie in separate planes: a
-// pair holds two columns, and one accumulator pair takes the real, one the imaginary part.
+// pair holds two columns, and one accumulator pair takes the real, one the imaginary part. Zero entries of the
+// operators are multiplied like the others unless a block sum is infinite or NaN: those spread over couplings only.
 //
 // 222 ADOs of 24 x 24: 64 columns 2,595 us (term by term) -> 354 us, bound by FP32 issue (12.6 GFLOP of block
 // products); one column 133 -> 50 us, bound by a CTA's chain of products. 16 x 16: 748 -> 118 us at 64
 // columns, 99 -> 25 us at one.
 #include <cstdint>
+#include <type_traits>
 
 #include "heom_ff.cuh"
 #include "heom_kernels.cuh"
@@ -105,6 +107,7 @@ __global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, cons
         bool any = o == v.n_ops;
         for (int t = 0; t < cnt && !any; ++t) any = ent[t].op == o;
         if (!any) continue;
+        bool fine = true;  // this thread's sums are finite
         for (int e = tid; e < D2; e += T) {
             const cx<float> w = ldc(v.dense + (int64_t)o * D2 + e);
             rec[e] = make_float4(w.re, w.re, w.im, w.im);
@@ -143,36 +146,47 @@ __global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, cons
                 const int w = (tid + (i + u) * T) * 4;
                 st_planes(Lr + w, Li + w, lr[u], li[u]);
                 st_planes(Rr + w, Ri + w, rr[u], ri[u]);
+                const float2 tot = f2_add(f2_add(f2_add(lr[u][0], lr[u][1]), f2_add(li[u][0], li[u][1])),
+                                          f2_add(f2_add(rr[u][0], rr[u][1]), f2_add(ri[u][0], ri[u][1])));
+                fine = fine && isfinite(tot.x) && isfinite(tot.y);
             }
         }
-        __syncthreads();
+        const bool wild = __syncthreads_or(!fine);
+        // a zero entry of the operator couples nothing, whatever S and T hold
+        const auto products = [&](auto masked) {
+            constexpr bool MASK = decltype(masked)::value;
 #pragma unroll 2
-        for (int l = 0; l < D; ++l) {  // O S
-            const int w = (l * D + c) * BT + 4 * bq;
-            const float4 xr = *reinterpret_cast<const float4 *>(Lr + w), xi = *reinterpret_cast<const float4 *>(Li + w),
-                         nx = neg(xi);
+            for (int l = 0; l < D; ++l) {  // O S
+                const int w = (l * D + c) * BT + 4 * bq;
+                const float4 xr = *reinterpret_cast<const float4 *>(Lr + w), xi = *reinterpret_cast<const float4 *>(Li + w),
+                             nx = neg(xi);
 #pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                const float4 q = rec[(r0 + r) * D + l];
-                are[r][0] = f2_fma(hi(q), lo(nx), f2_fma(lo(q), lo(xr), are[r][0]));
-                are[r][1] = f2_fma(hi(q), hi(nx), f2_fma(lo(q), hi(xr), are[r][1]));
-                aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
-                aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
+                for (int r = 0; r < RT; ++r) {
+                    const float4 q = rec[(r0 + r) * D + l];
+                    if (MASK && q.x == 0.f && q.z == 0.f) continue;
+                    are[r][0] = f2_fma(hi(q), lo(nx), f2_fma(lo(q), lo(xr), are[r][0]));
+                    are[r][1] = f2_fma(hi(q), hi(nx), f2_fma(lo(q), hi(xr), are[r][1]));
+                    aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
+                    aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
+                }
             }
-        }
 #pragma unroll 2
-        for (int l = 0; l < D; ++l) {  // T O
-            const float4 q = rec[l * D + c], nq = neg(q);
+            for (int l = 0; l < D; ++l) {  // T O
+                const float4 q = rec[l * D + c], nq = neg(q);
+                if (MASK && q.x == 0.f && q.z == 0.f) continue;
 #pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                const int w = ((r0 + r) * D + l) * BT + 4 * bq;
-                const float4 xr = *reinterpret_cast<const float4 *>(Rr + w), xi = *reinterpret_cast<const float4 *>(Ri + w);
-                are[r][0] = f2_fma(hi(nq), lo(xi), f2_fma(lo(q), lo(xr), are[r][0]));
-                are[r][1] = f2_fma(hi(nq), hi(xi), f2_fma(lo(q), hi(xr), are[r][1]));
-                aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
-                aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
+                for (int r = 0; r < RT; ++r) {
+                    const int w = ((r0 + r) * D + l) * BT + 4 * bq;
+                    const float4 xr = *reinterpret_cast<const float4 *>(Rr + w), xi = *reinterpret_cast<const float4 *>(Ri + w);
+                    are[r][0] = f2_fma(hi(nq), lo(xi), f2_fma(lo(q), lo(xr), are[r][0]));
+                    are[r][1] = f2_fma(hi(nq), hi(xi), f2_fma(lo(q), hi(xr), are[r][1]));
+                    aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
+                    aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
+                }
             }
-        }
+        };
+        if (wild) products(std::true_type{});
+        else products(std::false_type{});
     }
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
