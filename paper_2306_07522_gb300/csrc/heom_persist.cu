@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
     cx<R> *s_pinv = reinterpret_cast<cx<R> *>(s_half + kPersThreads / 2);
     ProgSmem<R> ps = prog_layout<R>(v.pers_terms, v.pers_slots, v.pers_ados, d2,
                                     reinterpret_cast<unsigned char *>(s_pinv + (size_t)v.pers_ados * d2));
-    build_programs<R>(v, ps, n0, n1, a.aug, a.set);
+    build_programs<R, true>(v, ps, n0, n1, a.aug, a.set);
     const cx<R> shift = a.shift ? a.shift[a.col] : cx<R>{R(0), R(0)};
     const int items = (n1 - n0) * d2;
     const int64_t row0 = (int64_t)n0 * d2;
