@@ -395,7 +395,7 @@ bool persist_ok(const heom_hier *h);
 template <class R>
 int64_t persist_max_cols(const heom_hier *h);  // up to this many columns run one after another
 template <class R>
-heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col, bool x_zero,
+heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col,
                                 const cx<R> *shift, R aug, double tol, int max_iter,
                                 int stall_iters, int *iters, int *status, double *rel_res,
                                 cudaStream_t s);

@@ -30,7 +30,6 @@ struct PersistArgs {
     cx<R> *x;
     int64_t B, col;
     int set;         // the column's parameter set
-    int x_zero;
     const cx<R> *shift;  // [1] or null
     R aug;
     int precond;
@@ -233,21 +232,16 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
                 *const ph = sizeof(R) == 8 ? own(6, a.ph) : a.ph + row0,
                 *const sh = sizeof(R) == 8 ? own(7, a.sh) : a.sh + row0;
 
-    // ---- r = b - A x, rh = r, p = v = 0
-    double val2[2] = {0.0, 0.0};
+    // ---- x = 0, r = b, rh = r, p = v = 0
+    double val1[1] = {0.0};
     for (int it = threadIdx.x; it < items; it += blockDim.x) {
-        const int64_t i = row0 + it;
-        cx<R> ax{R(0), R(0)};
-        if (!a.x_zero) ax = prog_apply(ps, it, a.x, shift);
-        x[it] = a.x_zero ? cx<R>{R(0), R(0)} : a.x[i];
-        const cx<R> bi = a.b[i * a.B + a.col];
-        const cx<R> ri = bi - ax;
+        const cx<R> ri = a.b[(row0 + it) * a.B + a.col];
+        x[it] = cx<R>{R(0), R(0)};
         r[it] = ri;
         rh[it] = ri;
         p[it] = cx<R>{R(0), R(0)};
         vv[it] = cx<R>{R(0), R(0)};
-        val2[0] += (double)norm2(ri);
-        val2[1] += (double)norm2(bi);
+        val1[0] += (double)norm2(ri);
     }
     if constexpr (sizeof(R) == 8) {
         // float-float programs for the iteration: fold the shift into every item's first
@@ -263,12 +257,12 @@ __global__ void __launch_bounds__(kPersThreads) k_persist_bicg(PersistArgs<R> a)
         for (int t = threadIdx.x; t < ps.item[items]; t += blockDim.x) cf[t] = ff_split(ps.coef[t]);
         __syncthreads();
     }
-    const bool started = grid_sum<2>(val2, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles);
+    const bool started = grid_sum<1>(val1, s_red, s_tot, a.bar, gen, nw_act, a.wait_cycles);
     // Thread 0 holds the scalars and takes the decisions, the same ones in every CTA (redundant FP64 operations of
     // 16 warps queue on the FP64 pipe); s_st < 0: go on
     __shared__ int s_st;
-    double nr = val2[0];
-    const double bn = val2[1], stop2 = a.tol * a.tol * bn;
+    double nr = val1[0];
+    const double bn = nr, stop2 = a.tol * a.tol * bn;
     cx<double> rho{nr, 0.0}, rho_old{1.0, 0.0}, alpha{1.0, 0.0}, omega{1.0, 0.0};
     double best = nr, rhn = nr;  // rhn = ||rh||^2
     int best_it = 0, it_done = 0;
@@ -440,10 +434,9 @@ int64_t persist_max_cols(const heom_hier *h) {
 template int64_t persist_max_cols<double>(const heom_hier *);
 template int64_t persist_max_cols<float>(const heom_hier *);
 
-// One persistent BiCGStab solve of (M + shift + aug e00 tr) x = b for column col of b and x ([rows][B]; a starting
-// vector other than zero only with B = 1).
+// One persistent BiCGStab solve of (M + shift + aug e00 tr) x = b from x = 0 for column col of b and x ([rows][B]).
 template <class R>
-heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col, bool x_zero,
+heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col,
                                 const cx<R> *shift, R aug, double tol, int max_iter,
                                 int stall_iters, int *iters, int *status, double *rel_res,
                                 cudaStream_t s) {
@@ -463,7 +456,6 @@ heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t 
     a.B = B;
     a.col = col;
     a.set = (int)(col / (B / h->n_sets));
-    a.x_zero = x_zero || B > 1 ? 1 : 0;
     a.shift = shift;
     a.aug = aug;
     a.precond = 1;
@@ -509,10 +501,10 @@ heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t 
     return HEOM_OK;
 }
 
-template heom_status bicgstab_persistent<double>(heom_hier *, const cx<double> *, cx<double> *, int64_t, int64_t, bool,
+template heom_status bicgstab_persistent<double>(heom_hier *, const cx<double> *, cx<double> *, int64_t, int64_t,
                                                  const cx<double> *, double, double, int, int, int *,
                                                  int *, double *, cudaStream_t);
-template heom_status bicgstab_persistent<float>(heom_hier *, const cx<float> *, cx<float> *, int64_t, int64_t, bool,
+template heom_status bicgstab_persistent<float>(heom_hier *, const cx<float> *, cx<float> *, int64_t, int64_t,
                                                 const cx<float> *, float, double, int, int, int *,
                                                 int *, double *, cudaStream_t);
 

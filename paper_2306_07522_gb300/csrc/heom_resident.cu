@@ -59,7 +59,7 @@ struct ResArgs {
     const cx<R> *s_val;     // [nS][n_sets], or with a drive [sample][nS][n_sets]
     int64_t B, cps, step0, steps, save, s_stride;  // s_stride: elements from one sample to the next (0: no drive)
     R dt;
-    int n_sets, nS, nc, d2, P, C, rows;            // P: positions, rows: program rows in shared memory
+    int n_sets, nS, nc, d2, P, C;                  // P: positions
 };
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -510,7 +510,6 @@ heom_status resident_steps(heom_hier *h, cx<R> *y, int64_t B, double dt, int64_t
     a.d2 = h->d2;
     a.P = p.chunks * 32;
     a.C = g.C;
-    a.rows = g.rows;
     const ResKernel<R> k = kernel_of<R>(g.M);
     HEOM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResSmem));
     for (int64_t n = 0; n < steps; n += kResSteps) {

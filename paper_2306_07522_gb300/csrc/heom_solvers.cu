@@ -1201,7 +1201,7 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
             o.res.assign(B, 0.0);
             for (int64_t b = 0; b < B && stt == HEOM_OK; ++b)
                 if (active[b])
-                    stt = bicgstab_persistent<RI>(h, rhs, dv, B, b, true, shift64 ? shift_in : nullptr, (RI)aug,
+                    stt = bicgstab_persistent<RI>(h, rhs, dv, B, b, shift64 ? shift_in : nullptr, (RI)aug,
                                                   inner_tol, std::min(inner_max, std::max(1, max_iter - res.iters[b])),
                                                   kStallIters, &o.iters[b], &o.status[b], &o.res[b], s);
         } else {
