@@ -1,7 +1,10 @@
 // The hot path: y = M x over all ADOs and batch columns (Eq. HEOM), matrix-free.
 //
-// Two kernels: the tiled one (heom_tile.cuh) for many columns of one parameter set, and the
-// row kernel below (heom_rows.cuh) for everything else.
+// By size, batch and operators (launch_apply): block products of dense FP32 operators (heom_dense.cu), the
+// tiled kernel for many columns of one parameter set (heom_tile.cuh), a block per lane for one FP64 column of many
+// ADOs and one element per thread for small launches (heom_block.cuh), neighbour blocks staged through shared memory
+// for a few columns (heom_staged.cuh), and the flat kernel below over rows, quads of elements or whole blocks
+// (heom_rows.cuh, heom_block.cuh) for everything else.
 #include <algorithm>
 #include <cstdint>
 

@@ -514,8 +514,8 @@ heom_status arnoldi_persistent(heom_hier *h, int64_t B, int mmax, int max_steps,
     HEOM_CUDA(grid_bar_reset(a.bar, G, (int)B, s));
     // on top, where they fit: the own rows of w (the dots read them for every basis vector) and as many of the
     // split rotations as there is room for (a shift's chain walks all of them in every step: from L2 24,000 of
-    // the 123,000 cycles of a step at 55 basis vectors, on one warp while the others wait; 1,024 frequencies of 2,325
-    // ADOs: 8.28 -> 8.17 ms)
+    // the 123,000 cycles of a step at 55 basis vectors, on one warp while the others wait. 1,024 frequencies of 2,325
+    // ADOs gained 0.1 of 8.3 ms: the chain itself stays on that warp)
     size_t sm = (arnoldi_smem(a.v, a.hcap) + 15) & ~size_t(15);
     const size_t wb = (size_t)a.v.pers_ados * a.v.d2 * B * sizeof(float4);
     a.w_off = -1;

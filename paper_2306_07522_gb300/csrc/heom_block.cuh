@@ -361,7 +361,8 @@ __device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *_
 // us, 2,325 x 16 29.5 against 25.4; fewer columns: 2,325 x 8 23.2 against 27.9, 12,951 x 3 48 against 32);
 // larger blocks have them only where 32-column blocks stand half empty (charge-cavity model, 790 ADOs of
 // 24 x 24: 16 columns 327 against 345 us, 17 columns 627 against 382). FP64: the smallest launches (25 ADOs x 5
-// columns 33.9 against 37.8 us).
+// columns 33.9 against 37.8 us). The lines lie between the sizes measured (elements x columns: 6,800, 297,600,
+// 595,200 and 621,648 at d = 4), not at a measured crossing.
 template <class R>
 inline bool point_ok(const DevView<R> &v, int64_t B) {
     const double el = (double)v.N * v.d2 * (double)B;

@@ -9,13 +9,13 @@
 // inner loop is 4 RT complex multiply-adds on packed FP32 pairs for RT + 2 (left) or 2 RT + 1 (right)
 // 16-byte shared-memory loads, most of them broadcasts. Real and imaginary parts lie in separate planes: a
 // pair holds two columns, and one accumulator pair takes the real, one the imaginary part. Zero entries of the
-// operators are multiplied like the others unless a block sum is infinite or NaN: those spread over couplings only.
+// operators are multiplied like the others; a thread whose results are not all finite forms them again without
+// (infinities and NaN spread over couplings only).
 //
 // 222 ADOs of 24 x 24: 64 columns 2,595 us (term by term) -> 354 us, bound by FP32 issue (12.6 GFLOP of block
 // products); one column 133 -> 50 us, bound by a CTA's chain of products. 16 x 16: 748 -> 118 us at 64
 // columns, 99 -> 25 us at one.
 #include <cstdint>
-#include <type_traits>
 
 #include "heom_ff.cuh"
 #include "heom_kernels.cuh"
@@ -66,9 +66,44 @@ constexpr size_t dense_smem() {
     return (size_t)D * D * (4 * BT * sizeof(float) + sizeof(float4)) + kDenseMaxEntries * sizeof(DenseEntry);
 }
 
+// The results of a thread again without the zero entries of the operators, for a thread whose results are not all
+// finite: a zero entry couples nothing, whatever the block sums hold. The same operations in the same order
+// otherwise, so the results that are finite do not change; one by one, and out of line, so that the products above
+// keep their registers.
+template <int D>
+__device__ __noinline__ void masked_results(const DevView<float> &v, const DenseEntry *ent, int cnt,
+                                            const cx<float> *__restrict__ X, cx<float> *__restrict__ Y, int64_t n, int r0,
+                                            int c, int64_t b0, int cols, int64_t B) {
+    constexpr int D2 = D * D;
+    const cx<float> dmp = ldc(v.damp + n);
+    for (int r = r0; r < r0 + D / 4; ++r)
+        for (int64_t b = b0; b < b0 + min(cols, 4); ++b) {
+            cx<float> y{0.f, 0.f};
+            fma_to(y, cx<float>{-dmp.re, -dmp.im}, ldc(X + (n * D2 + r * D + c) * B + b));
+            for (int o = 0; o <= v.n_ops; ++o)
+                for (int right = 0; right < 2; ++right)
+                    for (int l = 0; l < D; ++l) {
+                        const cx<float> q = ldc(v.dense + (int64_t)o * D2 + (right ? l * D + c : r * D + l));
+                        if (q.re == 0.f && q.im == 0.f) continue;
+                        const int64_t at = right ? r * D + l : l * D + c;
+                        cx<float> sum{0.f, 0.f};
+                        if (o == v.n_ops) {
+                            fma_to(sum, cx<float>{0.f, right ? 1.f : -1.f}, ldc(X + (n * D2 + at) * B + b));
+                        } else {
+                            for (int t = 0; t < cnt; ++t)
+                                if (ent[t].op == o)
+                                    fma_to(sum, right ? ent[t].b : ent[t].a, ldc(X + (ent[t].nb * (int64_t)D2 + at) * B + b));
+                        }
+                        fma_to(y, q, sum);
+                    }
+            Y[(n * D2 + r * D + c) * B + b] = y;
+        }
+}
+
 template <int D, int BT>
-__global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, const cx<float> *__restrict__ X,
-                                                          cx<float> *__restrict__ Y, int64_t B, bool vec) {
+__global__ void __launch_bounds__(D *BT, 2) k_apply_dense(const __grid_constant__ DevView<float> v,
+                                                          const cx<float> *__restrict__ X, cx<float> *__restrict__ Y,
+                                                          int64_t B, bool vec) {
     constexpr int D2 = D * D, RT = D / 4, Q = BT / 4, T = D * BT;
     extern __shared__ __align__(16) unsigned char dense_sm[];
     float4 *rec = reinterpret_cast<float4 *>(dense_sm);  // operator (re, re, im, im)
@@ -107,7 +142,6 @@ __global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, cons
         bool any = o == v.n_ops;
         for (int t = 0; t < cnt && !any; ++t) any = ent[t].op == o;
         if (!any) continue;
-        bool fine = true;  // this thread's sums are finite
         for (int e = tid; e < D2; e += T) {
             const cx<float> w = ldc(v.dense + (int64_t)o * D2 + e);
             rec[e] = make_float4(w.re, w.re, w.im, w.im);
@@ -146,48 +180,38 @@ __global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, cons
                 const int w = (tid + (i + u) * T) * 4;
                 st_planes(Lr + w, Li + w, lr[u], li[u]);
                 st_planes(Rr + w, Ri + w, rr[u], ri[u]);
-                const float2 tot = f2_add(f2_add(f2_add(lr[u][0], lr[u][1]), f2_add(li[u][0], li[u][1])),
-                                          f2_add(f2_add(rr[u][0], rr[u][1]), f2_add(ri[u][0], ri[u][1])));
-                fine = fine && isfinite(tot.x) && isfinite(tot.y);
             }
         }
-        const bool wild = __syncthreads_or(!fine);
-        // a zero entry of the operator couples nothing, whatever S and T hold
-        const auto products = [&](auto masked) {
-            constexpr bool MASK = decltype(masked)::value;
+        __syncthreads();
 #pragma unroll 2
-            for (int l = 0; l < D; ++l) {  // O S
-                const int w = (l * D + c) * BT + 4 * bq;
-                const float4 xr = *reinterpret_cast<const float4 *>(Lr + w), xi = *reinterpret_cast<const float4 *>(Li + w),
-                             nx = neg(xi);
+        for (int l = 0; l < D; ++l) {  // O S
+            const int w = (l * D + c) * BT + 4 * bq;
+            const float4 xr = *reinterpret_cast<const float4 *>(Lr + w), xi = *reinterpret_cast<const float4 *>(Li + w),
+                         nx = neg(xi);
 #pragma unroll
-                for (int r = 0; r < RT; ++r) {
-                    const float4 q = rec[(r0 + r) * D + l];
-                    if (MASK && q.x == 0.f && q.z == 0.f) continue;
-                    are[r][0] = f2_fma(hi(q), lo(nx), f2_fma(lo(q), lo(xr), are[r][0]));
-                    are[r][1] = f2_fma(hi(q), hi(nx), f2_fma(lo(q), hi(xr), are[r][1]));
-                    aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
-                    aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
-                }
+            for (int r = 0; r < RT; ++r) {
+                const float4 q = rec[(r0 + r) * D + l];
+                are[r][0] = f2_fma(hi(q), lo(nx), f2_fma(lo(q), lo(xr), are[r][0]));
+                are[r][1] = f2_fma(hi(q), hi(nx), f2_fma(lo(q), hi(xr), are[r][1]));
+                aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
+                aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
             }
+        }
 #pragma unroll 2
-            for (int l = 0; l < D; ++l) {  // T O
-                const float4 q = rec[l * D + c], nq = neg(q);
-                if (MASK && q.x == 0.f && q.z == 0.f) continue;
+        for (int l = 0; l < D; ++l) {  // T O
+            const float4 q = rec[l * D + c], nq = neg(q);
 #pragma unroll
-                for (int r = 0; r < RT; ++r) {
-                    const int w = ((r0 + r) * D + l) * BT + 4 * bq;
-                    const float4 xr = *reinterpret_cast<const float4 *>(Rr + w), xi = *reinterpret_cast<const float4 *>(Ri + w);
-                    are[r][0] = f2_fma(hi(nq), lo(xi), f2_fma(lo(q), lo(xr), are[r][0]));
-                    are[r][1] = f2_fma(hi(nq), hi(xi), f2_fma(lo(q), hi(xr), are[r][1]));
-                    aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
-                    aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
-                }
+            for (int r = 0; r < RT; ++r) {
+                const int w = ((r0 + r) * D + l) * BT + 4 * bq;
+                const float4 xr = *reinterpret_cast<const float4 *>(Rr + w), xi = *reinterpret_cast<const float4 *>(Ri + w);
+                are[r][0] = f2_fma(hi(nq), lo(xi), f2_fma(lo(q), lo(xr), are[r][0]));
+                are[r][1] = f2_fma(hi(nq), hi(xi), f2_fma(lo(q), hi(xr), are[r][1]));
+                aim[r][0] = f2_fma(hi(q), lo(xr), f2_fma(lo(q), lo(xi), aim[r][0]));
+                aim[r][1] = f2_fma(hi(q), hi(xr), f2_fma(lo(q), hi(xi), aim[r][1]));
             }
-        };
-        if (wild) products(std::true_type{});
-        else products(std::false_type{});
+        }
     }
+    float2 tot = make_float2(0.f, 0.f);
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
         cx<float> *p = Y + (n * D2 + (r0 + r) * D + c) * B + b0 + 4 * bq;
@@ -201,7 +225,9 @@ __global__ void __launch_bounds__(D *BT, 2) k_apply_dense(DevView<float> v, cons
             for (int u = 0; u < 4; ++u)
                 if (u < cols) p[u] = cx<float>{re[u], im[u]};
         }
+        tot = f2_add(tot, f2_add(f2_add(are[r][0], are[r][1]), f2_add(aim[r][0], aim[r][1])));
     }
+    if (!(isfinite(tot.x) && isfinite(tot.y)) && cols > 0) masked_results<D>(v, ent, cnt, X, Y, n, r0, c, b0 + 4 * bq, cols, B);
 }
 
 template <int D, int BT>
