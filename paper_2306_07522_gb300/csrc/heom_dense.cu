@@ -1,4 +1,4 @@
-// FP32 apply of operators without zeros (d = 8, 16, 24, 32): block products from shared memory.
+// FP32 apply of operators with few zeros (d = 8, 16, 24, 32): block products from shared memory.
 //
 // Term by term (heom_tile.cuh) a dense operator costs 2 d complex multiply-adds per neighbour and
 // element, each with its own load from L1 or L2. Here a CTA owns one ADO and BT columns and works operator
@@ -12,8 +12,8 @@
 // operators are multiplied like the others; a thread whose results are not all finite forms them again without
 // (infinities and NaN spread over couplings only).
 //
-// 222 ADOs of 24 x 24: 64 columns 2,595 us (term by term) -> 354 us, bound by FP32 issue (12.6 GFLOP of block
-// products); one column 133 -> 50 us, bound by a CTA's chain of products. 16 x 16: 748 -> 118 us at 64
+// 222 ADOs of 24 x 24: 64 columns 2,595 us (term by term) -> 352 us, bound by shared-memory wavefronts (61 %) with two
+// CTAs per SM (12.6 GFLOP of block products, FMA pipe half busy); one column 133 -> 50 us, bound by a CTA's chain of products. 16 x 16: 748 -> 118 us at 64
 // columns, 99 -> 25 us at one.
 #include <cstdint>
 

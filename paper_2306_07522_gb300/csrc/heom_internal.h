@@ -84,7 +84,7 @@ struct DevView {
     // fixed-width operator records [op][side][i][w], w < op_width, side 0 the nonzeros of row i
     // and 1 those of column i, idx = -1 where there is none (null for op_width > 2)
     const OpRec<R> *op_ell;
-    // operators and H without zeros as [n_ops + 1][d2], H last (FP32 view; null unless one parameter
+    // operators and H as dense blocks [n_ops + 1][d2], H last (FP32 view; null unless one parameter
     // set, no Lindblad terms and a block size the dense kernel takes: heom_dense.cu)
     const cx<R> *dense;
     int dense_min;            // CTAs from which a launch takes the dense kernel
@@ -371,7 +371,7 @@ struct Prof {
 cudaError_t memcpy_counted(void *dst, const void *src, size_t bytes, cudaMemcpyKind kind,
                            cudaStream_t s);
 
-// FP32 apply of operators without zeros (heom_dense.cu)
+// FP32 apply of operators with few zeros (heom_dense.cu)
 bool dense_ok(const DevView<float> &v, int64_t B);
 cudaError_t launch_apply_dense(const DevView<float> &v, const cx<float> *x, cx<float> *y, int64_t B, cudaStream_t s);
 
