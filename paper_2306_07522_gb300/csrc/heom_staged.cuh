@@ -172,10 +172,15 @@ struct StageGeom {
 };
 constexpr size_t kStageOps = 24 * 1024;   // largest operator table
 constexpr int64_t kStageMaxB = 15;        // wider batches read whole sectors column by column
+// FP64: elements from which staging pays. Below them its groups leave most of the chip idle and one element per thread
+// (RowsLayout) is faster, us: 13 ADOs of 24 x 24 39 against 18, 130 of 8 x 8 53 against 28, 301 of 4 x 4 with 24
+// exponents 44 against 32, 2,325 46 against 30; 316 of 16 x 16, two columns (161,792 elements) 65 against 66.
+constexpr double kStageMin64 = 160e3;
 template <class R>
 inline StageGeom stage_geom(const DevView<R> &v, int64_t B) {
     StageGeom g;
     if (v.d < 2 || v.d % 2 || v.op_width < 1 || v.op_width > 2 || B > kStageMaxB) return g;
+    if (sizeof(R) == 8 && (double)v.N * v.d2 * (double)B < kStageMin64) return g;
     const size_t ops = (size_t)v.n_ops * 2 * v.d * v.op_width * sizeof(OpRec<R>);
     if (ops > kStageOps) return g;
     const int cw = v.d % 4 == 0 ? 4 : 2, T = v.d2 / cw;
