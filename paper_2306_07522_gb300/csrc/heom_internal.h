@@ -393,7 +393,7 @@ heom_status shifted_gmres(heom_hier *h, const cx<double> *bvec, int64_t B,
 template <class R>
 bool persist_ok(const heom_hier *h);
 template <class R>
-int64_t persist_max_cols(const heom_hier *h);  // up to this many columns run one after another
+int64_t persist_max_cols(const heom_hier *h, bool shifted);  // up to this many columns run one after another
 template <class R>
 heom_status bicgstab_persistent(heom_hier *h, const cx<R> *b, cx<R> *x, int64_t B, int64_t col,
                                 const cx<R> *shift, R aug, double tol, int max_iter,

@@ -1085,7 +1085,7 @@ heom_status refine_solve(heom_hier *h, const cx<double> *b64, cx<double> *x64, i
     const LayoutPick lp = pick_layout(v64, B);
     const Geom ga = make_geom(rows / lp.ne, B, std::max<int64_t>(1, 2048 / ((B + 31) / 32)));
     // few columns: the whole BiCGStab solve of a column is one cooperative launch
-    const bool one_by_one = B <= persist_max_cols<RI>(h) && !strict && persist_ok<RI>(h);
+    const bool one_by_one = B <= persist_max_cols<RI>(h, shift64 != nullptr) && !strict && persist_ok<RI>(h);
     stt = ensure_ws(h->ws_small, align_up(2 * B * sizeof(ColState)) + 3 * align_up(B * sizeof(int)) +
                                      align_up(reg_cap * sizeof(ColRegion)) +
                                      (one_by_one ? (size_t)ga.grid.x * 2 * B * sizeof(double) : 0));

@@ -60,3 +60,24 @@ def test_columns_of_long_neighbour_lists(tier, cols, prec, one_by_one):
     applies = pr["krylov_apply_fp64" if prec == "FP64" else "krylov_apply_fp32"]["launches"]
     assert (applies <= cols * pr["residual_fp64"]["launches"]) == one_by_one
     assert float((torch.diagonal(x[0]).sum(-1) - 1).abs().max()) < 1e-9
+
+
+@pytest.mark.parametrize("n_omega,one_by_one", [(3, True), (4, False)])
+def test_few_frequencies_in_mixed_precision(n_omega, one_by_one):
+    """Shifted systems, two columns a frequency: six run one by one, eight together (2,325 ADOs: eight take 8.2 ms one by
+    one and 6.3 together)."""
+    import numpy as np
+    import torch
+    import paper_2306_07522_gb300 as heom
+    m = W.siam_model(tier=2)
+    even, odd = (heom.build_hierarchy(heom.problem_from_model(m, p)) for p in (1, -1))
+    x = torch.zeros((even.n_ado, 4, 4), dtype=torch.complex128, device="cuda")
+    heom.steady(even, x, tol=1e-10, prec=heom.FP64)
+    om = np.linspace(-12.0, 9.0, n_omega)
+    out = []
+    pr = _accounted(heom, lambda: out.append(heom.spectrum(odd, x, m.fermion_baths[0][0], om, tol=1e-8, max_iter=1500,
+                                                           prec=heom.MIXED)[0]))
+    applies = pr["krylov_apply_fp32"]["launches"]
+    assert (applies <= 2 * n_omega * pr["residual_fp64"]["launches"]) == one_by_one
+    ref = heom.spectrum(odd, x, m.fermion_baths[0][0], om, tol=1e-10, max_iter=500, prec=heom.SHIFTED)[0]
+    assert float(np.abs(out[-1] - ref).max() / np.abs(ref).max()) < 1e-6
