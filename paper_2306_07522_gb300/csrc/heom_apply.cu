@@ -168,11 +168,12 @@ cudaError_t launch_apply(const DevView<R> &v, const cx<R> *x, cx<R> *y, int64_t 
         return cudaGetLastError();
     }
     const StageGeom sg = stage_geom(v, B);
-    if (point_ok(v, B)) {
-        const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
-        k_apply_point<R><<<g.grid, g.block, 0, s>>>(v, x, y, B, cps, mods);
-        return cudaGetLastError();
-    }
+    if constexpr (sizeof(R) == 4)
+        if (point_ok(v, B)) {
+            const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
+            k_apply_point<R><<<g.grid, g.block, 0, s>>>(v, x, y, B, cps, mods);
+            return cudaGetLastError();
+        }
     if (sg.cw && !quad) {
         const bool vec = row_vec<R>(B, x, y);
 #define CALL(CW, BLOCK, W) \

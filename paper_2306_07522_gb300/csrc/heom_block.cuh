@@ -356,31 +356,17 @@ __device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *_
 }
 
 // ---------------------------------------------------------------- choice
-// Columns a block of make_geom's shape holds for each that exists.
-inline double column_padding(int64_t B) {
-    int64_t bx = 1;
-    while (bx < B && bx < 32) bx <<= 1;
-    return (double)((B + bx - 1) / bx * bx) / (double)B;
-}
-// Whether a launch runs one element per thread in (32 columns x 8 elements) blocks.
-// FP32, operators with at most two non-zeros per row, several columns: the wider layouts need enough threads to pay off
+// Whether an FP32 launch runs one element per thread in (32 columns x 8 elements) blocks. Operators with at most
+// two non-zeros per row, several columns: the wider layouts need enough threads to pay off
 // (d = 4, 16 and more columns: 25 ADOs x 17 columns 17.3 against 24.4
 // us, 2,325 x 16 29.5 against 25.4; fewer columns: 2,325 x 8 23.2 against 27.9, 12,951 x 3 48 against 32);
 // larger blocks have them only where 32-column blocks stand half empty (charge-cavity model, 790 ADOs of
 // 24 x 24: 16 columns 327 against 345 us, 17 columns 627 against 382). One column of larger blocks: the smallest
 // launches (13 ADOs of 6 x 6 13 against 16 us, 4 of 24 x 24 10 against 12). The lines lie between the sizes measured
 // (elements x columns: 6,800, 297,600, 595,200 and 621,648 at d = 4), not at a measured crossing.
-// Operators with more non-zeros: the rows' shared decoding no longer pays, RK4 of 222 ADOs of 16 x 16 (24 x 24), three
-// steps, FP32, 20 columns 4.0 against 5.3 ms (13.0 against 16.2); below eight columns lanes of one element side by
-// side (flat_geom) share more lines: 27 ADOs of 24 x 24, two columns 0.52 against 0.92 ms. FP64 wherever the columns
-// fill the blocks: 27 ADOs of 24 x 24, two columns 3.4 against 4.4 ms, but five (padded to eight) 7.8 against 5.7;
-// of 16 x 16 twelve (padded to sixteen) 4.8 against 4.1.
-template <class R>
-inline bool point_ok(const DevView<R> &v, int64_t B) {
+inline bool point_ok(const DevView<float> &v, int64_t B) {
     const double el = (double)v.N * v.d2 * (double)B;
-    if (el >= 2147483647.0) return false;
-    if (sizeof(R) == 8) return v.op_width > 2 && column_padding(B) < (el < 150e3 ? 1.05 : 1.45);
-    if (v.d > 4 && v.op_width > 2) return B >= 8;
+    if (el >= 2147483647.0 || (v.d > 4 && v.op_width > 2)) return false;
     if (B == 1) return v.d > 4 && el < 2500;
     if (v.d <= 4) return el < (B >= 16 ? 430e3 : 590e3);
     return B <= 16 || el < 800e3 || (double)((B + 31) / 32 * 32) < 1.5 * (double)B;
@@ -503,7 +489,7 @@ struct PointLayout {  // one element
 // many-column one.
 struct LayoutPick {
     int cw = 1, d = 0, rows = 0, w = 0, ne = 1;
-    bool quad = false;
+    bool quad = false, point = false;
     size_t smem = 0;
 };
 constexpr int64_t kColsMinB = 16;
@@ -532,9 +518,14 @@ inline LayoutPick pick_layout(const DevView<R> &v, int64_t B, bool quad = false,
         return p;
     }
     p.cw = p.ne = row_width(v.N, v.d, B);
-    // more than two non-zeros per row: runs of elements only in FP64 and where they leave threads enough (27 ADOs of
-    // 24 x 24, RK4, 17 columns 13.9 ms one by one against 15.6, 64 columns 45.8 against 40.2)
-    if (v.op_width > 2 && ((sizeof(R) == 4 && v.d > 4) || (double)v.N * v.d2 * (double)B < 250e3)) p.cw = p.ne = 1;
+    // More than two non-zeros per row: decoding shared by a run no longer pays, one element per thread with every
+    // coefficient multiplied as a whole does. RK4, three steps, in rows, in 32 x 8 blocks of elements, so: 222 ADOs of
+    // 16 x 16, 20 columns FP32 5.3, 4.0, 2.7 ms; 27 of 24 x 24 FP64, two columns 4.4, 3.4, 2.3 ms, 15 columns 16.2, 9.7, 8.7
+    // ms, 32 columns 25.9, 14.9, 14.8 ms. An iteration's FP64 apply of 27 ADOs of 8 x 8, five columns: 160 us in rows.
+    if (v.op_width > 2) {
+        p.cw = p.ne = 1;
+        p.point = true;
+    }
     return p;
 }
 // one element per thread: FP64 leaves out the zero halves of coefficients
@@ -551,6 +542,7 @@ using OneLayout = std::conditional_t<sizeof(R) == 8, RowsLayout<R, 1>, PointLayo
     do {                                                                                        \
         if ((p).cw == 4) { using Ly = RowsLayout<R, 4>; CALL(Ly); }                             \
         else if ((p).cw == 2) { using Ly = RowsLayout<R, 2>; CALL(Ly); }                        \
+        else if ((p).cw == 1 && (p).point) { using Ly = PointLayout<R>; CALL(Ly); }             \
         else if ((p).cw == 1) { using Ly = OneLayout<R>; CALL(Ly); }                            \
         else if ((p).d == 2) HEOM_COLS_W(R, 2, 2, (p).w, CALL);                                 \
         else if ((p).rows == 4) HEOM_COLS_W(R, 4, 4, (p).w, CALL);                              \

@@ -88,11 +88,12 @@ cudaError_t launch_rk4_stage(const DevView<R> &v, const cx<R> *z_in, cx<R> *z_ou
     const ColSets cps(B / v.n_sets);
     const bool quad = quad_ok(v, B, z_in, z_out, y, acc);
     const StageGeom sg = stage_geom(v, B);
-    if (point_ok(v, B)) {
-        const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
-        k_rk4_point<R><<<g.grid, g.block, 0, s>>>(v, z_in, z_out, y, acc, B, cps, dt, stage);
-        return cudaGetLastError();
-    }
+    if constexpr (sizeof(R) == 4)
+        if (point_ok(v, B)) {
+            const Geom g = make_geom(v.N * v.d2, B, 1 << 30);
+            k_rk4_point<R><<<g.grid, g.block, 0, s>>>(v, z_in, z_out, y, acc, B, cps, dt, stage);
+            return cudaGetLastError();
+        }
     if (sg.cw && !quad) {
         const bool vec = row_vec<R>(B, z_in, z_out, y, acc);
 #define CALL(CW, BLOCK, W) \
