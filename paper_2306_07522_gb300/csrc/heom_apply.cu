@@ -2,8 +2,9 @@
 //
 // By size, batch and operators (launch_apply): block products of dense FP32 operators (heom_dense.cu), the
 // tiled kernel for many columns of one parameter set (heom_tile.cuh), a block per lane for one FP64 column of many
-// ADOs and one element per thread for small launches (heom_block.cuh), neighbour blocks staged through shared memory
-// for a few columns (heom_staged.cuh), and the flat kernel below over rows, quads of elements or whole blocks
+// ADOs and one element per thread for small FP32 launches (heom_block.cuh), neighbour blocks staged through shared
+// memory for a few columns, in FP64 of large hierarchies only (heom_staged.cuh), and the flat kernel below over rows,
+// quads of elements, whole blocks or, where operators have more than two non-zeros per row, single elements
 // (heom_rows.cuh, heom_block.cuh) for everything else.
 #include <algorithm>
 #include <cstdint>

@@ -316,9 +316,10 @@ __device__ __forceinline__ void apply_cols(const DevView<R> &v, const OpRec<R> *
     for (int u = 0; u < RP * D; ++u) s[u] = acc.value(u);
 }
 
-// ---------------------------------------------------------------- small launches
-// y = (M X)[n][e][b] term by term, one element per thread. Most threads and least bookkeeping per thread: the
-// fastest layout while a launch does not fill the chip. Term order as in apply_rows.
+// ---------------------------------------------------------------- one element per thread
+// y = (M X)[n][e][b] term by term, one element per thread, every coefficient multiplied as a whole. Most threads and
+// least bookkeeping per thread: the fastest layout of FP32 launches that do not fill the chip, and in both precisions
+// of operators with more than two non-zeros per row. Term order as in apply_rows.
 template <class R>
 __device__ __forceinline__ cx<R> apply_point(const DevView<R> &v, const cx<R> *__restrict__ X, int64_t n, int e,
                                              int64_t b, int64_t B, int set, cx<R> &x0) {
@@ -386,7 +387,8 @@ inline bool quad_ok(const DevView<double> &, int64_t, const void *, const void *
 
 // Whether the one-column layout runs a launch: FP64, small blocks, 16-byte aligned buffers, an ADO order
 // (built from kWarpMinAdos ADOs on, one warp of 32 per SM sub-partition; below that, groups of
-// d^2 / 4 threads per ADO use more of the chip: heom_staged.cuh).
+// d^2 / 4 threads per ADO use more of the chip (heom_staged.cuh), and below kStageMin64 elements
+// one thread per element).
 template <class R>
 inline bool warp_ok(const DevView<R> &v, int64_t B, const void *a, const void *b, const void *c = nullptr,
                     const void *e = nullptr) {
@@ -485,8 +487,8 @@ struct PointLayout {  // one element
     }
 };
 
-// Layout of a launch: cw > 0 the row layout, quad the FP32 one-column layout, else rows/w of the
-// many-column one.
+// Layout of a launch: cw > 0 the row layout (point: one element per thread with whole coefficients), quad the FP32
+// one-column layout, else rows/w of the many-column one.
 struct LayoutPick {
     int cw = 1, d = 0, rows = 0, w = 0, ne = 1;
     bool quad = false, point = false;

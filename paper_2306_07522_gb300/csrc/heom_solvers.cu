@@ -655,8 +655,8 @@ struct SolveOut {
 // row kernel's longer chains and its sums over up to 256 threads a column cost more than its decoding saves. us per
 // launch against the row kernel: 400 elements x 8 to 64 columns 23 / 33, 4,816 x 5 26 / 35, x 64 28 / 34, 37,200 x 8
 // 32 / 37, x 9 50 / 39, 207,216 x 2 44 / 47, x 3 68 / 48; one column: 207,216 30 / 43, 469,072 58 / 81, 6.3 million
-// 526 / 330. (B: the columns of the whole solve, so that the rounding does not change as columns converge.) Operators with more than two non-zeros per row have nothing to
-// share: 222 ADOs of 8 x 8, 32 columns 81 / 93.
+// 526 / 330. (B: the columns of the whole solve, so that the rounding does not change as columns converge.) Operators
+// with more than two non-zeros per row have nothing to share: 222 ADOs of 8 x 8, 32 columns 81 / 93.
 template <class R>
 inline bool bicg_point(const DevView<R> &v, int64_t B) {
     return sizeof(R) == 4 && (v.op_width > 2 || (double)v.N * v.d2 * (double)B < (B == 1 ? 1e6 : 320e3));

@@ -10,7 +10,7 @@
 // shared memory when its turn comes and the operator's row and column lists, which sit there
 // too, index it at shared-memory latency. A group inside one warp needs no block barrier.
 // Operators: at most W (1 or 2) nonzeros per row and column (annihilators, number operators,
-// Pauli matrices, a + a^dag); others take the list kernel (heom_rows.cuh).
+// Pauli matrices, a + a^dag); others run one element per thread (PointLayout, heom_block.cuh).
 #pragma once
 
 #include "heom_rows.cuh"
