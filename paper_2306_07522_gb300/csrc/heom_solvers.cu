@@ -91,9 +91,13 @@ constexpr int kRegPieces = 32;  // pieces the regions are cut into, about
          q < q_end; q += (int64_t)gridDim.x * rstep)
 
 // Adds the block's sums of NV per-column values to dst (fixed-order tree over the threads of a
-// column); every thread of the block calls it.
-template <int NV>
-__device__ __forceinline__ void region_add(const ColRegion &rg, double (&val)[NV], double *const (&dst)[NV], bool on) {
+// column); every thread of the block calls it. again(val) forms a column's sums anew where they are not finite, by
+// the one thread that adds them: FP32 sums that have left their range (ColDots). Told by every thread from its own sums
+// it cost k_bicg_x 3 us a launch of 2,325 ADOs x 9 columns, by a vote of the block 1.5 us, so less than 1 us; in line, as
+// a call within the kernels takes registers.
+template <class R, int NV, class Again>
+__device__ __forceinline__ void region_add(const ColRegion &rg, const double (&val)[NV], double *const (&dst)[NV], bool on,
+                                           const Again &again) {
     __shared__ double sh[NV][kRegThreads];
     const int A = rg.acols, n = kRegThreads / A, k = threadIdx.x / A;
 #pragma unroll
@@ -109,6 +113,17 @@ __device__ __forceinline__ void region_add(const ColRegion &rg, double (&val)[NV
         __syncthreads();
     }
     if (k == 0 && on) {
+        if constexpr (sizeof(R) == 4) {
+            bool finite = true;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) finite = finite && isfinite(sh[i][threadIdx.x]);
+            if (!finite) {
+                double w[3];
+                again(w);
+#pragma unroll
+                for (int i = 0; i < NV; ++i) sh[i][threadIdx.x] = w[i];
+            }
+        }
 #pragma unroll
         for (int i = 0; i < NV; ++i)
             if (dst[i]) atomicAdd(dst[i], sh[i][threadIdx.x]);
@@ -260,36 +275,19 @@ __global__ void __launch_bounds__(256, Ly::MINB) k_bicg_apply(DevView<R> v, cons
             }
         }
     }
-    DotVals sum(dots);
-    if (dots.overflowed()) {  // again from what has been stored, in FP64
-        ColDots<double> wide;
-        REGION_RUNS(Ly) {
-            int64_t n;
-            int e0;
-            Ly::pos(v, q, small, n, e0);
-            if (beyond_cap(v, n, set)) continue;
-            for (int u = 0; u < NE; ++u) {
-                const int64_t i = (n * v.d2 + e0 + u) * B + b;
-                const cx<double> y = cast<double>(out[i]), wv = cast<double>(w[i]);
-                if (mode == 0) {
-                    wide.cross(wv, y);
-                } else {
-                    wide.cross(y, wv);
-                    wide.norm(y);
-                }
-            }
-        }
-        sum = DotVals(wide);
-    }
+    const auto again = [&](double (&val)[3]) {
+        wide_dots(val, out + b, w + b, B, (int64_t)rg.ado0 * Ly::per_ado(v) + (int64_t)blockIdx.x * rstep,
+                  (int64_t)rg.ado1 * Ly::per_ado(v), (int64_t)gridDim.x * rstep, rstep, NE, v.d2, Kept(v, set), mode != 0);
+    };
     if (mode == 0) {
-        double val[2] = {sum.re, sum.im};
+        const double val[2] = {dots.c_re(), dots.c_im()};
         double *const dst[2] = {act ? &st[b].acc_rv.re : nullptr, act ? &st[b].acc_rv.im : nullptr};
-        region_add<2>(rg, val, dst, act);
+        region_add<R, 2>(rg, val, dst, act, again);
     } else {
-        double val[3] = {sum.re, sum.im, sum.n};
+        const double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
         double *const dst[3] = {act ? &st[b].acc_ts.re : nullptr, act ? &st[b].acc_ts.im : nullptr,
                                 act ? &st[b].acc_tt.re : nullptr};
-        region_add<3>(rg, val, dst, act);
+        region_add<R, 3>(rg, val, dst, act, again);
         if (act && lead) {
             st[b].acc_rr = {0.0, 0.0};
             st[b].acc_nr = 0.0;
@@ -433,22 +431,13 @@ __global__ void __launch_bounds__(256) k_bicg_x(DevView<R> v, cx<R> *x, const cx
             dots.norm(ri);
         }
     }
-    DotVals sum(dots);
-    if (dots.overflowed()) {  // again from what has been stored, in FP64
-        ColDots<double> wide;
-        const Kept kept(v, set);
-        REGION_ROWS {
-            if (!kept(ado_of(row, v.d2, v.N * v.d2))) continue;
-            const cx<double> rd = cast<double>(r[row * B + b]);
-            wide.cross(cast<double>(rh[row * B + b]), rd);
-            wide.norm(rd);
-        }
-        sum = DotVals(wide);
-    }
-    double val[3] = {sum.re, sum.im, sum.n};
+    const double val[3] = {dots.c_re(), dots.c_im(), dots.n()};
     double *const dst[3] = {act ? &st[b].acc_rr.re : nullptr, act ? &st[b].acc_rr.im : nullptr,
                             act ? &st[b].acc_nr : nullptr};
-    region_add<3>(rg, val, dst, act);
+    region_add<R, 3>(rg, val, dst, act, [&](double (&again)[3]) {
+        wide_dots(again, r + b, rh + b, B, (int64_t)rg.ado0 * v.d2 + (int64_t)blockIdx.x * rstep, (int64_t)rg.ado1 * v.d2,
+                  (int64_t)gridDim.x * rstep, rstep, 1, v.d2, Kept(v, set), false);
+    });
     if (c.on && lead) {
         st[b].omega = c.keep;
         if (c.on == 2) st[b].flag = 1;
